@@ -229,6 +229,8 @@ void free_dictionary(act_grid *g) {
     free_dev(g->shift.tpl16);
     free_dev(g->shift.scaleT);
     free_dev(g->shift.eps_bits);
+    free_dev(g->shift.span);
+    free_dev(g->shift.blk_order);
     g->shift = ShiftPlan();
     g->built = -1;
     // the tensor-core search scratch is sized by the dictionary's shape
@@ -682,6 +684,14 @@ static act_status build_templates(act_grid *g, cudaStream_t st) {
     const size_t bs = sizeof(float) * (size_t)sp.TB * sp.NtcP * 32;
     cudaError_t e = dev_alloc((void **)&sp.tpl, bt);
     if (e == cudaSuccess) e = dev_alloc((void **)&sp.scale, bs);
+    std::vector<int> order;
+    if (e == cudaSuccess && sp.Kt > 0) {
+        try {
+            shift_block_order(sp, g->ax, order);
+        } catch (const std::bad_alloc &) {
+            e = cudaErrorMemoryAllocation;
+        }
+    }
     if (e == cudaSuccess && sp.Kt > 0) {
         // the tensor-core view: BF16 templates, transposed scales, BF16 error bound
         const size_t b16 = sizeof(__nv_bfloat16) * (size_t)sp.T_pad * sp.Kt;
@@ -689,6 +699,10 @@ static act_status build_templates(act_grid *g, cudaStream_t st) {
         e = dev_alloc((void **)&sp.tpl16, b16);
         if (e == cudaSuccess) e = dev_alloc((void **)&sp.scaleT, bst);
         if (e == cudaSuccess) e = dev_alloc((void **)&sp.eps_bits, sizeof(unsigned int));
+        if (e == cudaSuccess) e = dev_alloc((void **)&sp.span, sizeof(short2) * (size_t)(sp.T_pad / 128));
+        if (e == cudaSuccess) e = dev_alloc((void **)&sp.blk_order, sizeof(int) * order.size());
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(sp.blk_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.scaleT, 0, bst, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.eps_bits, 0, sizeof(unsigned int), st);
     }
@@ -699,6 +713,8 @@ static act_status build_templates(act_grid *g, cudaStream_t st) {
         free_dev(sp.tpl16);
         free_dev(sp.scaleT);
         free_dev(sp.eps_bits);
+        free_dev(sp.span);
+        free_dev(sp.blk_order);
         note_error("template dictionary", e);
         return ACT_ERR_OOM;
     }

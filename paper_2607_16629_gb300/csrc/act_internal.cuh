@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/act.h"
 #include "act_device.cuh"
 
@@ -221,12 +223,21 @@ struct ShiftPlan {
     float *tpl = nullptr;       // [TB][Sa][rows][32]
     float *scale = nullptr;     // [TB][NtcP][32]
     // tensor-core view (act_shift_tc.cu): templates over m = n - tc in
-    // [m_lo, m_lo + Kt) as BF16 rows, tile-major [T_pad / 256][Kt / 64][256][64]
+    // [m_lo, m_lo + Kt) as BF16 rows, tile-major [T_pad / 256][Kt / 64][256][64],
+    // the 32-template blocks ordered by duration (shift_block_order)
     int m_lo = 0, Kt = 0, T_pad = 0;
     __nv_bfloat16 *tpl16 = nullptr;
-    float *scaleT = nullptr;         // [NtcP][T_pad]
-    unsigned int *eps_bits = nullptr;  // largest |bf16(u) - u| / |u| over the atoms (float bits)
+    float *scaleT = nullptr;         // [NtcP][T_pad], in the view's template order
+    int *blk_order = nullptr;        // [2][T_pad / 32]: template block at each position, position of each block
+    short2 *span = nullptr;          // [T_pad / 128]: first and last 16-lag step multiplied, per 128-template group
+    unsigned int *eps_bits = nullptr;  // largest |u~ - u| / |u| over the atoms, u~ as multiplied (float bits)
 };
+// The order of the 32-template blocks in the BF16 view: longest duration
+// first, so that the 256 templates of one GEMM tile vanish at similar lags
+// and the tile multiplies only those it needs (a tile in grid order holds
+// every duration and would need the longest).  order = the block at each
+// position, then the position of each block (T_pad / 32 entries each).
+void shift_block_order(const ShiftPlan &sp, const GridAxes &ax, std::vector<int> &order);
 // Layout of the template dictionary; cudaErrorNotSupported unless the tc
 // axis is whole samples (lo and step integers, step >= 1).
 cudaError_t shift_plan(ShiftPlan &sp, const GridAxes &ax);

@@ -22,7 +22,7 @@
 //     (lane = template), row rho holds k = rho - (NtcP - 1); rows =
 //     NtcP + P - 1, NtcP = Ntc rounded up to 32, P = ceil(L / S) rounded up
 //     to 16.  Zero for padding templates.
-//   scales [TB][NtcP][32]: 1/|u| in FP32 from an FP64 sum over the window,
+//   scales [TB][NtcP][32]: 1/|u| in FP32 from a float-pair sum over the window,
 //     0 for a degenerate atom, a padding template or a padding lag.
 // The flat index of (lag j, template t) is j T + t, the order of the grid.
 //
@@ -40,7 +40,10 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
+#include <utility>
+#include <vector>
 
 #include "act_device.cuh"
 #include "act_ff.cuh"
@@ -110,18 +113,21 @@ __global__ void __launch_bounds__(256) k_shift_templates(GridAxes ax, int S, int
 }
 
 // BF16 templates for the tensor-core search, tile-major like the BF16
-// dictionary: element (t, kk) = bf16(u_t(m_lo + kk)) at
-// [t / 256][kk / 64][t % 256][kk % 64]; zero for padding templates.  A warp
+// dictionary: row q of the view is template t = 32 perm[q / 32] + q % 32
+// (shift_block_order), element (q, kk) = bf16(u_t(m_lo + kk)) at
+// [q / 256][kk / 64][q % 256][kk % 64]; zero for padding templates.  A warp
 // takes 32 templates: lane l forms template l's constants once, then the
 // warp writes the templates one after another, lane = kk stride 32.
 __global__ void __launch_bounds__(256) k_shift_tpl16(GridAxes ax, int m_lo, int Kt, int T, int T_pad,
+                                                     const int *__restrict__ perm,
                                                      __nv_bfloat16 *__restrict__ tpl16) {
     const double inv_fs = 1.0 / ax.fs;
     const int nkc = Kt >> 6;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t t0 = warp * 32; t0 < T_pad; t0 += nwarps * 32) {
+    for (int64_t q0 = warp * 32; q0 < T_pad; q0 += nwarps * 32) {
+        const int64_t t0 = (int64_t)perm[q0 >> 5] * 32;
         ChirpFF mine = {};
         if (t0 + lane < T) {
             double p[4];
@@ -133,7 +139,8 @@ __global__ void __launch_bounds__(256) k_shift_tpl16(GridAxes ax, int m_lo, int 
             const ChirpFF k = chirp_ff_shfl(mine, q);
             for (int kk = lane; kk < Kt; kk += 32) {
                 const float v = t < T ? template_sample(m_lo + kk, k) : 0.0f;
-                const int64_t off = (((t >> 8) * nkc + (kk >> 6)) * 256 + (t & 255)) * 64 + (kk & 63);
+                const int64_t row = q0 + q;
+                const int64_t off = (((row >> 8) * nkc + (kk >> 6)) * 256 + (row & 255)) * 64 + (kk & 63);
                 tpl16[off] = __float2bfloat16_rn(v);
             }
         }
@@ -141,14 +148,13 @@ __global__ void __launch_bounds__(256) k_shift_tpl16(GridAxes ax, int m_lo, int 
 }
 
 // One thread per (template block, lag, lane): |u|^2 over the window (a
-// float-float sum),
-// the scale 1/|u| in both layouts ([TB][NtcP][32] for the FP32 search,
-// [NtcP][T_pad] for the tensor-core epilogue) and the largest relative BF16
-// rounding error |bf16(u) - u| / |u| over all atoms (float bits, rounded up).
+// float-float sum) and the scale 1/|u| in both layouts ([TB][NtcP][32] for
+// the FP32 search, [NtcP][T_pad] in the BF16 view's template order for the
+// tensor-core epilogue; inv[tb] = where block tb sits in that order).
 __global__ void __launch_bounds__(256) k_shift_scales(int S, int Sa, int L, int NtcP, int Ntc, int rows, int T,
                                                       int T_pad, int64_t total, const float *__restrict__ tpl,
-                                                      float *__restrict__ scale, float *__restrict__ scaleT,
-                                                      unsigned int *__restrict__ eps_bits,
+                                                      const int *__restrict__ inv, float *__restrict__ scale,
+                                                      float *__restrict__ scaleT,
                                                       unsigned long long *__restrict__ degenerate) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -159,30 +165,163 @@ __global__ void __launch_bounds__(256) k_shift_scales(int S, int Sa, int L, int 
         const int64_t t = tb * 32 + lane;
         float sc = 0.0f;
         if (t < T && j < Ntc) {
-            ff ef = {0.0f, 0.0f}, def = {0.0f, 0.0f};
+            ff ef = {0.0f, 0.0f};
             const float *base = tpl + (size_t)tb * Sa * rows * 32 + lane;
             // sample n = a + S p sits in phase a, row p - j + NtcP - 1
             for (int a = 0; a < Sa; ++a) {
                 const float *col = base + ((size_t)a * rows + (NtcP - 1 - j)) * 32;
                 for (int p = 0; a + S * p < L; ++p) {
                     const float u = col[(size_t)p * 32];
-                    const float d = __bfloat162float(__float2bfloat16_rn(u)) - u;  // exact
                     ff_fma_acc(ef, u, u);
-                    ff_fma_acc(def, d, d);
                 }
             }
-            const double e = ff_to_double(ef), de = ff_to_double(def);
-            if (e > 0.0 && isfinite(e)) {
+            const double e = ff_to_double(ef);
+            if (e > 0.0 && isfinite(e))
                 sc = (float)(1.0 / sqrt(e));
-                if (eps_bits)
-                    atomicMax(eps_bits, __float_as_uint(__double2float_ru(sqrt(de / e) * (1.0 + 1e-6))));
-            } else if (degenerate) {
+            else if (degenerate)
                 atomicAdd(degenerate, 1ull);
-            }
         }
         scale[i] = sc;
-        if (scaleT && t < T_pad) scaleT[(size_t)j * T_pad + t] = sc;
+        if (scaleT) scaleT[(size_t)j * T_pad + (size_t)inv[tb] * 32 + lane] = sc;
     }
+}
+
+// Which lags of the BF16 view the tensor-core search multiplies.  A template
+// of duration Dt vanishes a few Dt from its centre, while the view spans
+// every lag any window can see: on the grids of short atoms most of the
+// matrix is negligible.  Per 128-template group of the view this finds the
+// lags [lo, hi) outside which every atom of the group (every template and
+// time centre) loses at most kSpanTau of its energy |u|^2 on either side, in
+// steps of 16 lags (one MMA).  What is dropped counts as rounding error of
+// the BF16 template: k_shift_eps measures it into the search's error bound,
+// so selections stay exact.  kSpanTau = 2^-23 (|dropped| <= 2^-11.5 |u| a
+// side) is small beside the rounding error itself (about 2^-9 |u|): the
+// bound grows by a few percent and the multiplied lags end near 3.7 Dt.
+//
+// One warp per 32-template block, lane = template.  Going up from lag 0, C =
+// energy below p; the window of time centre j starts at S (Ntc - 1 - j), and
+// lags below p may go while C(p) - C(start) <= tau |u_j|^2 for every window
+// that starts below p.  The upper end mirrors it.  Sums of FP32 squares grow
+// from the vanishing tail, so no cancellation; an error here only moves the
+// cut, the error bound is formed from the cut as made.
+constexpr float kSpanTau = 1.1920929e-07f;
+
+__global__ void __launch_bounds__(128) k_shift_spans(int S, int Sa, int L, int NtcP, int Ntc, int rows, int T,
+                                                     const float *__restrict__ tpl, const float *__restrict__ scale,
+                                                     const int *__restrict__ perm, short2 *__restrict__ span) {
+    __shared__ int lo_s[4], hi_s[4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t tb = perm[blockIdx.x * 4 + warp];
+    const bool valid = tb * 32 + lane < T;
+    const int used = S * (Ntc - 1) + L;  // lags any window sees
+    int lo = used, hi = 0;
+    if (tb * 32 < T) {
+        const float *sc = scale + (size_t)tb * NtcP * 32 + lane;
+        // lag kk sits in phase kk % S, row kk / S + NtcP - Ntc (phases from Sa on hold no sample of any window)
+        auto energy = [&](int kk) {
+            const int a = kk % S;
+            if (kk < 0 || kk >= used || a >= Sa) return 0.0f;
+            const float u = tpl[(((size_t)tb * Sa + a) * rows + kk / S + NtcP - Ntc) * 32 + lane];
+            return u * u;
+        };
+        auto room = [&](int i) {  // what the window starting at lag S i may lose
+            const float v = sc[(Ntc - 1 - i) * 32];
+            return v > 0.0f ? kSpanTau / (v * v) : __int_as_float(0x7f800000);
+        };
+        constexpr int U = 8;
+        bool live = valid;
+        float lim = __int_as_float(0x7f800000), c = 0.0f;
+        for (int k0 = 0; k0 < used && __any_sync(0xffffffffu, live); k0 += U) {
+            float e[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) e[i] = energy(k0 + i);
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int kk = k0 + i;
+                if (kk % S == 0 && kk / S < Ntc) lim = fminf(lim, c + room(kk / S));
+                c += e[i];
+                if (live && kk < used && !(c <= lim)) {
+                    live = false;
+                    lo = kk;
+                }
+            }
+        }
+        live = valid;
+        lim = __int_as_float(0x7f800000);
+        c = 0.0f;
+        for (int k0 = used - 1; k0 >= 0 && __any_sync(0xffffffffu, live); k0 -= U) {
+            float e[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) e[i] = energy(k0 - i);
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                const int kk = k0 - i, st = kk + 1 - L;  // a window that ends here starts at st
+                if (st >= 0 && st % S == 0 && st / S < Ntc) lim = fminf(lim, c + room(st / S));
+                c += e[i];
+                if (live && kk >= 0 && !(c <= lim)) {
+                    live = false;
+                    hi = kk + 1;
+                }
+            }
+        }
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+        lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+        hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+    }
+    if (lane == 0) {
+        lo_s[warp] = lo;
+        hi_s[warp] = hi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 4; ++w) {
+            lo = min(lo, lo_s[w]);
+            hi = max(hi, hi_s[w]);
+        }
+        // an empty group (padding, degenerate atoms) spans nothing
+        span[blockIdx.x] = hi > lo ? make_short2((short)(lo / 16), (short)((hi - 1) / 16)) : make_short2(32767, -1);
+    }
+}
+
+// The largest relative error |u~ - u| / |u| over all atoms of what the
+// tensor-core search multiplies: u~ = bf16(u) inside the group's span, 0
+// outside it (a launch that multiplies more lags than the span errs less:
+// rounding changes a sample by less than the sample).  FP32 sums of at most
+// 2048 squares are within 1.3e-4 of the exact ones and 1/|u| within 1e-7:
+// inflated by 1e-3 the result bounds them (float bits, rounded up).  Same
+// threads as k_shift_scales.
+__global__ void __launch_bounds__(256) k_shift_eps(int S, int Sa, int L, int NtcP, int Ntc, int rows, int T,
+                                                   int64_t total, const float *__restrict__ tpl,
+                                                   const float *__restrict__ scale, const int *__restrict__ inv,
+                                                   const short2 *__restrict__ span,
+                                                   unsigned int *__restrict__ eps_bits) {
+    float worst = 0.0f;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int lane = (int)(i & 31);
+        const int64_t rest = i >> 5;
+        const int j = (int)(rest % NtcP);
+        const int64_t tb = rest / NtcP;
+        const float sc = scale[i];
+        if (tb * 32 + lane >= T || j >= Ntc || sc == 0.0f) continue;
+        const short2 sp = span[inv[tb] >> 2];
+        // samples n = kk - S (Ntc - 1 - j) of the kept lags
+        const int n_lo = 16 * sp.x - S * (Ntc - 1 - j), n_hi = 16 * (sp.y + 1) - S * (Ntc - 1 - j);
+        float de = 0.0f;
+        const float *base = tpl + (size_t)tb * Sa * rows * 32 + lane;
+        for (int a = 0; a < Sa; ++a) {
+            const float *col = base + ((size_t)a * rows + (NtcP - 1 - j)) * 32;
+            for (int p = 0, n = a; n < L; ++p, n += S) {
+                const float u = col[(size_t)p * 32];
+                const float d = n >= n_lo && n < n_hi ? __bfloat162float(__float2bfloat16_rn(u)) - u : u;
+                de = fmaf(d, d, de);
+            }
+        }
+        worst = fmaxf(worst, __double2float_ru(sqrt((double)de) * (double)sc * (1.0 + 1e-3)));
+    }
+    for (int off = 16; off > 0; off >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, off));
+    if ((threadIdx.x & 31) == 0) atomicMax(eps_bits, __float_as_uint(worst));
 }
 
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
@@ -500,6 +639,25 @@ cudaError_t shift_plan(ShiftPlan &sp, const GridAxes &ax) {
     return cudaSuccess;
 }
 
+void shift_block_order(const ShiftPlan &sp, const GridAxes &ax, std::vector<int> &order) {
+    const int n = sp.T_pad / 32;
+    const int64_t Nl = ax.count[2], Nc = ax.count[3];
+    std::vector<std::pair<double, int>> key(n);  // (-longest logDt of the block, block)
+    for (int b = 0; b < n; ++b) {
+        double longest = -HUGE_VAL;  // padding blocks last
+        const int64_t t1 = std::min<int64_t>((int64_t)b * 32 + 32, sp.T);
+        for (int64_t t = (int64_t)b * 32; t < t1; t = (t / Nc + 1) * Nc)  // one step per logDt run
+            longest = std::max(longest, axis_value(ax.lo[2], ax.step[2], t / Nc % Nl));
+        key[b] = {-longest, b};
+    }
+    std::sort(key.begin(), key.end());
+    order.resize(2 * (size_t)n);
+    for (int q = 0; q < n; ++q) {
+        order[q] = key[q].second;
+        order[(size_t)n + key[q].second] = q;
+    }
+}
+
 cudaError_t shift_configure(ShiftPlan &sp, int J, int W, int NS, int sm_count, int ctas_per_sm) {
     if (!shift_config_valid(sp, J, W, NS)) return cudaErrorInvalidValue;
     const size_t smem = shift_smem(sp, J, W, NS);
@@ -540,13 +698,22 @@ cudaError_t launch_shift_build(const ShiftPlan &sp, const GridAxes &ax, unsigned
     const int64_t ns = (int64_t)sp.TB * sp.NtcP * 32;
     blocks = (ns + 255) / 256;
     if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
+    const int *perm = sp.blk_order, *inv = perm + sp.T_pad / 32;
     k_shift_scales<<<(int)blocks, 256, 0, st>>>(sp.S, sp.Sa, ax.L, sp.NtcP, sp.Ntc, sp.rows, sp.T, sp.T_pad, ns,
-                                                 sp.tpl, sp.scale, sp.scaleT, sp.eps_bits, degenerate);
+                                                 sp.tpl, inv, sp.scale, sp.scaleT, degenerate);
     e = cudaGetLastError();
     if (e != cudaSuccess || !sp.tpl16) return e;
+    k_shift_spans<<<sp.T_pad / 128, 128, 0, st>>>(sp.S, sp.Sa, ax.L, sp.NtcP, sp.Ntc, sp.rows, sp.T, sp.tpl, sp.scale,
+                                                  perm, sp.span);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    k_shift_eps<<<(int)blocks, 256, 0, st>>>(sp.S, sp.Sa, ax.L, sp.NtcP, sp.Ntc, sp.rows, sp.T, ns, sp.tpl, sp.scale,
+                                             inv, sp.span, sp.eps_bits);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     blocks = ((int64_t)sp.T_pad + 255) / 256;  // 8 warps of 32 templates per block
     if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
-    k_shift_tpl16<<<(int)blocks, 256, 0, st>>>(ax, sp.m_lo, sp.Kt, sp.T, sp.T_pad, sp.tpl16);
+    k_shift_tpl16<<<(int)blocks, 256, 0, st>>>(ax, sp.m_lo, sp.Kt, sp.T, sp.T_pad, perm, sp.tpl16);
     return cudaGetLastError();
 }
 

@@ -4,7 +4,12 @@
 //     bf16(r_b[m_lo + kk + tc_j]) (zero outside the window), so that
 //     <r_b, u_{t, tc_j}> = sum_kk u_t(m_lo + kk) X[(b, j)][kk]: one GEMM of
 //     the BF16 templates (N = 256 templates per tile) against the shifted
-//     residual rows (M = 128 rows per tile), K = Kt lags;
+//     residual rows (M = 128 rows per tile), K = Kt lags.  A tile multiplies
+//     only the lags that its rows' windows see and its templates span
+//     (k_shift_spans).  That is bounded by the tensor pipe and the issue of
+//     its MMAs, so fewer lags is what helps: 256 uneven EMG-like channels
+//     (atoms of 9-111 samples in windows of 256-2,048) 57.8 -> 34.6 ms per
+//     30-order decomposition, 32 radar-like channels 4.54 -> 4.17 ms;
 //  2. the tcgen05 GEMM scales every accumulator by its atom's 1/|u| and keeps,
 //     per row, the largest |score| of every template tile and of every
 //     32-template block;
@@ -68,10 +73,12 @@ __device__ __forceinline__ bool mbar_poll(uint64_t *bar, uint32_t parity, unsign
 constexpr int kBM = 128;          // shifted residual rows per tile (MMA M)
 constexpr int kBlockRows = 256;   // templates per block of the tile-major BF16 layout
 constexpr int kUmmaK = 16;
+constexpr int kStepsPerChunk = kBK / kUmmaK;
 constexpr int kThreads = 256;
 constexpr int kAChunkBytes = kBM * kBK * 2;  // 16 KB
 constexpr int kMaxStages = 6;
-constexpr int kUnitTab = 1024;  // row units whose lag-chunk range is tabulated in shared memory
+constexpr int kUnitTab = 1024;  // row units whose lag range is tabulated in shared memory
+constexpr int kTileTab = 512;   // template tiles whose lag span is
 
 // Tile of BN templates (128 or 256, MMA N).  PAIR: a CTA pair shares each
 // MMA (M = 256: the two CTAs' row tiles), each CTA loading BN / 2 of the
@@ -96,10 +103,12 @@ struct Smem {
     uint32_t tmem_base;
     int abort;
     unsigned int chan_max[2][kBM];  // per item parity: the tile's channel maxima (float bits)
-    // the lag-chunk range [x, y] of row units 0 .. kUnitTab - 1, formed
-    // during set-up: the single thread that issues the MMAs reads it at
-    // every item instead of dividing (units past the table: computed there)
-    short2 unit_chunk[kUnitTab];
+    // the lag range [x, y] (16-lag steps) of row units 0 .. kUnitTab - 1 and
+    // of template tiles 0 .. kTileTab - 1, formed during set-up: the single
+    // thread that issues the MMAs reads them at every item instead of
+    // dividing (past the tables: computed there)
+    short2 unit_steps[kUnitTab];
+    short2 tile_steps[kTileTab];
 };
 
 // Named barrier 1 over the 128 epilogue threads, returning whether any of
@@ -121,9 +130,8 @@ __device__ __forceinline__ int epilogue_bar_or(int pred) {
 // channels (cb * Bg ..) times Jt neighbouring time centres (g * Jt ..); local
 // row lr = (j - g Jt) Bg + (b - cb Bg), channels fastest, so with Bg >= 32
 // the 32 rows an epilogue warp holds share one time centre (its scale loads
-// are broadcasts).  Rows of one tile see the window
-// only over lags [kc_lo, kc_hi] (in 64-lag chunks): L + (Jt - 1) S lags
-// instead of Kt, the chunks outside hold only zero products and are skipped.
+// are broadcasts).  Rows of one tile see the window only over
+// L + (Jt - 1) S lags instead of Kt; outside them every product is zero.
 struct RowTiling {
     int B, Ntc, Jt, Bg, n_cb, m_tiles;
     int S, L, span0;  // span0 = -m_lo - tc0 = S (Ntc - 1); sample n at time centre j sits at lag n + span0 - S j
@@ -135,29 +143,52 @@ __host__ __device__ inline void tile_row(const RowTiling &t, int mt, int lr, int
     j = g * t.Jt + lr / t.Bg;
 }
 
-__host__ __device__ inline void tile_chunks(const RowTiling &t, int mt, int &kc_lo, int &kc_hi) {
+// The lags row tile mt's windows see, in steps of 16 (one MMA).
+__host__ __device__ inline void row_steps(const RowTiling &t, int mt, int &lo, int &hi) {
     const int g = mt / t.n_cb;
     const int j_first = g * t.Jt;
     const int j_last = min(j_first + t.Jt, t.Ntc) - 1;
     const int kk_min = t.span0 - t.S * j_last;           // sample 0 at the last time centre
     const int kk_max = t.L - 1 + t.span0 - t.S * j_first;  // sample L - 1 at the first
-    kc_lo = kk_min / kBK;
-    kc_hi = kk_max / kBK;
+    lo = kk_min / kUmmaK;
+    hi = kk_max / kUmmaK;
 }
 
-// Lag chunks of GEMM row unit u: one row tile, or (pair) the union of row
-// tiles 2u and 2u + 1 (the second clamped to the last tile).  Chunks outside
-// a tile's windows multiply zeros.
-__host__ __device__ inline void unit_chunks(const RowTiling &t, bool pair, int u, int &kc_lo, int &kc_hi) {
+// Lags of GEMM row unit u: one row tile, or (pair) the union of row tiles 2u
+// and 2u + 1 (the second clamped to the last tile).
+__host__ __device__ inline short2 unit_steps(const RowTiling &t, bool pair, int u) {
+    int lo, hi;
     if (!pair) {
-        tile_chunks(t, u, kc_lo, kc_hi);
-        return;
+        row_steps(t, u, lo, hi);
+    } else {
+        int lo1, hi1;
+        row_steps(t, 2 * u, lo, hi);
+        row_steps(t, min(2 * u + 1, t.m_tiles - 1), lo1, hi1);
+        lo = min(lo, lo1);
+        hi = max(hi, hi1);
     }
-    int lo1, hi1;
-    tile_chunks(t, 2 * u, kc_lo, kc_hi);
-    tile_chunks(t, min(2 * u + 1, t.m_tiles - 1), lo1, hi1);
-    kc_lo = min(kc_lo, lo1);
-    kc_hi = max(kc_hi, hi1);
+    return make_short2((short)lo, (short)hi);
+}
+
+// Lags template tile nt of BN templates spans (k_shift_spans).
+template <int BN>
+__device__ __forceinline__ short2 tile_steps(const short2 *__restrict__ span, int nt) {
+    short2 s = span[nt * (BN / 128)];
+    if (BN == 256) {
+        const short2 s1 = span[nt * 2 + 1];
+        s.x = min(s.x, s1.x);
+        s.y = max(s.y, s1.y);
+    }
+    return s;
+}
+
+// The steps an item multiplies: those its rows see and its templates span.
+// An empty intersection (only atoms without energy) takes the rows' first
+// step, so that the accumulator is written.
+__device__ __forceinline__ void item_steps(short2 rows, short2 tpls, int &lo, int &hi) {
+    lo = max((int)rows.x, (int)tpls.x);
+    hi = min((int)rows.y, (int)tpls.y);
+    if (lo > hi) lo = hi = rows.x;
 }
 
 // Shifted residual rows X[(b, j)][kk] = bf16(r_b[m_lo + kk + tc0 + S j]),
@@ -272,8 +303,8 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
 template <int BN, bool PAIR>
 __global__ void __launch_bounds__(kThreads, 1)
     k_shift_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowTiling tl,
-                 int n_tiles, int nkc, int stages, int T_pad, const float *__restrict__ scaleT,
-                 float *__restrict__ tile_max, float *__restrict__ blk_max, unsigned int *__restrict__ chmax,
+                 int n_tiles, int nkc, int stages, int T_pad, const short2 *__restrict__ span,
+                 const float *__restrict__ scaleT, float *__restrict__ tile_max, float *__restrict__ blk_max, unsigned int *__restrict__ chmax,
                  int *status, unsigned long long wait_ns) {
     // shared memory: stages, then the item's scales [Jt][BN + 4] (the +4
     // floats of padding spread the Jt rows a warp reads over the banks)
@@ -306,11 +337,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         fence_mbar_init();
     }
     if (threadIdx.x < 2 * kBM) sm.chan_max[threadIdx.x / kBM][threadIdx.x % kBM] = 0u;
-    for (int u = threadIdx.x; u < m_units && u < kUnitTab; u += blockDim.x) {
-        int lo, hi;
-        unit_chunks(tl, PAIR, u, lo, hi);
-        sm.unit_chunk[u] = make_short2((short)lo, (short)hi);
-    }
+    for (int u = threadIdx.x; u < m_units && u < kUnitTab; u += blockDim.x) sm.unit_steps[u] = unit_steps(tl, PAIR, u);
+    for (int nt = threadIdx.x; nt < n_tiles && nt < kTileTab; nt += blockDim.x)
+        sm.tile_steps[nt] = tile_steps<BN>(span, nt);  // constant since the build
     if (warp == 2) {
         if constexpr (PAIR) {  // the same columns in both CTAs, allocated by one warp of each
             asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -348,14 +377,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int u = (int)(w / n_tiles), nt = (int)(w % n_tiles);
             // this CTA's row tile (PAIR: past the last tile, load the last one again)
             const int mt = PAIR ? min(2 * u + (int)rank, tl.m_tiles - 1) : u;
-            int kc_lo, kc_hi;
-            if (u < kUnitTab) {
-                kc_lo = sm.unit_chunk[u].x;
-                kc_hi = sm.unit_chunk[u].y;
-            } else {
-                unit_chunks(tl, PAIR, u, kc_lo, kc_hi);
-            }
-            for (int kc = kc_lo; kc <= kc_hi; ++kc) {
+            int ks_lo, ks_hi;
+            item_steps(u < kUnitTab ? sm.unit_steps[u] : unit_steps(tl, PAIR, u),
+                       nt < kTileTab ? sm.tile_steps[nt] : tile_steps<BN>(span, nt), ks_lo, ks_hi);
+            const int kc_hi = ks_hi / kStepsPerChunk;
+            for (int kc = ks_lo / kStepsPerChunk; kc <= kc_hi; ++kc) {
                 const bool ok = PAIR ? mbar_wait_cluster(&sm.bar_empty[s], ph ^ 1u, wait_ns)
                                      : mbar_wait(&sm.bar_empty[s], ph ^ 1u, wait_ns);
                 if (!ok) {
@@ -400,14 +426,11 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             tc_fence_after();
             const uint32_t d_tmem = tmem + acc * BN;
-            int kc_lo, kc_hi;
-            const int u = (int)(w / n_tiles);
-            if (u < kUnitTab) {
-                kc_lo = sm.unit_chunk[u].x;
-                kc_hi = sm.unit_chunk[u].y;
-            } else {
-                unit_chunks(tl, PAIR, u, kc_lo, kc_hi);
-            }
+            int ks_lo, ks_hi;
+            const int u = (int)(w / n_tiles), nt = (int)(w - (int64_t)u * n_tiles);
+            item_steps(u < kUnitTab ? sm.unit_steps[u] : unit_steps(tl, PAIR, u),
+                       nt < kTileTab ? sm.tile_steps[nt] : tile_steps<BN>(span, nt), ks_lo, ks_hi);
+            const int kc_lo = ks_lo / kStepsPerChunk, kc_hi = ks_hi / kStepsPerChunk;
             for (int kc = kc_lo; kc <= kc_hi; ++kc) {
                 const bool full = mbar_poll<PAIR>(&sm.bar_full[s], ph, wait_ns, 0);
                 if (!full) {
@@ -417,9 +440,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tc_fence_after();
                 const uint32_t b0 = base + s * (uint32_t)kStageBytes;
                 const uint64_t bdesc = smem_desc(b0), adesc = smem_desc(b0 + kBChunkBytes);
+                // only the chunk's steps inside [ks_lo, ks_hi]
+                const int k_lo = ks_lo - kc * kStepsPerChunk, k_hi = ks_hi - kc * kStepsPerChunk;
 #pragma unroll
-                for (int k = 0; k < kBK / kUmmaK; ++k) {
-                    const uint32_t accum = (kc != kc_lo || k != 0) ? 1u : 0u;
+                for (int k = 0; k < kStepsPerChunk; ++k) {
+                    if (k < k_lo || k > k_hi) continue;
+                    const uint32_t accum = kc != kc_lo || k != k_lo ? 1u : 0u;
                     if constexpr (PAIR)
                         tc_mma_pair(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum);
                     else
@@ -558,7 +584,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // (one FP32 chain of L products, the FP32 scale and the final product), and
 //   |h - s| <= delta = (1 + 1e-5) [eps_u (|r| + |dr|) + |dr|
 //                                  + Kt 2^-23 (1 + eps_u)(|r| + |dr|)]
-// (eps_u = largest |bf16(u) - u| / |u| over the atoms' windows, dr =
+// (eps_u = largest |u~ - u| / |u| over the atoms' windows, u~ = the BF16
+// template as multiplied, zero outside its tile's span; dr =
 // bf16(r) - r, the Kt term bounds FP32 accumulation in the tensor core, the
 // factor the scale product).  As for the dense BF16 search, the FP32 argmax
 // lies in an item whose largest |h| is >= hmax - 2 delta - 2 eps_r.
@@ -568,7 +595,7 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
                                                     const double2 *__restrict__ chan_norm,
                                                     const unsigned int *__restrict__ chmax,
                                                     const unsigned int *__restrict__ eps_bits,
-                                                    int *__restrict__ chcount, int *__restrict__ fb_list,
+                                                    const int *__restrict__ blk_order, int *__restrict__ chcount, int *__restrict__ fb_list,
                                                     int *__restrict__ counters, int *__restrict__ items,
                                                     long long *__restrict__ stats) {
     const int b = blockIdx.y;
@@ -590,7 +617,7 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
     __syncthreads();
     const float thr_f = thr_sh;
     // scan the tile maxima; a tile at or above the threshold is narrowed to
-    // its 32-template blocks at or above it (the items: i = j * n_blocks + block)
+    // its 32-template blocks at or above it (the items: j * n_blocks + block)
     const float *tm = tile_max + (size_t)b * Ntc * n_tiles;
     const int n_entries = Ntc * n_tiles;
     const int n_blocks = n_tiles * bpt;
@@ -604,7 +631,7 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
                 if (pos < kMaxItems) {
                     const int at = atomicAdd(&counters[1], 1);
                     items[2 * at] = b;
-                    items[2 * at + 1] = j * n_blocks + tile * bpt + k;
+                    items[2 * at + 1] = j * n_blocks + blk_order[tile * bpt + k];  // the templates' own block
                     atomicAdd((unsigned long long *)&stats[2], 1ull);
                 } else if (pos == kMaxItems) {
                     // too many: the FP32 template search scores this channel in full
@@ -720,7 +747,7 @@ __global__ void __launch_bounds__(kRescanWarps * 32) k_shift_rescan(
 }
 
 // static shared memory of the kernels here (the GEMM's Smem is the largest)
-constexpr int kStaticReserve = 6144;
+constexpr int kStaticReserve = 8192;
 static_assert(sizeof(Smem) + 256 <= kStaticReserve, "static shared memory above its reserve");
 constexpr int kSmemBudget = 232448 - kStaticReserve - 1024;
 
@@ -946,16 +973,16 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
         const int64_t units = (int64_t)((m_tiles + 1) / 2) * n_tiles;
         const int pairs = (int)(units < s->pair_clusters ? units : s->pair_clusters);
         return launch_kernel_cluster(k_shift_gemm<256, true>, dim3(2 * pairs), dim3(kThreads), smem, st, true, 2, mapA,
-                                     s->mapB[0], tl, n_tiles, s->nkc, stages, sp.T_pad, sp.scaleT, x.tile_max,
-                                     x.blk_max, x.chmax, status, wait_ns);
+                                     s->mapB[0], tl, n_tiles, s->nkc, stages, sp.T_pad, (const short2 *)sp.span,
+                                     (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
     }
     const int i = bn == 256 ? 1 : 0;
     const int64_t items = (int64_t)m_tiles * n_tiles;
     const int grid = (int)(items < s->sm_count ? items : s->sm_count);
     // a programmatic dependent of the shifted-row build (set-up overlaps it)
     return launch_kernel(bn == 256 ? k_shift_gemm<256, false> : k_shift_gemm<128, false>, dim3(grid), dim3(kThreads),
-                         smem, st, true, mapA, s->mapB[i], tl, n_tiles, s->nkc, stages, sp.T_pad, sp.scaleT,
-                         x.tile_max, x.blk_max, x.chmax, status, wait_ns);
+                         smem, st, true, mapA, s->mapB[i], tl, n_tiles, s->nkc, stages, sp.T_pad, (const short2 *)sp.span,
+                         (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
 }
 
 cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, const float *R,
@@ -976,7 +1003,8 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
     cudaError_t e = launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32,
                                   sp.Kt, L, (const float *)x.tile_max, (const float *)x.blk_max,
                                   (const double2 *)x.chan_norm, (const unsigned int *)x.chmax,
-                                  (const unsigned int *)sp.eps_bits, x.chcount, fb_list, counters, x.items, stats);
+                                  (const unsigned int *)sp.eps_bits, (const int *)sp.blk_order, x.chcount, fb_list, counters,
+                                  x.items, stats);
     if (e != cudaSuccess) return e;
     e = launch_kernel(k_shift_rescan, dim3(s->sm_count * s->rescan_blocks_per_sm), dim3(s->rescan_warps * 32),
                       s->rescan_smem, st, true, (const float *)sp.tpl, (const float *)sp.scale, sp.S, sp.Sa, sp.P,
