@@ -74,7 +74,7 @@ constexpr int kBM = 128;          // shifted residual rows per tile (MMA M)
 constexpr int kBlockRows = 256;   // templates per block of the tile-major BF16 layout
 constexpr int kUmmaK = 16;
 constexpr int kStepsPerChunk = kBK / kUmmaK;
-constexpr int kThreads = 256;
+constexpr int kMaxThreads = 384;  // two epilogue groups
 constexpr int kAChunkBytes = kBM * kBK * 2;  // 16 KB
 constexpr int kMaxStages = 6;
 constexpr int kUnitTab = 1024;  // row units whose lag range is tabulated in shared memory
@@ -102,7 +102,7 @@ struct Smem {
     uint64_t bar_acc_empty[2];
     uint32_t tmem_base;
     int abort;
-    unsigned int chan_max[2][kBM];  // per item parity: the tile's channel maxima (float bits)
+    unsigned int chan_max[2][kBM];  // per epilogue group: the tile's channel maxima (float bits)
     // the lag range [x, y] (16-lag steps) of row units 0 .. kUnitTab - 1 and
     // of template tiles 0 .. kTileTab - 1, formed during set-up: the single
     // thread that issues the MMAs reads them at every item instead of
@@ -111,18 +111,27 @@ struct Smem {
     short2 tile_steps[kTileTab];
 };
 
-// Named barrier 1 over the 128 epilogue threads, returning whether any of
-// them passed a nonzero predicate (all of them get the same answer).
-__device__ __forceinline__ int epilogue_bar_or(int pred) {
+// Named barrier `id` over the 128 threads of one epilogue group, returning
+// whether any of them passed a nonzero predicate (all of them get the same
+// answer).
+__device__ __forceinline__ int epilogue_bar_or(int id, int pred) {
     int r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.s32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, 1, 128, p;\n\t"
+        "bar.red.or.pred q, %2, 128, p;\n\t"
         "selp.s32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
-        : "r"(pred)
+        : "r"(pred), "r"(id)
         : "memory");
+    return r;
+}
+__device__ __forceinline__ void epilogue_bar(int id) { asm volatile("bar.sync %0, 128;" ::"r"(id) : "memory"); }
+
+// max(|a|, |b|, |c|) in one instruction; a NaN operand is passed over, as fmaxf does.
+__device__ __forceinline__ float max_abs3(float a, float b, float c) {
+    float r;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
 
@@ -292,7 +301,10 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
 // GEMM work item w: row unit w / n_tiles, template tile w % n_tiles.  Every
 // stage holds one template chunk (BN x 64) and the matching residual chunk
 // (128 x 64).  Warp 0: TMA producer; warp 1: MMA issuer; warp 2: tensor
-// memory owner; warps 4-7: epilogue (thread = residual row).
+// memory owner; warps 4-7, and 8-11 where launched: epilogue groups (thread =
+// residual row).  Two groups take alternate items, one accumulator each: a
+// narrow tile's MMAs take less time than one group needs to stage a tile's
+// scales, read its accumulator and store its maxima.
 //
 // PAIR (launched as clusters of 2): a unit is the row tiles 2u and 2u + 1,
 // one per CTA of the pair, over the union of their lag chunks.  Each CTA
@@ -301,7 +313,7 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
 // its commits arrive on both CTAs' barriers; each CTA's epilogue reads its
 // own accumulator and releases it on the leader's barrier.
 template <int BN, bool PAIR>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kMaxThreads, 1)
     k_shift_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowTiling tl,
                  int n_tiles, int nkc, int stages, int T_pad, const short2 *__restrict__ span,
                  const float *__restrict__ scaleT, float *__restrict__ tile_max, float *__restrict__ blk_max, unsigned int *__restrict__ chmax,
@@ -467,12 +479,14 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp >= 4) {
         // ---------------- epilogue: thread = shifted residual row ----------------
-        const int q = warp - 4;
-        const int et = threadIdx.x - 128;  // 0..127 over the epilogue warps
+        const int eg = (warp - 4) >> 2, q = warp & 3;  // this warp's group; its quarter of the tensor-memory lanes
+        const uint32_t n_eg = (blockDim.x - 128) >> 7;
+        const int et = threadIdx.x & 127, bar_id = 1 + eg;
         constexpr int kScaleLd = BN + 4;
-        float *sc_sm = reinterpret_cast<float *>(dyn_raw + (base - smem_u32(dyn_raw)) + (size_t)stages * kStageBytes);
-        uint32_t local = 0;
-        for (int64_t w = unit0; w < items; w += n_units, ++local) {
+        float *sc_sm = reinterpret_cast<float *>(dyn_raw + (base - smem_u32(dyn_raw)) + (size_t)stages * kStageBytes) +
+                       (size_t)eg * tl.Jt * kScaleLd;
+        uint32_t local = (uint32_t)eg;
+        for (int64_t w = unit0 + eg * n_units; w < items; w += n_eg * n_units, local += n_eg) {
             const int unit = (int)(w / n_tiles), nt = (int)(w % n_tiles);
             const int mt = PAIR ? 2 * unit + (int)rank : unit;  // PAIR: may be one past the last tile (no rows)
             // the tile's Jt scale rows (j0 .. j0 + Jt - 1, those below Ntc), BN each
@@ -487,12 +501,12 @@ __global__ void __launch_bounds__(kThreads, 1)
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
                 }
                 asm volatile("cp.async.wait_all;" ::: "memory");
-                asm volatile("bar.sync 1, 128;" ::: "memory");
+                epilogue_bar(bar_id);
             }
             const uint32_t acc = local & 1u, aph = (local >> 1) & 1u;
             const bool landed = mbar_poll<PAIR>(&sm.bar_acc_full[acc], aph, wait_ns, 256);
             const int failed = (*abort_flag || !landed) ? 1 : 0;
-            if (epilogue_bar_or(failed)) {  // the epilogue warps leave together
+            if (epilogue_bar_or(bar_id, failed)) {  // the group's warps leave together
                 *abort_flag = 1;
                 break;
             }
@@ -516,10 +530,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const float4 s = valid ? sc4[c * 8 + e] : make_float4(0.f, 0.f, 0.f, 0.f);
                     const float2 p01 = mul_f32x2(v[4 * e], v[4 * e + 1], s.x, s.y);
                     const float2 p23 = mul_f32x2(v[4 * e + 2], v[4 * e + 3], s.z, s.w);
-                    m0 = fmaxf(m0, fabsf(p01.x));
-                    m1 = fmaxf(m1, fabsf(p01.y));
-                    m0 = fmaxf(m0, fabsf(p23.x));
-                    m1 = fmaxf(m1, fabsf(p23.y));
+                    m0 = max_abs3(m0, p01.x, p01.y);
+                    m1 = max_abs3(m1, p23.x, p23.y);
                 }
                 bmv[c] = fmaxf(m0, m1);
                 mx = fmaxf(mx, bmv[c]);
@@ -547,13 +559,13 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const unsigned o = __shfl_xor_sync(0xffffffffu, bits, off);
                 bits = o > bits ? o : bits;
             }
-            unsigned int *cm = sm.chan_max[local & 1u];
+            unsigned int *cm = sm.chan_max[eg];
             if (tl.Bg >= 32 || lane < tl.Bg) atomicMax(cm + lr % tl.Bg, bits);
-            asm volatile("bar.sync 1, 128;" ::: "memory");  // also: the scale rows are reloaded for the next item
+            epilogue_bar(bar_id);  // also: the scale rows are reloaded for the next item
             if (et < tl.Bg) {
                 const int bc = (mt % tl.n_cb) * tl.Bg + et;
                 if (bc < tl.B) atomicMax(chmax + bc, cm[et]);
-                cm[et] = 0u;  // rewritten two items later, after another barrier
+                cm[et] = 0u;  // the next item adds to it after the barrier that follows its scale rows
             }
         }
     }
@@ -791,7 +803,7 @@ cudaError_t shift_tc_prepare(ShiftTc **out, const ShiftPlan &sp, int sm_count) {
         attr[0].val.clusterDim.y = 1;
         attr[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(2 * (unsigned)sm_count);
-        cfg.blockDim = dim3(kThreads);
+        cfg.blockDim = dim3(kMaxThreads);
         cfg.dynamicSmemBytes = 1024 + (size_t)kSmemBudget;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
@@ -891,36 +903,42 @@ cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, Shift
 // GEMM form of a B-channel launch: the template tile width (256 unless that
 // leaves SMs idle or leaves room for fewer than two stages beside the tile's
 // scale rows) and whether CTA pairs share each MMA (256-wide tiles, at least
-// two row tiles, a work unit for every pair that fits, pairs allowed).
+// two row tiles, a work unit for every pair that fits, pairs allowed).  Two
+// epilogue groups (*threads) where a second set of scale rows costs no stage
+// below four.
 static int shift_tc_bn(const ShiftTc *s, const ShiftPlan &sp, const RowTiling &tl, bool pairs_allowed, int *stages,
-                       size_t *smem, bool *pair) {
+                       size_t *smem, bool *pair, int *threads) {
     auto smem_for = [&](int bn, int stage_bytes, int *stg_out) {
         const size_t sc = (size_t)tl.Jt * (bn + 4) * sizeof(float);
-        int stg = (int)((kSmemBudget - (int64_t)sc) / stage_bytes);
+        int groups = 2;
+        int stg = (int)((kSmemBudget - 2 * (int64_t)sc) / stage_bytes);
+        if (stg < 4) {
+            groups = 1;
+            stg = (int)((kSmemBudget - (int64_t)sc) / stage_bytes);
+        }
         stg = stg > kMaxStages ? kMaxStages : stg;
         *stg_out = stg;
-        return 1024 + (size_t)stg * stage_bytes + sc;
+        *threads = 128 + 128 * groups;
+        return 1024 + (size_t)stg * stage_bytes + groups * sc;
     };
     *pair = false;
     int st256 = 0;
-    const size_t sm256 = smem_for(256, ShiftTile<256>::kStageBytes, &st256);
+    smem_for(256, ShiftTile<256>::kStageBytes, &st256);
     if ((int64_t)tl.m_tiles * (sp.T_pad / 256) >= s->sm_count && st256 >= 2) {
         int stp = 0;
-        const size_t smp = smem_for(256, ShiftTile<256, true>::kStageBytes, &stp);
+        smem_for(256, ShiftTile<256, true>::kStageBytes, &stp);
         const int64_t units = (int64_t)((tl.m_tiles + 1) / 2) * (sp.T_pad / 256);
         if (pairs_allowed && s->pair_clusters > 0 && tl.m_tiles >= 2 && units >= s->pair_clusters && stp >= 2) {
             // the whole budget: every operand read of a stage's MMAs stays
             // inside the allocation even at the last stage
             static_assert((kMaxStages - 1) * ShiftTile<256, true>::kStageBytes + 48 * 1024 <= kSmemBudget,
                           "paired stages beyond the shared-memory budget");
-            (void)smp;
             *pair = true;
             *stages = stp;
             *smem = 1024 + (size_t)kSmemBudget;
             return 256;
         }
-        *stages = st256;
-        *smem = sm256;
+        *smem = smem_for(256, ShiftTile<256>::kStageBytes, stages);
         return 256;
     }
     *smem = smem_for(128, ShiftTile<128>::kStageBytes, stages);
@@ -929,10 +947,10 @@ static int shift_tc_bn(const ShiftTc *s, const ShiftPlan &sp, const RowTiling &t
 
 bool shift_tc_uses_pairs(const ShiftTc *s, const ShiftPlan &sp, int B, bool pairs_allowed) {
     if (!s || B < 1) return false;
-    int stages = 0;
+    int stages = 0, threads = 0;
     size_t smem = 0;
     bool pair = false;
-    shift_tc_bn(s, sp, make_tiling(sp, B), pairs_allowed, &stages, &smem, &pair);
+    shift_tc_bn(s, sp, make_tiling(sp, B), pairs_allowed, &stages, &smem, &pair, &threads);
     return pair;
 }
 
@@ -962,17 +980,17 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
     const int m_tiles = tl.m_tiles;
     CUtensorMap mapA;
     if (!make_map(&mapA, x.X, (uint64_t)sp.Kt, (uint64_t)m_tiles * kBM, kBM)) return cudaErrorInvalidValue;
-    int stages = 0;
+    int stages = 0, threads = 0;
     size_t smem = 0;
     bool pair = false;
-    const int bn = shift_tc_bn(s, sp, tl, pairs_allowed, &stages, &smem, &pair);
+    const int bn = shift_tc_bn(s, sp, tl, pairs_allowed, &stages, &smem, &pair, &threads);
     const int n_tiles = sp.T_pad / bn;
     if (stages < 2) return cudaErrorInvalidValue;
     if (pair) {
         // clusters of 2: each CTA loads 128-template halves (box height 128)
         const int64_t units = (int64_t)((m_tiles + 1) / 2) * n_tiles;
         const int pairs = (int)(units < s->pair_clusters ? units : s->pair_clusters);
-        return launch_kernel_cluster(k_shift_gemm<256, true>, dim3(2 * pairs), dim3(kThreads), smem, st, true, 2, mapA,
+        return launch_kernel_cluster(k_shift_gemm<256, true>, dim3(2 * pairs), dim3(threads), smem, st, true, 2, mapA,
                                      s->mapB[0], tl, n_tiles, s->nkc, stages, sp.T_pad, (const short2 *)sp.span,
                                      (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
     }
@@ -980,7 +998,7 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
     const int64_t items = (int64_t)m_tiles * n_tiles;
     const int grid = (int)(items < s->sm_count ? items : s->sm_count);
     // a programmatic dependent of the shifted-row build (set-up overlaps it)
-    return launch_kernel(bn == 256 ? k_shift_gemm<256, false> : k_shift_gemm<128, false>, dim3(grid), dim3(kThreads),
+    return launch_kernel(bn == 256 ? k_shift_gemm<256, false> : k_shift_gemm<128, false>, dim3(grid), dim3(threads),
                          smem, st, true, mapA, s->mapB[i], tl, n_tiles, s->nkc, stages, sp.T_pad, (const short2 *)sp.span,
                          (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
 }
@@ -991,10 +1009,10 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
                                     unsigned long long wait_ns) {
     if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
     const RowTiling tl = make_tiling(sp, B);
-    int stages = 0;
+    int stages = 0, threads = 0;
     size_t smem = 0;
     bool pair = false;
-    const int bn = shift_tc_bn(s, sp, tl, false, &stages, &smem, &pair);  // the GEMM's tile width for B channels
+    const int bn = shift_tc_bn(s, sp, tl, false, &stages, &smem, &pair, &threads);  // the GEMM's tile width for B channels
     const int n_tiles = sp.T_pad / bn;
     const int entries = sp.Ntc * n_tiles;
     int slices = (entries + 255) / 256;
