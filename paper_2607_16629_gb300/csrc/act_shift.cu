@@ -147,10 +147,45 @@ __global__ void __launch_bounds__(256) k_shift_tpl16(GridAxes ax, int m_lo, int 
     }
 }
 
-// One thread per (template block, lag, lane): |u|^2 over the window (a
+// What a window's samples of one template add up to, for kSumJ neighbouring
+// time centres j0 .. j0 + kSumJ - 1 per thread (lane = template).  Sample
+// n = a + S p of time centre j sits in phase a, row p - j + NtcP - 1: the
+// windows of neighbouring time centres overlap in all but one row, so every
+// template row is read once for all kSumJ of them; each window still adds its
+// own samples in the order a, p.  add(q, a, p, u) takes sample (a, p) of j0 + q.
+constexpr int kSumJ = 8;
+
+template <typename Add>
+__device__ __forceinline__ void window_rows(const float *__restrict__ base, int S, int Sa, int L, int rows, int first,
+                                            Add add) {
+    for (int a = 0; a < Sa; ++a) {
+        const int n_p = (L - a + S - 1) / S;  // samples of phase a
+        const float *col = base + ((size_t)a * rows + first - (kSumJ - 1)) * 32;
+        // row i (from the last time centre's first) is sample p = i - (kSumJ - 1 - q) of time centre j0 + q
+        const int n_i = n_p + kSumJ - 1;
+        for (int i = 0; i < n_i; ++i) {
+            const float u = col[(size_t)i * 32];
+            if (i >= kSumJ - 1 && i < n_p) {
+#pragma unroll
+                for (int q = 0; q < kSumJ; ++q) add(q, a, i - (kSumJ - 1 - q), u);
+            } else {
+#pragma unroll
+                for (int q = 0; q < kSumJ; ++q) {
+                    const int p = i - (kSumJ - 1 - q);
+                    if (p >= 0 && p < n_p) add(q, a, p, u);
+                }
+            }
+        }
+    }
+}
+
+// Per (template block, kSumJ lags, lane): |u|^2 over the window (a
 // float-float sum) and the scale 1/|u| in both layouts ([TB][NtcP][32] for
 // the FP32 search, [NtcP][T_pad] in the BF16 view's template order for the
-// tensor-core epilogue; inv[tb] = where block tb sits in that order).
+// tensor-core epilogue; inv[tb] = where block tb sits in that order).  Bound
+// by the float-float adds; with one time centre per thread it waited on a
+// load and a dependent chain per sample (EEG-like grid, with the error bound:
+// 2.0 ms, now 0.6 and k_shift_eps 0.5; radar-like 16 ms, now 3.8 and 2.5).
 __global__ void __launch_bounds__(256) k_shift_scales(int S, int Sa, int L, int NtcP, int Ntc, int rows, int T,
                                                       int T_pad, int64_t total, const float *__restrict__ tpl,
                                                       const int *__restrict__ inv, float *__restrict__ scale,
@@ -160,29 +195,29 @@ __global__ void __launch_bounds__(256) k_shift_scales(int S, int Sa, int L, int 
          i += (int64_t)gridDim.x * blockDim.x) {
         const int lane = (int)(i & 31);
         const int64_t rest = i >> 5;
-        const int j = (int)(rest % NtcP);
-        const int64_t tb = rest / NtcP;
-        const int64_t t = tb * 32 + lane;
-        float sc = 0.0f;
-        if (t < T && j < Ntc) {
-            ff ef = {0.0f, 0.0f};
-            const float *base = tpl + (size_t)tb * Sa * rows * 32 + lane;
-            // sample n = a + S p sits in phase a, row p - j + NtcP - 1
-            for (int a = 0; a < Sa; ++a) {
-                const float *col = base + ((size_t)a * rows + (NtcP - 1 - j)) * 32;
-                for (int p = 0; a + S * p < L; ++p) {
-                    const float u = col[(size_t)p * 32];
-                    ff_fma_acc(ef, u, u);
-                }
+        const int j0 = (int)(rest % (NtcP / kSumJ)) * kSumJ;
+        const int64_t tb = rest / (NtcP / kSumJ);
+        const bool valid = tb * 32 + lane < T;
+        ff ef[kSumJ];
+#pragma unroll
+        for (int q = 0; q < kSumJ; ++q) ef[q] = {0.0f, 0.0f};
+        if (valid && j0 < Ntc)
+            window_rows(tpl + (size_t)tb * Sa * rows * 32 + lane, S, Sa, L, rows, NtcP - 1 - j0,
+                        [&](int q, int, int, float u) { ff_fma_acc(ef[q], u, u); });
+#pragma unroll
+        for (int q = 0; q < kSumJ; ++q) {
+            const int j = j0 + q;
+            float sc = 0.0f;
+            if (valid && j < Ntc) {
+                const double e = ff_to_double(ef[q]);
+                if (e > 0.0 && isfinite(e))
+                    sc = (float)(1.0 / sqrt(e));
+                else if (degenerate)
+                    atomicAdd(degenerate, 1ull);
             }
-            const double e = ff_to_double(ef);
-            if (e > 0.0 && isfinite(e))
-                sc = (float)(1.0 / sqrt(e));
-            else if (degenerate)
-                atomicAdd(degenerate, 1ull);
+            scale[((size_t)tb * NtcP + j) * 32 + lane] = sc;
+            if (scaleT) scaleT[(size_t)j * T_pad + (size_t)inv[tb] * 32 + lane] = sc;
         }
-        scale[i] = sc;
-        if (scaleT) scaleT[(size_t)j * T_pad + (size_t)inv[tb] * 32 + lane] = sc;
     }
 }
 
@@ -198,7 +233,7 @@ __global__ void __launch_bounds__(256) k_shift_scales(int S, int Sa, int L, int 
 // side) is small beside the rounding error itself (about 2^-9 |u|): the
 // bound grows by a few percent and the multiplied lags end near 3.7 Dt.
 //
-// One warp per 32-template block, lane = template.  Going up from lag 0, C =
+// Two warps per 32-template block (one a side), lane = template.  Going up from lag 0, C =
 // energy below p; the window of time centre j starts at S (Ntc - 1 - j), and
 // lags below p may go while C(p) - C(start) <= tau |u_j|^2 for every window
 // that starts below p.  The upper end mirrors it.  Sums of FP32 squares grow
@@ -206,11 +241,12 @@ __global__ void __launch_bounds__(256) k_shift_scales(int S, int Sa, int L, int 
 // cut, the error bound is formed from the cut as made.
 constexpr float kSpanTau = 1.1920929e-07f;
 
-__global__ void __launch_bounds__(128) k_shift_spans(int S, int Sa, int L, int NtcP, int Ntc, int rows, int T,
+__global__ void __launch_bounds__(256) k_shift_spans(int S, int Sa, int L, int NtcP, int Ntc, int rows, int T,
                                                      const float *__restrict__ tpl, const float *__restrict__ scale,
                                                      const int *__restrict__ perm, short2 *__restrict__ span) {
     __shared__ int lo_s[4], hi_s[4];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) & 3;
+    const bool upper = threadIdx.x >= 128;  // warps 4-7: the upper ends
     const int64_t tb = perm[blockIdx.x * 4 + warp];
     const bool valid = tb * 32 + lane < T;
     const int used = S * (Ntc - 1) + L;  // lags any window sees
@@ -229,7 +265,7 @@ __global__ void __launch_bounds__(128) k_shift_spans(int S, int Sa, int L, int N
             return v > 0.0f ? kSpanTau / (v * v) : __int_as_float(0x7f800000);
         };
         constexpr int U = 8;
-        bool live = valid;
+        bool live = valid && !upper;
         float lim = __int_as_float(0x7f800000), c = 0.0f;
         for (int k0 = 0; k0 < used && __any_sync(0xffffffffu, live); k0 += U) {
             float e[U];
@@ -246,7 +282,7 @@ __global__ void __launch_bounds__(128) k_shift_spans(int S, int Sa, int L, int N
                 }
             }
         }
-        live = valid;
+        live = valid && upper;
         lim = __int_as_float(0x7f800000);
         c = 0.0f;
         for (int k0 = used - 1; k0 >= 0 && __any_sync(0xffffffffu, live); k0 -= U) {
@@ -269,13 +305,11 @@ __global__ void __launch_bounds__(128) k_shift_spans(int S, int Sa, int L, int N
         lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, off));
         hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, off));
     }
-    if (lane == 0) {
-        lo_s[warp] = lo;
-        hi_s[warp] = hi;
-    }
+    if (lane == 0 && !upper) lo_s[warp] = lo;
+    if (lane == 0 && upper) hi_s[warp] = hi;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int w = 1; w < 4; ++w) {
+        for (int w = 0; w < 4; ++w) {
             lo = min(lo, lo_s[w]);
             hi = max(hi, hi_s[w]);
         }
@@ -301,24 +335,27 @@ __global__ void __launch_bounds__(256) k_shift_eps(int S, int Sa, int L, int Ntc
          i += (int64_t)gridDim.x * blockDim.x) {
         const int lane = (int)(i & 31);
         const int64_t rest = i >> 5;
-        const int j = (int)(rest % NtcP);
-        const int64_t tb = rest / NtcP;
-        const float sc = scale[i];
-        if (tb * 32 + lane >= T || j >= Ntc || sc == 0.0f) continue;
+        const int j0 = (int)(rest % (NtcP / kSumJ)) * kSumJ;
+        const int64_t tb = rest / (NtcP / kSumJ);
+        if (tb * 32 + lane >= T || j0 >= Ntc) continue;
         const short2 sp = span[inv[tb] >> 2];
-        // samples n = kk - S (Ntc - 1 - j) of the kept lags
-        const int n_lo = 16 * sp.x - S * (Ntc - 1 - j), n_hi = 16 * (sp.y + 1) - S * (Ntc - 1 - j);
-        float de = 0.0f;
-        const float *base = tpl + (size_t)tb * Sa * rows * 32 + lane;
-        for (int a = 0; a < Sa; ++a) {
-            const float *col = base + ((size_t)a * rows + (NtcP - 1 - j)) * 32;
-            for (int p = 0, n = a; n < L; ++p, n += S) {
-                const float u = col[(size_t)p * 32];
-                const float d = n >= n_lo && n < n_hi ? __bfloat162float(__float2bfloat16_rn(u)) - u : u;
-                de = fmaf(d, d, de);
-            }
+        float de[kSumJ];
+#pragma unroll
+        for (int q = 0; q < kSumJ; ++q) de[q] = 0.0f;
+        // sample n of time centre j is lag n + S (Ntc - 1 - j): the same lag, and the same error, for every window
+        const int lag0 = S * (Ntc - 1 - j0), k_lo = 16 * sp.x, k_hi = 16 * (sp.y + 1);
+        window_rows(tpl + (size_t)tb * Sa * rows * 32 + lane, S, Sa, L, rows, NtcP - 1 - j0,
+                    [&](int q, int a, int p, float u) {
+                        const int kk = a + S * (p - q) + lag0;
+                        const float d = kk >= k_lo && kk < k_hi ? __bfloat162float(__float2bfloat16_rn(u)) - u : u;
+                        de[q] = fmaf(d, d, de[q]);
+                    });
+#pragma unroll
+        for (int q = 0; q < kSumJ; ++q) {
+            if (j0 + q >= Ntc) continue;
+            const float sc = scale[((size_t)tb * NtcP + j0 + q) * 32 + lane];
+            if (sc > 0.0f) worst = fmaxf(worst, __double2float_ru(sqrt((double)de[q]) * (double)sc * (1.0 + 1e-3)));
         }
-        worst = fmaxf(worst, __double2float_ru(sqrt((double)de) * (double)sc * (1.0 + 1e-3)));
     }
     for (int off = 16; off > 0; off >>= 1) worst = fmaxf(worst, __shfl_xor_sync(0xffffffffu, worst, off));
     if ((threadIdx.x & 31) == 0) atomicMax(eps_bits, __float_as_uint(worst));
@@ -695,7 +732,7 @@ cudaError_t launch_shift_build(const ShiftPlan &sp, const GridAxes &ax, unsigned
     k_shift_templates<<<(int)blocks, 256, 0, st>>>(ax, sp.S, sp.Sa, sp.tc0, sp.NtcP, sp.rows, sp.T, nt, sp.tpl);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t ns = (int64_t)sp.TB * sp.NtcP * 32;
+    const int64_t ns = (int64_t)sp.TB * (sp.NtcP / kSumJ) * 32;
     blocks = (ns + 255) / 256;
     if (blocks > (int64_t)sm_count * 16) blocks = (int64_t)sm_count * 16;
     const int *perm = sp.blk_order, *inv = perm + sp.T_pad / 32;
@@ -703,7 +740,7 @@ cudaError_t launch_shift_build(const ShiftPlan &sp, const GridAxes &ax, unsigned
                                                  sp.tpl, inv, sp.scale, sp.scaleT, degenerate);
     e = cudaGetLastError();
     if (e != cudaSuccess || !sp.tpl16) return e;
-    k_shift_spans<<<sp.T_pad / 128, 128, 0, st>>>(sp.S, sp.Sa, ax.L, sp.NtcP, sp.Ntc, sp.rows, sp.T, sp.tpl, sp.scale,
+    k_shift_spans<<<sp.T_pad / 128, 256, 0, st>>>(sp.S, sp.Sa, ax.L, sp.NtcP, sp.Ntc, sp.rows, sp.T, sp.tpl, sp.scale,
                                                   perm, sp.span);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
