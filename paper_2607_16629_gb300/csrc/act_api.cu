@@ -187,6 +187,7 @@ void drop_graphs(act_grid *g) {
 void free_lem(WorkBuffers &w) {
     free_dev(w.lem.cand);
     free_dev(w.lem.score);
+    free_dev(w.lem.screen);
     free_dev(w.lem.kept);
     free_dev(w.lem.kept_score);
     free_dev(w.lem.ncand);
@@ -288,6 +289,7 @@ act_status alloc_lem(const act_grid *g, WorkBuffers &w, int B) {
     const int k = g->lem.top_k;
     ACT_AL(w.lem.cand, sizeof(double) * 4 * (size_t)B * cap);
     ACT_AL(w.lem.score, sizeof(double) * (size_t)B * cap);
+    ACT_AL(w.lem.screen, sizeof(float2) * (size_t)B * cap);
     ACT_AL(w.lem.kept, sizeof(double) * 4 * (size_t)B * k);
     ACT_AL(w.lem.kept_score, sizeof(double) * (size_t)B * k);
     ACT_AL(w.lem.ncand, sizeof(int) * (size_t)B);

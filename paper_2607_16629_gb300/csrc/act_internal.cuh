@@ -184,6 +184,7 @@ struct LemBuffers {
     int cap = 0;                  // candidates per channel
     double *cand = nullptr;       // [B][cap][4]
     double *score = nullptr;      // [B][cap]
+    float2 *screen = nullptr;     // [B][cap] FP32 |score| and its error bound over |r|
     double *kept = nullptr;       // [B][top_k][4]
     double *kept_score = nullptr; // [B][top_k]
     int *ncand = nullptr;         // [B]

@@ -8,6 +8,10 @@
 //   3. per refinement level, the local neighbourhood dictionary of each kept
 //      candidate (offsets -R..R steps of that level per axis, clamped to the
 //      box), all candidates pooled, projected and reranked to a new top_k;
+//      (2 and 3 as two kernels a level: k_lem_screen projects every candidate
+//      in plain FP32 with an error bound, k_lem_pick projects again, in
+//      float-float, those that the bound leaves among the top_k, and keeps
+//      the top_k by that score: the selection is the float-float score's)
 //   4. the best candidate then starts the BFGS refinement (act_refine.cu).
 // The random draws come from SplitMix64 (Steele, Lea and Flood, 2014): draw
 // n of a stream seeded s is mix(s + (n + 1) 0x9E3779B97F4A7C15), with n
@@ -38,281 +42,564 @@ __device__ __forceinline__ uint64_t lem_counter(int channel, int order, int axis
            (uint64_t)i;
 }
 
-// 1. Latin hypercube: one block per (channel, axis); keys sorted in shared
-// memory (bitonic sort over npow2 >= n entries, padding keys sort last).
-__global__ void __launch_bounds__(kLemThreads) k_lem_lhs(int n, int npow2, LemBox box, uint64_t seed, int order,
+// 1. Latin hypercube: one block per (channel, axis).  The stratum of sample i
+// is the rank of its key (all keys of a call differ: SplitMix64's mix is a
+// bijection).  The keys are uniform, so the rank comes from 2^log2b >= n / 2
+// buckets of the leading bits: count, scan, gather, and compare within the
+// bucket (a key or two each).  Five barriers; a bitonic sort of 2,048 keys took 66 steps
+// (69 us against 15 per order at 64 channels).
+constexpr int kLhsThreads = 512;
+
+__global__ void __launch_bounds__(kLhsThreads) k_lem_lhs(int n, int log2b, LemBox box, uint64_t seed, int order,
                                                         int cap, double *__restrict__ cand, int *__restrict__ ncand) {
     extern __shared__ uint8_t sm_raw[];
-    uint64_t *key = reinterpret_cast<uint64_t *>(sm_raw);
-    uint32_t *idx = reinterpret_cast<uint32_t *>(key + npow2);
+    __shared__ uint32_t part[kLhsThreads / 32];
+    const int nb = 1 << log2b;
+    uint64_t *key = reinterpret_cast<uint64_t *>(sm_raw);         // [n] gathered by bucket
+    uint32_t *start = reinterpret_cast<uint32_t *>(key + n);      // [nb] first position of each bucket
+    uint32_t *fill = start + nb;                                  // [nb] keys counted, then gathered
     const int b = blockIdx.x, a = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double *out = cand + (size_t)b * cap * 4;
-    for (int i = threadIdx.x; i < npow2; i += blockDim.x) {
-        key[i] = i < n ? splitmix64_at(seed, lem_counter(b, order, a, 0, i)) : ~0ull;
-        idx[i] = (uint32_t)i;
+    auto bucket = [&](uint64_t k) { return log2b ? (uint32_t)(k >> (64 - log2b)) : 0u; };
+    for (int i = threadIdx.x; i < nb; i += blockDim.x) fill[i] = 0u;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        atomicAdd(&fill[bucket(splitmix64_at(seed, lem_counter(b, order, a, 0, i)))], 1u);
+    __syncthreads();
+    // exclusive scan: each thread its run of buckets, then the warps, then the block
+    const int per = (nb + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int lo = min(nb, (int)threadIdx.x * per), hi = min(nb, lo + per);
+    uint32_t sum = 0u;
+    for (int i = lo; i < hi; ++i) sum += fill[i];
+    uint32_t incl = sum;
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
+    }
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    uint32_t at = incl - sum;
+    for (int w = 0; w < warp; ++w) at += part[w];
+    for (int i = lo; i < hi; ++i) {
+        const uint32_t c = fill[i];
+        start[i] = at;
+        fill[i] = 0u;
+        at += c;
     }
     __syncthreads();
-    for (int size = 2; size <= npow2; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < npow2; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const bool up = (i & size) == 0;
-                    const uint64_t ki = key[i], kj = key[j];
-                    if ((ki > kj) == up) {
-                        key[i] = kj;
-                        key[j] = ki;
-                        const uint32_t t = idx[i];
-                        idx[i] = idx[j];
-                        idx[j] = t;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint64_t k = splitmix64_at(seed, lem_counter(b, order, a, 0, i));
+        const uint32_t q = bucket(k);
+        key[start[q] + atomicAdd(&fill[q], 1u)] = k;
     }
-    // sorted position p is the stratum (rank) of sample idx[p].  For n a
-    // power of two the quotient (p + u) / n is the exact product with 2^-k:
-    // the same correctly rounded value without an FP64 division
+    __syncthreads();
+    // For n a power of two the quotient (p + u) / n is the exact product with
+    // 2^-k: the same correctly rounded value without an FP64 division
     const bool pow2 = (n & (n - 1)) == 0;
     const double inv_n = pow2 ? __longlong_as_double((long long)(1023 - (31 - __clz(n))) << 52) : 0.0;
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        const int i = (int)idx[p];
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint64_t k = splitmix64_at(seed, lem_counter(b, order, a, 0, i));
+        const uint32_t q = bucket(k), s0 = start[q], s1 = s0 + fill[q];
+        uint32_t p = s0;  // the rank
+        for (uint32_t e = s0; e < s1; ++e) p += key[e] < k ? 1u : 0u;
         const uint64_t h = splitmix64_at(seed, lem_counter(b, order, a, 1, i));
         const double u = (double)(h >> 11) * 0x1.0p-53;
-        const double q = __dadd_rn((double)p, u);
-        const double t = pow2 ? __dmul_rn(q, inv_n) : __ddiv_rn(q, (double)n);
+        const double v = __dadd_rn((double)p, u);
+        const double t = pow2 ? __dmul_rn(v, inv_n) : __ddiv_rn(v, (double)n);
         out[4 * i + a] = __dadd_rn(box.lo[a], __dmul_rn(t, __dadd_rn(box.hi[a], -box.lo[a])));
     }
     if (threadIdx.x == 0 && a == 0) ncand[b] = n;
 }
 
-// 2. Scores s = <r, u>/|u| of every candidate of every channel.  A block
-// takes kScoreCands candidates of one channel: their per-atom constants are
-// formed once (FP64, one thread per candidate), then each warp runs its
-// candidates one after another, lane = sample stride 32.  A lane's samples
-// n_k = lane + 32 k advance tau by D = 32 / fs, so the phase
-// (c tau + fc) tau steps by d1_k = D (c (2 tau_k + D) + fc), and d1 by
-// d2 = 2 c D^2: tau, the phase and d1 are carried by these recurrences in
-// float-float (phase and d1 mod 1), from exact starting values at k = 0.
+// The candidate that offset o (0 .. per - 1, c fastest) of the neighbourhood
+// of kept parameters th names, clamped to the box.
+__device__ __forceinline__ void lem_neighbour(const double *__restrict__ th, int o, const LemBox &box,
+                                              const LemLevel &lev, double *p) {
+#pragma unroll
+    for (int a = 3; a >= 0; --a) {
+        const int w = 2 * lev.radius[a] + 1;
+        const double v = __dadd_rn(th[a], __dmul_rn((double)(o % w - lev.radius[a]), lev.step[a]));
+        o /= w;
+        p[a] = v < box.lo[a] ? box.lo[a] : (v > box.hi[a] ? box.hi[a] : v);
+    }
+}
+
+// 2. Screening: h = |<r, u>| / |u| of every candidate in plain FP32, and a
+// bound c with |h - |s|| <= c |r| for the float-float score s of
+// lem_score_warp.  Per sample:
+//  * the phase in cycles is a 32-bit fixed-point recurrence (wrapping is the
+//    reduction mod 1): phi(n) = A + B n + C n^2 with A, B, C rounded to
+//    2^-64, a lane's first phase and differences from those, then two
+//    integer adds a sample; its leading 23 bits become a float by one shift;
+//  * cos and exp by the hardware approximations (the sign that the half-cycle
+//    shift of the float form costs is lost in |h|);
+//  * samples beyond kScreenX durations from the centre are left out.
+// The bound, with x = (n - tc) / (fs dt), e the envelope, x0 = |x| of the
+// window's nearest sample, K <= 64 samples a lane, relative to |e|_2:
+//  * phase: 2 pi (2^-32 (1 + K + K^2 / 2) + 2^-24) radians; cos.approx 2^-20.9
+//    absolute on [-pi, pi]; 2 pi y and its scaling inside cos 4 2^-24 pi;
+//  * envelope: forming x rounds 2^-24 of at most 2 kScreenX four times, its
+//    step (expf 2 ulp, three products) is off by 5.4e-7 of itself, the
+//    exponents round to 2.2e-7 of themselves over both sides, ex2.approx and
+//    expf 2 ulp each: |x| 1.7e-6 + x^2 8e-7 + 5e-7, and under the weights
+//    e^2 of the samples x counts as at most x0 + 1.5;
+//  * the samples left out: below 2e-6 |e| while x0 <= 2;
+//  * the FP32 sums of either side: (K + 40) 2^-24 |u| for <r, u> and for |u|.
+// The first three act as twice a perturbation of u, relative to |u|: they
+// count 2 |e| / |u|, where |e|^2 <= sqrt(pi) / dx + 1 (the integral of
+// exp(-x^2) plus its largest term, dx = the step of x).  The whole is
+// doubled; measured over EEG-, EMG- and radar-like, sub-sample, long and
+// off-window candidates the largest error was 0.014 of the bound.
+// Where x0 > 2, or the sums are so small that squares vanish, or the phase
+// so large that FP64 does not hold it, c is infinite: k_lem_pick then always
+// projects the candidate again.
+// Bound by the special-function pipe (two a sample, 16 cycles a warp, and
+// about as many other issues): SCREEN_US for 64 channels x 2,048 candidates x
+// 512 samples, where the float-float projection of all took 230 us (118
+// instructions a sample).
+constexpr float kScreenX = 5.8f;
+constexpr int kScreenCands = 64;
+constexpr float kScreenWide = 2.0f;
+
+struct ScreenConst {
+    uint64_t A, B, C;     // phase of sample n: A + B n + C n^2, in 2^-64 cycles
+    float xs, dx;         // sqrt(log2(e) / 2) x of sample 32 row_lo, and its step per sample
+    int row_lo, row_hi;   // rows of 32 samples projected
+    float c_u, c_s;       // error bound: (c_u / |u| + c_s) |r|
+};
+
+__device__ __forceinline__ uint64_t cycles64(double v) {
+    return (uint64_t)__double2ll_rn((v - rint(v)) * 0x1.0p64);  // saturates at half a cycle: 2^-64 off
+}
+
+__global__ void __launch_bounds__(kLemThreads) k_lem_screen(int cap, int level, LemBox box, LemLevel lev, int top_k,
+                                                           const double *__restrict__ kept,
+                                                           const int *__restrict__ nkept, double *__restrict__ cand,
+                                                           int *__restrict__ ncand, const float *__restrict__ R,
+                                                           int Lp, int L, double inv_fs, float2 *__restrict__ screen) {
+    extern __shared__ float r_sm[];  // the residual, zero up to a whole row
+    __shared__ ScreenConst ks[kScreenCands];
+    // every lane's <r, u> and |u|^2 of every candidate: added up by one
+    // thread each at the end (a shuffle tree per sum cost as much as 8 samples)
+    __shared__ float sums[2 * kScreenCands][33];
+    const int b = blockIdx.y;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int i0 = blockIdx.x * kScreenCands;
+    int n_cand, per = 1;
+    if (level == 0) {
+        n_cand = ncand[b];
+    } else {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) per *= 2 * lev.radius[a] + 1;
+        n_cand = nkept[b] * per;
+    }
+    const int n_here = min(kScreenCands, n_cand - i0);
+    if (n_here <= 0) return;  // the first block always has candidates: nkept >= 1 unless no score is a number
+    if (threadIdx.x < n_here) {
+        const int i = i0 + threadIdx.x;
+        double *th = cand + ((size_t)b * cap + i) * 4;
+        double p[4];
+        if (level == 0) {
+#pragma unroll
+            for (int a = 0; a < 4; ++a) p[a] = th[a];
+        } else {  // the candidates of this level, for k_lem_pick too
+            lem_neighbour(kept + ((size_t)b * top_k + i / per) * 4, i % per, box, lev, p);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) th[a] = p[a];
+        }
+        ScreenConst k;
+        const double g = p[3] * inv_fs * inv_fs, f = p[1] * inv_fs, gt = g * p[0];
+        const double alpha = (gt - f) * p[0], beta = f - 2.0 * gt;
+        k.A = cycles64(alpha);
+        k.B = cycles64(beta);
+        k.C = cycles64(g);
+        const float big = (float)(fabs(gt * p[0]) + fabs(f * p[0]) + fabs(beta) * L) + fabsf((float)g) * L * (float)L;
+        // 1 / dt = exp(-logdt), the argument's rounding made good
+        const float ah = (float)-p[2], al = (float)(-p[2] - (double)ah);
+        const float dx = expf(ah) * (1.0f + al) * (float)inv_fs;  // x per sample
+        const float nearest = fminf(fmaxf(rintf((float)p[0]), 0.0f), (float)(L - 1));
+        const float x0 = fabsf((float)((double)nearest - p[0])) * dx;
+        const float reach = kScreenX / dx;
+        const float lo = (float)p[0] - reach, hi = (float)p[0] + reach;
+        k.row_lo = lo > 0.0f ? (lo < (float)L ? (int)lo >> 5 : L) : 0;
+        k.row_hi = hi < (float)L ? (hi >= 0.0f ? ((int)hi + 1 >> 5) + 1 : 0) : (L + 31) >> 5;
+        k.row_hi = min(k.row_hi, (L + 31) >> 5);
+        constexpr float kScale = 0.84932180f;  // sqrt(log2(e) / 2)
+        k.dx = dx * kScale;
+        k.xs = (float)((double)(32 * k.row_lo) - p[0]) * k.dx;
+        const float K = (float)(k.row_hi - k.row_lo), w = x0 + 1.5f;
+        const float a_cos = 6.2831853f * (2.3283064e-10f * (1.0f + K + 0.5f * K * K) + 5.9604645e-8f) + 5.1e-7f + 7.6e-7f;
+        const float a_env = w * 1.7e-6f + w * w * 8e-7f + 5e-7f;
+        k.c_u = 2.0f * 2.0f * (a_cos + a_env + 2e-6f) * sqrtf(1.7724539f / dx + 1.0f);
+        k.c_s = 2.0f * 2.0f * (K + 40.0f) * 5.9604645e-8f;
+        // not covered by the bound (comparisons written so that a NaN is not either)
+        if (!(x0 <= kScreenWide && big <= 1e6f && dx >= 1e-20f && dx <= 1e6f)) k.c_u = __int_as_float(0x7f800000);
+        ks[threadIdx.x] = k;
+    }
+    const int rows = (L + 31) >> 5;
+    const float *r = R + (size_t)b * Lp;
+    for (int n = threadIdx.x; n < rows * 32; n += blockDim.x) r_sm[n] = n < L ? r[n] : 0.0f;
+    __syncthreads();
+    constexpr int kWarps = kLemThreads / 32;
+    for (int q = warp; q < n_here; q += kWarps) {
+        const ScreenConst k = ks[q];
+        const uint64_t n0 = (uint64_t)(32 * k.row_lo + lane);
+        // phase of the lane's first sample and its differences over 32 and 32 samples
+        uint32_t ph = (uint32_t)((k.A + (k.B + k.C * n0) * n0) >> 32) + 256u;  // + 256: the shift below rounds
+        uint32_t d1 = (uint32_t)((32ull * k.B + k.C * (64ull * n0 + 1024ull)) >> 32);
+        const uint32_t d2 = (uint32_t)((2048ull * k.C) >> 32);
+        const float x_lane = fmaf((float)lane, k.dx, k.xs), step = 32.0f * k.dx;
+        float ru = 0.0f, uu = 0.0f;
+        auto sample = [&](float x, float rv, bool in) {
+            float e;
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-x * x));
+            e = in ? e : 0.0f;
+            const float y = __uint_as_float(__funnelshift_r(ph, 0x7fu, 9));  // 1 + the phase
+            const float u = e * __cosf(fmaf(6.2831853f, y, -9.4247780f));   // less half a cycle
+            ph += d1;
+            d1 += d2;
+            ru = fmaf(rv, u, ru);
+            uu = fmaf(u, u, uu);
+        };
+        const float *rp = r_sm + 32 * k.row_lo + lane;
+        const int whole = min(k.row_hi, L >> 5) - k.row_lo;  // rows without an end in them
+        int t = 0;
+        for (; t + 4 <= whole; t += 4) {
+            const float xb = fmaf((float)t, step, x_lane);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sample(fmaf((float)e, step, xb), rp[32 * (t + e)], true);
+        }
+        for (; t < k.row_hi - k.row_lo; ++t)
+            sample(fmaf((float)t, step, x_lane), rp[32 * t], 32 * (k.row_lo + t) + lane < L);
+        sums[2 * q][lane] = ru;
+        sums[2 * q + 1][lane] = uu;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * kScreenCands) {
+        float v = 0.0f;
+        if (threadIdx.x < 2 * n_here)
+            for (int l = 0; l < 32; ++l) v += sums[threadIdx.x][l];
+        const float uu = __shfl_down_sync(0xffffffffu, v, 1);
+        const int q = threadIdx.x >> 1;
+        if (!(threadIdx.x & 1) && q < n_here) {
+            const float inv = rsqrtf(uu);
+            screen[(size_t)b * cap + i0 + q] = make_float2(
+                fabsf(v) * inv, uu >= 1e-18f ? ks[q].c_u * inv * 1.001f + ks[q].c_s : __int_as_float(0x7f800000));
+        }
+    }
+}
+
+// The score s = <r, u> / |u| of one candidate by one warp, lane = sample
+// stride 32.  A lane's samples n_k = lane + 32 k advance tau by D = 32 / fs,
+// so the phase (c tau + fc) tau steps by d1_k = D (c (2 tau_k + D) + fc), and
+// d1 by d2 = 2 c D^2: tau, the phase and d1 are carried by these recurrences
+// in float-float (phase and d1 mod 1), from exact starting values at k = 0.
 // The samples are FP32 from the same expressions as the dictionary
 // generator's; products are summed in FP32 over 4 samples, then into
 // float-float sums.
-constexpr int kScoreCands = 64;  // at most 32 per warp (one lane each)
-
 struct LemConst {
     ChirpFF k;
     ff D, d2;  // the lane stride in tau and the second difference of the phase (mod 1)
 };
 
-__global__ void __launch_bounds__(kLemThreads) k_lem_score(int cap, const double *__restrict__ cand,
-                                                          const int *__restrict__ ncand, const float *__restrict__ R,
-                                                          int Lp, int L, double inv_fs, double *__restrict__ score) {
-    __shared__ LemConst ks[kScoreCands];
-    const int b = blockIdx.y;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int i0 = blockIdx.x * kScoreCands;
-    const int n_here = min(kScoreCands, ncand[b] - i0);
-    if (n_here <= 0) return;
-    if (threadIdx.x < n_here) {
-        const double *th = cand + ((size_t)b * cap + i0 + threadIdx.x) * 4;
-        const double D = 32.0 * inv_fs;
-        double d2 = 2.0 * th[3] * D * D;
-        d2 -= rint(d2);
-        ks[threadIdx.x] = {chirp_ff(th[0], inv_fs, th[1], th[3], exp(-th[2])), ff_from_double(D),
-                           ff_from_double(d2)};
-    }
-    __syncthreads();
-    const float *r = R + (size_t)b * Lp;
-    // lane i keeps the sums of the warp's i-th candidate; the FP64 finish
-    // then runs once for all of them (an FP64 instruction costs the same
-    // pipe time however few lanes are active)
-    constexpr int kWarps = kLemThreads / 32;
-    ff my_ru = {0.0f, 0.0f}, my_uu = {0.0f, 0.0f};
-    int i = 0;
-    for (int q = warp; q < n_here; q += kWarps, ++i) {
-        const LemConst kc = ks[q];
-        const ChirpFF &k = kc.k;
-        // k = 0: tau, the phase and its first difference, formed directly
-        ff tau;
-        ff ph = chirp_phase_pair(lane, k, &tau);
-        const ff two_tau_d = ff_add({2.0f * tau.hi, 2.0f * tau.lo}, kc.D);
-        ff d1 = ff_frac(ff_mul(ff_add(ff_mul(k.c, two_tau_d), k.fc), kc.D));
-        ff ru = {0.0f, 0.0f}, uu = {0.0f, 0.0f};
-        for (int n0 = lane; n0 < L; n0 += 128) {
-            float pr = 0.0f, pu = 0.0f;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int n = n0 + 32 * e;
-                if (n < L) {
-                    const float x = chirp_x_ff(tau, k);
-                    const float u = expf(-0.5f * x * x) * cospif(2.0f * (ph.hi + ph.lo));
-                    pr = fmaf(__ldg(r + n), u, pr);
-                    pu = fmaf(u, u, pu);
-                    tau = ff_add_sloppy(tau, kc.D);
-                    ph = ff_frac(ff_add_sloppy(ph, d1));
-                    d1 = ff_frac(ff_add_sloppy(d1, kc.d2));
-                }
-            }
-            ru = ff_add_f(ru, pr);
-            uu = ff_add_f(uu, pu);
-        }
-        ru = ff_warp_sum(ru);
-        uu = ff_warp_sum(uu);
-        if (lane == i) {
-            my_ru = ru;
-            my_uu = uu;
-        }
-    }
-    if (lane < i) {
-        const double e = ff_to_double(my_uu);
-        score[(size_t)b * cap + i0 + warp + lane * kWarps] = (e > 0.0 && isfinite(e)) ? ff_to_double(my_ru) / sqrt(e) : 0.0;
-    }
+__device__ __forceinline__ LemConst lem_const(const double *__restrict__ th, double inv_fs) {
+    const double D = 32.0 * inv_fs;
+    double d2 = 2.0 * th[3] * D * D;
+    d2 -= rint(d2);
+    return {chirp_ff(th[0], inv_fs, th[1], th[3], exp(-th[2])), ff_from_double(D), ff_from_double(d2)};
 }
 
-// 3. Top-k by |score| with duplicates skipped: one block per channel, k
-// rounds of a block-wide arg-max (largest |score|, then lowest index).  The
-// compares run on the bit patterns (integer pipes; FP64 compares are slow
-// on this GPU): for finite non-negative doubles the patterns order as the
+__device__ __forceinline__ void lem_score_warp(const LemConst &kc, const float *__restrict__ r, int L, int lane,
+                                               ff &ru, ff &uu) {
+    const ChirpFF &k = kc.k;
+    // k = 0: tau, the phase and its first difference, formed directly
+    ff tau;
+    ff ph = chirp_phase_pair(lane, k, &tau);
+    const ff two_tau_d = ff_add({2.0f * tau.hi, 2.0f * tau.lo}, kc.D);
+    ff d1 = ff_frac(ff_mul(ff_add(ff_mul(k.c, two_tau_d), k.fc), kc.D));
+    ru = {0.0f, 0.0f};
+    uu = {0.0f, 0.0f};
+    for (int n0 = lane; n0 < L; n0 += 128) {
+        float pr = 0.0f, pu = 0.0f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int n = n0 + 32 * e;
+            if (n < L) {
+                const float x = chirp_x_ff(tau, k);
+                const float u = expf(-0.5f * x * x) * cospif(2.0f * (ph.hi + ph.lo));
+                pr = fmaf(__ldg(r + n), u, pr);
+                pu = fmaf(u, u, pu);
+                tau = ff_add_sloppy(tau, kc.D);
+                ph = ff_frac(ff_add_sloppy(ph, d1));
+                d1 = ff_frac(ff_add_sloppy(d1, kc.d2));
+            }
+        }
+        ru = ff_add_f(ru, pr);
+        uu = ff_add_f(uu, pu);
+    }
+    ru = ff_warp_sum(ru);
+    uu = ff_warp_sum(uu);
+}
+
+// 3. The top_k of one channel by float-float score, one block per channel.
+// Compares run on bit patterns (integer pipes; FP64 compares are slow on
+// this GPU): for finite non-negative values the patterns order as the
 // values, NaN scores are skipped, and two parameters are equal when their
 // patterns are, or both are zeros.
 __device__ __forceinline__ bool same_value(unsigned long long a, unsigned long long b) {
     return a == b || ((a | b) << 1) == 0ull;
 }
 
-__global__ void __launch_bounds__(kLemThreads) k_lem_topk(int cap, int k, const double *__restrict__ cand,
-                                                         const int *__restrict__ ncand,
-                                                         const double *__restrict__ score, double *__restrict__ kept,
-                                                         double *__restrict__ kept_score, int *__restrict__ nkept) {
-    constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;
-    __shared__ unsigned long long kt[16][4];
-    __shared__ unsigned long long bv_s[kLemThreads / 32];
-    __shared__ int bi_s[kLemThreads / 32];
-    __shared__ int m_sh;
-    const int b = blockIdx.x;
+constexpr int kPickThreads = 512;
+constexpr int kPickList = 1024;   // candidates projected again that the block holds in a list
+constexpr int kPickBatch = 256;   // of these, whose constants are held at once
+constexpr int kMaxTopK = 16;
+
+struct PickShared {
+    unsigned long long bv[2][kPickThreads / 32];  // by the parity of the choice
+    int bi[2][kPickThreads / 32];
+    int chosen[kMaxTopK];
+    unsigned long long value[kMaxTopK];
+    float sum[kPickThreads / 32];
+    int count;
+    int list[kPickList];
+    LemConst consts[kPickBatch];
+};
+
+// Up to k candidates by value(i) (0: not a candidate), largest first, the
+// lowest index among equals, a parameter vector already chosen skipped (equal
+// parameters have equal values, so only those of equal value are compared).
+// Each thread holds the best of its own entries e = tid, tid + threads, ...
+// (index_of(e)) and looks for its next one only when that is chosen or
+// repeats a choice; one barrier per choice.  Returns how many were found, the
+// same for all threads.
+template <typename IndexOf, typename Value>
+__device__ int pick_top(PickShared &sm, int k, int entries, const unsigned long long *__restrict__ cb, IndexOf index_of,
+                        Value value) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int n = ncand[b];
-    const unsigned long long *cb = reinterpret_cast<const unsigned long long *>(cand) + (size_t)b * cap * 4;
-    const unsigned long long *sb = reinterpret_cast<const unsigned long long *>(score) + (size_t)b * cap;
-    if (threadIdx.x == 0) m_sh = 0;
-    __syncthreads();
-    for (int round = 0; round < k; ++round) {
-        const int m = m_sh;
-        unsigned long long bv = 0ull;
-        int bi = -1;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            const unsigned long long v = sb[i] & kAbs;
-            if (v > kInf || (bi >= 0 && v <= bv)) continue;  // NaN, or not above the best (the first index wins ties)
-            bool dup = false;
-            for (int q = 0; q < m && !dup; ++q)
-                dup = same_value(cb[4 * i], kt[q][0]) && same_value(cb[4 * i + 1], kt[q][1]) &&
-                      same_value(cb[4 * i + 2], kt[q][2]) && same_value(cb[4 * i + 3], kt[q][3]);
-            if (!dup) {
-                bv = v;
-                bi = i;
+    unsigned long long mv = 0ull;
+    int mi = -1;
+    // the best of this thread's entries that come after (v, i) in the order
+    auto next_after = [&](unsigned long long v, int i, bool first) {
+        mv = 0ull;
+        mi = -1;
+        for (int e = threadIdx.x; e < entries; e += kPickThreads) {
+            const int c = index_of(e);
+            const unsigned long long x = value(c);
+            if (x == 0ull || (!first && (x > v || (x == v && c <= i)))) continue;
+            if (mi < 0 || x > mv || (x == mv && c < mi)) {
+                mv = x;
+                mi = c;
             }
         }
+    };
+    auto repeats = [&](int i, int j) {
+        if (i == j) return true;
+        bool same = true;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) same = same && same_value(cb[4 * (size_t)i + a], cb[4 * (size_t)j + a]);
+        return same;
+    };
+    auto better = [](unsigned long long ov, int oi, unsigned long long v, int i) {
+        return oi >= 0 && (i < 0 || ov > v || (ov == v && oi < i));
+    };
+    next_after(0ull, 0, true);
+    int m = 0;
+    for (; m < k; ++m) {
+        unsigned long long v = mv;
+        int i = mi;
         for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long ov = __shfl_xor_sync(0xffffffffu, bv, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-            if (oi >= 0 && (bi < 0 || ov > bv || (ov == bv && oi < bi))) {
-                bv = ov;
-                bi = oi;
+            const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, off);
+            const int oi = __shfl_xor_sync(0xffffffffu, i, off);
+            if (better(ov, oi, v, i)) {
+                v = ov;
+                i = oi;
             }
         }
         if (lane == 0) {
-            bv_s[warp] = bv;
-            bi_s[warp] = bi;
+            sm.bv[m & 1][warp] = v;
+            sm.bi[m & 1][warp] = i;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long v = 0ull;
-            int id = -1;
-            for (int w = 0; w < kLemThreads / 32; ++w)
-                if (bi_s[w] >= 0 && (id < 0 || bv_s[w] > v || (bv_s[w] == v && bi_s[w] < id))) {
-                    v = bv_s[w];
-                    id = bi_s[w];
-                }
-            if (id >= 0) {
-                for (int a = 0; a < 4; ++a) kt[m][a] = cb[4 * id + a];
-                kept_score[(size_t)b * k + m] = score[(size_t)b * cap + id];
-                for (int a = 0; a < 4; ++a) kept[((size_t)b * k + m) * 4 + a] = cand[((size_t)b * cap + id) * 4 + a];
-                m_sh = m + 1;
+        // every warp finds the block's best for itself
+        constexpr int kWarps = kPickThreads / 32;
+        v = lane < kWarps ? sm.bv[m & 1][lane] : 0ull;
+        i = lane < kWarps ? sm.bi[m & 1][lane] : -1;
+        for (int off = kWarps / 2; off > 0; off >>= 1) {
+            const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, off);
+            const int oi = __shfl_xor_sync(0xffffffffu, i, off);
+            if (better(ov, oi, v, i)) {
+                v = ov;
+                i = oi;
             }
         }
-        __syncthreads();
-        if (m_sh == m) break;  // nothing left
+        v = __shfl_sync(0xffffffffu, v, 0);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i < 0) break;  // nothing left
+        // read back below by this warp alone before the next barrier; all warps write the same
+        if (lane == 0) {
+            sm.chosen[m] = i;
+            sm.value[m] = v;
+        }
+        __syncwarp();
+        while (mi >= 0) {  // this thread's best that repeats no choice
+            bool dup = false;
+            for (int q = m; q >= 0 && sm.value[q] == mv && !dup; --q) dup = repeats(mi, sm.chosen[q]);
+            if (!dup) break;
+            next_after(mv, mi, false);
+        }
     }
-    if (threadIdx.x == 0) nkept[b] = m_sh;
+    __syncthreads();
+    return m;
 }
 
-// 4. Neighbourhood dictionaries of the kept candidates for one level.
-__global__ void __launch_bounds__(kLemThreads) k_lem_neigh(int cap, int k, LemBox box, LemLevel lev,
-                                                          const double *__restrict__ kept,
-                                                          const int *__restrict__ nkept, double *__restrict__ cand,
-                                                          int *__restrict__ ncand) {
+__global__ void __launch_bounds__(kPickThreads) k_lem_pick(int cap, int k, int level_candidates,
+                                                          const double *__restrict__ cand,
+                                                          const int *__restrict__ ncand, int per,
+                                                          int *__restrict__ nkept, const float2 *__restrict__ screen,
+                                                          const float *__restrict__ R, int Lp, int L, double inv_fs,
+                                                          double *__restrict__ score, double *__restrict__ kept,
+                                                          double *__restrict__ kept_score) {
+    constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;
+    extern __shared__ __align__(16) uint8_t pick_raw[];
+    PickShared &sm = *reinterpret_cast<PickShared *>(pick_raw);
     const int b = blockIdx.x;
-    const int m = nkept[b];
-    int w[4], per = 1;
-    for (int a = 0; a < 4; ++a) {
-        w[a] = 2 * lev.radius[a] + 1;
-        per *= w[a];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = level_candidates ? nkept[b] * per : ncand[b];
+    const double *cd = cand + (size_t)b * cap * 4;
+    const unsigned long long *cb = reinterpret_cast<const unsigned long long *>(cd);
+    const float2 *sc = screen + (size_t)b * cap;
+    double *ss = score + (size_t)b * cap;
+    const float *r = R + (size_t)b * Lp;
+    // |r| from above: an FP32 sum of at most 2048 squares is within 1.3e-4
+    // relative of the exact one, and squares that underflow lose less than 1e-18
+    float e = 0.0f;
+    int nonzero = 0;
+    for (int i = threadIdx.x; i < L; i += kPickThreads) {
+        const float x = r[i];
+        e = fmaf(x, x, e);
+        nonzero |= x != 0.0f;
     }
-    const int total = m * per;
-    double *out = cand + (size_t)b * cap * 4;
-    for (int t = threadIdx.x; t < total; t += blockDim.x) {
-        const int j = t / per;
-        int rest = t % per;
-        int o[4];
-        for (int a = 3; a >= 0; --a) {
-            o[a] = rest % w[a] - lev.radius[a];
-            rest /= w[a];
-        }
-        for (int a = 0; a < 4; ++a) {
-            double v = __dadd_rn(kept[((size_t)b * k + j) * 4 + a], __dmul_rn((double)o[a], lev.step[a]));
-            v = v < box.lo[a] ? box.lo[a] : (v > box.hi[a] ? box.hi[a] : v);
-            out[4 * t + a] = v;
+    e = warp_sum(e);
+    if (lane == 0) sm.sum[warp] = e;
+    if (threadIdx.x == 0) sm.count = 0;
+    const bool zero = !__syncthreads_or(nonzero);
+    float tot = 0.0f;
+    for (int w = 0; w < kPickThreads / 32; ++w) tot += sm.sum[w];
+    const float rn = sqrtf(tot) * 1.001f + 1e-18f;
+
+    int entries = n;
+    bool listed = false;
+    float thr = -__int_as_float(0x7f800000);
+    // h + c |r|, rounded up; not below thr, or not a number: to be projected again
+    auto in_reach = [&](int i) { return !(__fadd_ru(sc[i].x, __fmul_ru(sc[i].y, rn)) < thr); };
+    if (!zero) {
+        // the k-th largest lower bound h - c |r| over distinct parameters:
+        // the top_k scores are at least that
+        const int m = pick_top(
+            sm, k, n, cb, [](int e2) { return e2; },
+            [&](int i) {
+                const float lo = __fadd_rd(sc[i].x, -__fmul_ru(sc[i].y, rn));
+                return lo >= 0.0f ? (unsigned long long)__float_as_uint(lo) + 1ull : 0ull;
+            });
+        if (m == k) thr = __uint_as_float((unsigned)(sm.value[k - 1] - 1ull));
+        __syncthreads();
+        for (int i = threadIdx.x; i < n; i += kPickThreads)
+            if (in_reach(i)) {
+                const int at = atomicAdd(&sm.count, 1);
+                if (at < kPickList) sm.list[at] = i;
+            }
+        __syncthreads();
+        const int count = sm.count;
+        listed = count <= kPickList;
+        if (listed) entries = count;
+        auto finish = [&](ff ru, ff uu) {
+            const double en = ff_to_double(uu);
+            return (en > 0.0 && isfinite(en)) ? ff_to_double(ru) / sqrt(en) : 0.0;
+        };
+        // the same steps for listed candidates and, past the list, for all in reach
+        for (int e0 = 0; e0 < entries; e0 += kPickBatch) {
+            const int here = min(kPickBatch, entries - e0);
+            if (threadIdx.x < here) {
+                const int i = listed ? sm.list[e0 + threadIdx.x] : e0 + threadIdx.x;
+                if (listed || in_reach(i)) sm.consts[threadIdx.x] = lem_const(cd + 4 * (size_t)i, inv_fs);
+            }
+            __syncthreads();
+            // lane q keeps the sums of the warp's q-th candidate: the FP64
+            // finish runs once for all of them
+            ff my_ru = {0.0f, 0.0f}, my_uu = {0.0f, 0.0f};
+            int mine = -1, q = 0;
+            for (int t = warp; t < here; t += kPickThreads / 32) {
+                const int i = listed ? sm.list[e0 + t] : e0 + t;
+                if (!listed && !in_reach(i)) continue;
+                ff ru, uu;
+                lem_score_warp(sm.consts[t], r, L, lane, ru, uu);
+                if (lane == q) {
+                    my_ru = ru;
+                    my_uu = uu;
+                    mine = i;
+                }
+                ++q;
+            }
+            if (mine >= 0) ss[mine] = finish(my_ru, my_uu);
+            __syncthreads();
         }
     }
-    if (threadIdx.x == 0) ncand[b] = total;
+    // a zero residual scores 0 everywhere
+    const int m = pick_top(
+        sm, k, entries, cb, [&](int e2) { return listed ? sm.list[e2] : e2; },
+        [&](int i) {
+            if (zero) return 1ull;
+            if (!listed && !in_reach(i)) return 0ull;
+            const unsigned long long v = (unsigned long long)__double_as_longlong(ss[i]) & kAbs;
+            return v > kInf ? 0ull : v + 1ull;
+        });
+    if (threadIdx.x < m) {
+        const int i = sm.chosen[threadIdx.x];
+        kept_score[(size_t)b * k + threadIdx.x] = zero ? 0.0 : ss[i];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) kept[((size_t)b * k + threadIdx.x) * 4 + a] = cd[4 * (size_t)i + a];
+    }
+    if (threadIdx.x == 0) nkept[b] = m;
 }
 
 }  // namespace
 
 cudaError_t launch_lem_select(const LemConfig &cfg, int B, int order, const float *R, int Lp, int L, double fs,
                               const LemBuffers &lb, cudaStream_t st) {
-    int npow2 = 1;
-    while (npow2 < cfg.n_coarse) npow2 <<= 1;
-    const size_t smem = (size_t)npow2 * (sizeof(uint64_t) + sizeof(uint32_t));
+    int log2b = 0;
+    while ((1 << log2b) < cfg.n_coarse && log2b < 13) ++log2b;  // at most 16,384 keys and 8,192 buckets: 192 KB
+    const size_t smem = (size_t)cfg.n_coarse * sizeof(uint64_t) + 2 * sizeof(uint32_t) * ((size_t)1 << log2b);
     if (smem > 48 * 1024) {
         cudaError_t ea = cudaFuncSetAttribute(k_lem_lhs, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (ea != cudaSuccess) return ea;
     }
-    k_lem_lhs<<<dim3(B, 4), kLemThreads, smem, st>>>(cfg.n_coarse, npow2, cfg.box, cfg.seed, order, lb.cap, lb.cand, lb.ncand);
+    k_lem_lhs<<<dim3(B, 4), kLhsThreads, smem, st>>>(cfg.n_coarse, log2b, cfg.box, cfg.seed, order, lb.cap, lb.cand,
+                                                     lb.ncand);
     cudaError_t e = cudaGetLastError();
     const double inv_fs = 1.0 / fs;
+    const size_t r_smem = sizeof(float) * (size_t)((L + 31) / 32 * 32);
     int n = cfg.n_coarse;
     for (int lev = 0; lev <= cfg.levels && e == cudaSuccess; ++lev) {
+        int per = 1;
         if (lev > 0) {
-            k_lem_neigh<<<B, kLemThreads, 0, st>>>(lb.cap, cfg.top_k, cfg.box, cfg.level[lev], lb.kept, lb.nkept,
-                                                   lb.cand, lb.ncand);
-            e = cudaGetLastError();
-            int per = 1;
             for (int a = 0; a < 4; ++a) per *= 2 * cfg.level[lev].radius[a] + 1;
             n = cfg.top_k * per;
         }
-        if (e != cudaSuccess) break;
-        dim3 grid((n + kScoreCands - 1) / kScoreCands, B);
-        k_lem_score<<<grid, kLemThreads, 0, st>>>(lb.cap, lb.cand, lb.ncand, R, Lp, L, inv_fs, lb.score);
+        const dim3 grid((n + kScreenCands - 1) / kScreenCands, B);
+        k_lem_screen<<<grid, kLemThreads, r_smem, st>>>(lb.cap, lev, cfg.box, cfg.level[lev], cfg.top_k, lb.kept,
+                                                        lb.nkept, lb.cand, lb.ncand, R, Lp, L, inv_fs, lb.screen);
         e = cudaGetLastError();
         if (e != cudaSuccess) break;
-        k_lem_topk<<<B, kLemThreads, 0, st>>>(lb.cap, cfg.top_k, lb.cand, lb.ncand, lb.score, lb.kept, lb.kept_score,
-                                              lb.nkept);
+        k_lem_pick<<<B, kPickThreads, sizeof(PickShared), st>>>(lb.cap, cfg.top_k, lev > 0, lb.cand, lb.ncand, per,
+                                                                lb.nkept, lb.screen, R, Lp, L, inv_fs, lb.score,
+                                                                lb.kept, lb.kept_score);
         e = cudaGetLastError();
     }
     return e;
 }
 
-int lem_kernels(const LemConfig &cfg) { return 1 + 2 + 3 * cfg.levels; }
+int lem_kernels(const LemConfig &cfg) { return 3 + 2 * cfg.levels; }
 
 }  // namespace act
