@@ -367,56 +367,73 @@ struct PickShared {
     LemConst consts[kPickBatch];
 };
 
+// The best (v, i) of the warp, by three reductions: largest v, then lowest i
+// (i >= 0 names a candidate); the same for all lanes.
+__device__ __forceinline__ void warp_best(unsigned long long &v, int &i) {
+    const uint32_t hi = (uint32_t)(v >> 32), lo = (uint32_t)v;
+    const uint32_t mh = __reduce_max_sync(0xffffffffu, i >= 0 ? hi : 0u);
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, i >= 0 && hi == mh ? lo : 0u);
+    const uint32_t mi = __reduce_min_sync(0xffffffffu, i >= 0 && hi == mh && lo == ml ? (uint32_t)i : 0xffffffffu);
+    v = ((unsigned long long)mh << 32) | ml;
+    i = (int)mi;  // -1: no candidate
+}
+
 // Up to k candidates by value(i) (0: not a candidate), largest first, the
 // lowest index among equals, a parameter vector already chosen skipped (equal
 // parameters have equal values, so only those of equal value are compared).
 // Each thread holds the best of its own entries e = tid, tid + threads, ...
 // (index_of(e)) and looks for its next one only when that is chosen or
-// repeats a choice; one barrier per choice.  Returns how many were found, the
-// same for all threads.
+// repeats a choice: the first kHeld of them stay in registers (reading them
+// again from L2 was most of the time).  One barrier per choice.  Returns how
+// many were found, the same for all threads.
 template <typename IndexOf, typename Value>
 __device__ int pick_top(PickShared &sm, int k, int entries, const unsigned long long *__restrict__ cb, IndexOf index_of,
                         Value value) {
+    constexpr int kHeld = 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long hv[kHeld];
+#pragma unroll
+    for (int h = 0; h < kHeld; ++h) {
+        const int e = threadIdx.x + h * kPickThreads;
+        hv[h] = e < entries ? value(index_of(e)) : 0ull;
+    }
     unsigned long long mv = 0ull;
     int mi = -1;
     // the best of this thread's entries that come after (v, i) in the order
     auto next_after = [&](unsigned long long v, int i, bool first) {
         mv = 0ull;
         mi = -1;
-        for (int e = threadIdx.x; e < entries; e += kPickThreads) {
-            const int c = index_of(e);
-            const unsigned long long x = value(c);
-            if (x == 0ull || (!first && (x > v || (x == v && c <= i)))) continue;
+        auto offer = [&](int c, unsigned long long x) {
+            if (x == 0ull || (!first && (x > v || (x == v && c <= i)))) return;
             if (mi < 0 || x > mv || (x == mv && c < mi)) {
                 mv = x;
                 mi = c;
             }
+        };
+#pragma unroll
+        for (int h = 0; h < kHeld; ++h)
+            if (hv[h]) offer(index_of(threadIdx.x + h * kPickThreads), hv[h]);
+        for (int e = threadIdx.x + kHeld * kPickThreads; e < entries; e += kPickThreads) {
+            const int c = index_of(e);
+            offer(c, value(c));
         }
     };
     auto repeats = [&](int i, int j) {
         if (i == j) return true;
-        bool same = true;
+        unsigned long long x[4], y[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) same = same && same_value(cb[4 * (size_t)i + a], cb[4 * (size_t)j + a]);
-        return same;
-    };
-    auto better = [](unsigned long long ov, int oi, unsigned long long v, int i) {
-        return oi >= 0 && (i < 0 || ov > v || (ov == v && oi < i));
+        for (int a = 0; a < 4; ++a) {
+            x[a] = cb[4 * (size_t)i + a];
+            y[a] = cb[4 * (size_t)j + a];
+        }
+        return same_value(x[0], y[0]) && same_value(x[1], y[1]) && same_value(x[2], y[2]) && same_value(x[3], y[3]);
     };
     next_after(0ull, 0, true);
     int m = 0;
     for (; m < k; ++m) {
         unsigned long long v = mv;
         int i = mi;
-        for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, i, off);
-            if (better(ov, oi, v, i)) {
-                v = ov;
-                i = oi;
-            }
-        }
+        warp_best(v, i);
         if (lane == 0) {
             sm.bv[m & 1][warp] = v;
             sm.bi[m & 1][warp] = i;
@@ -426,16 +443,7 @@ __device__ int pick_top(PickShared &sm, int k, int entries, const unsigned long 
         constexpr int kWarps = kPickThreads / 32;
         v = lane < kWarps ? sm.bv[m & 1][lane] : 0ull;
         i = lane < kWarps ? sm.bi[m & 1][lane] : -1;
-        for (int off = kWarps / 2; off > 0; off >>= 1) {
-            const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, i, off);
-            if (better(ov, oi, v, i)) {
-                v = ov;
-                i = oi;
-            }
-        }
-        v = __shfl_sync(0xffffffffu, v, 0);
-        i = __shfl_sync(0xffffffffu, i, 0);
+        warp_best(v, i);
         if (i < 0) break;  // nothing left
         // read back below by this warp alone before the next barrier; all warps write the same
         if (lane == 0) {
