@@ -418,6 +418,19 @@ int fused_ctas(const act_grid *g, int B, act_search_mode mode, bool profiling) {
     return want < most ? want : most;
 }
 
+// One FP32 search over the stored rows: several channels share passes over
+// them; one takes the GEMV form in use.
+cudaError_t launch_fp32_search(const act_grid *g, const WorkBuffers &w, int B, cudaStream_t st, bool pdl) {
+    if (B > 1)
+        return launch_gemv_multi_argmax(g->d32, g->K, g->Lp, w.R, B, w.keys, g->status, g->sm_count, st, g->wait_ns,
+                                        pdl);
+    if (g->gemv_stream)
+        return launch_gemv_stream_argmax(g->d32, g->K, g->Lp, w.R, B, nullptr, nullptr, w.keys, g->status, g->sm_count,
+                                         st, g->wait_ns, pdl);
+    return launch_gemv_argmax(g->d32, g->K, g->Lp, w.R, B, nullptr, nullptr, w.keys, g->status, g->gemv_grid, st,
+                              g->wait_ns, pdl);
+}
+
 // Records the whole decomposition (init + P orders) on stream st (being captured).
 act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_search_mode mode, GraphEntry &ge,
                             cudaStream_t st, bool profiling, bool allow_fused) {
@@ -470,12 +483,7 @@ act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_searc
             kernels += 4;
         } else {
             // programmatic dependents between kernel nodes only (not next to profiling events)
-            if (g->gemv_stream)
-                ACT_CK(launch_gemv_stream_argmax(g->d32, g->K, g->Lp, w.R, B, nullptr, nullptr, w.keys, g->status,
-                                                 g->sm_count, st, g->wait_ns, !profiling));
-            else
-                ACT_CK(launch_gemv_argmax(g->d32, g->K, g->Lp, w.R, B, nullptr, nullptr, w.keys, g->status,
-                                          g->gemv_grid, st, g->wait_ns, !profiling));
+            ACT_CK(launch_fp32_search(g, w, B, st, !profiling));
             if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
             kernels += 1;
         }
@@ -897,7 +905,7 @@ act_status act_project(act_grid *g, const float *signals, int32_t channels, floa
         ACT_CK(launch_shift_search(g->shift, g->w.R, g->Lp, g->L, channels, nullptr, scores, g->status, false, st,
                                    nullptr, nullptr, g->wait_ns));
     } else {
-        ACT_CK(launch_project(g->d32, g->K, g->Lp, g->w.R, channels, scores, g->status, g->gemv_grid, st,
+        ACT_CK(launch_project(g->d32, g->K, g->Lp, g->w.R, channels, scores, g->status, g->sm_count, st,
                               g->wait_ns));
     }
     return ACT_OK;
@@ -1022,11 +1030,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
                                                 g->w.fb_list, g->w.fb_count, g->stats, g->status, g->gemv_grid, st,
                                                 g->wait_ns);
                 } else {
-                    e = g->gemv_stream
-                            ? launch_gemv_stream_argmax(g->d32, g->K, g->Lp, g->w.R, channels, nullptr, nullptr,
-                                                        g->w.keys, g->status, g->sm_count, st, g->wait_ns)
-                            : launch_gemv_argmax(g->d32, g->K, g->Lp, g->w.R, channels, nullptr, nullptr, g->w.keys,
-                                                 g->status, g->gemv_grid, st, g->wait_ns);
+                    e = launch_fp32_search(g, g->w, channels, st, false);
                 }
             }
             if (e == cudaSuccess) e = cudaEventRecord(e1, st);

@@ -14,25 +14,24 @@ namespace act {
 // ---------------------------------------------------------------------------
 // Each warp owns rows gw, gw + nw, gw + 2 nw, ... (nw = warps in the grid)
 // and streams two rows at a time with 128-bit loads: lane l reads float4
-// l + 32 j of a row, j = 0..NV-1.  The NB residuals of a channel group are
-// brought into shared memory by the TMA bulk-copy engine and then held in
-// registers.  A warp-shuffle reduction gives every lane the row's score;
-// the warp keeps its best |score| (lowest row on ties, rows are visited in
-// increasing order), the block combines its warps and issues one 64-bit
-// atomicMax of the packed key per channel.
-// With WRITE_SCORES the raw scores are stored instead (projection only).
-template <int NV, int NB, bool WRITE_SCORES>
+// l + 32 j of a row, j = 0..NV-1.  The residual is brought into shared memory
+// by the TMA bulk-copy engine and then held in registers; several channels
+// (the queue of a tensor-core search's full searches) follow one another.  A
+// warp-shuffle reduction gives every lane the row's score; the warp keeps its
+// best |score| (lowest row on ties, rows are visited in increasing order),
+// the block combines its warps and issues one 64-bit atomicMax of the packed
+// key per channel.
+template <int NV>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__ D, int64_t K, int Lp,
                                                        const float *__restrict__ R, int B,
                                                        const int *__restrict__ chlist,
                                                        const int *__restrict__ count_dev,
-                                                       unsigned long long *__restrict__ keys,
-                                                       float *__restrict__ scores, int *status,
+                                                       unsigned long long *__restrict__ keys, int *status,
                                                        unsigned long long wait_ns) {
-    extern __shared__ __align__(128) float smem_r[];  // NB * Lp floats
+    extern __shared__ __align__(128) float smem_r[];  // Lp floats
     __shared__ __align__(8) uint64_t bar;
-    __shared__ float red_s[kGemvThreads / 32][NB];
-    __shared__ uint32_t red_i[kGemvThreads / 32][NB];
+    __shared__ float red_s[kGemvThreads / 32];
+    __shared__ uint32_t red_i[kGemvThreads / 32];
 
     // launched as a programmatic dependent of the kernel before it (the
     // residual update, or the queue that count_dev counts): every block waits
@@ -55,14 +54,11 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
     __syncthreads();
     uint32_t parity = 0;
 
-    for (int g0 = 0; g0 < count; g0 += NB) {
-        const int ng = min(NB, count - g0);
+    for (int g = 0; g < count; ++g) {
+        const int ch = chlist ? chlist[g] : g;
         if (threadIdx.x == 0) {
-            mbar_expect_tx(&bar, (uint32_t)(ng * Lp * 4));
-            for (int c = 0; c < ng; ++c) {
-                const int ch = chlist ? chlist[g0 + c] : g0 + c;
-                bulk_g2s(smem_r + c * Lp, R + (int64_t)ch * Lp, (uint32_t)(Lp * 4), &bar);
-            }
+            mbar_expect_tx(&bar, (uint32_t)(Lp * 4));
+            bulk_g2s(smem_r, R + (int64_t)ch * Lp, (uint32_t)(Lp * 4), &bar);
         }
         const int timed_out = mbar_wait(&bar, parity, wait_ns) ? 0 : 1;
         if (__syncthreads_or(timed_out)) {
@@ -74,22 +70,11 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
         }
         parity ^= 1u;
 
-        float4 rv[NB][NV];
+        float4 rv[NV];
 #pragma unroll
-        for (int c = 0; c < NB; ++c)
-#pragma unroll
-            for (int j = 0; j < NV; ++j)
-                rv[c][j] = c < ng ? reinterpret_cast<const float4 *>(smem_r + c * Lp)[lane + 32 * j]
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-
-        float best[NB];
-        uint32_t bidx[NB];
-#pragma unroll
-        for (int c = 0; c < NB; ++c) {
-            best[c] = -1.0f;
-            bidx[c] = 0u;
-        }
-
+        for (int j = 0; j < NV; ++j) rv[j] = reinterpret_cast<const float4 *>(smem_r)[lane + 32 * j];
+        float best = -1.0f;
+        uint32_t bidx = 0u;
         for (int64_t row = gw; row < K; row += 2 * nw) {
             const int64_t row2 = row + nw;
             const bool has2 = row2 < K;
@@ -105,127 +90,65 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
 #pragma unroll
                 for (int j = 0; j < NV; ++j) b[j] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            float sa[NB], sb[NB];
+            float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f;
 #pragma unroll
-            for (int c = 0; c < NB; ++c) {
-                float x0 = 0.f, x1 = 0.f, y0 = 0.f, y1 = 0.f;
-#pragma unroll
-                for (int j = 0; j < NV; ++j) {
-                    x0 = fmaf(a[j].x, rv[c][j].x, x0);
-                    x1 = fmaf(a[j].y, rv[c][j].y, x1);
-                    x0 = fmaf(a[j].z, rv[c][j].z, x0);
-                    x1 = fmaf(a[j].w, rv[c][j].w, x1);
-                    y0 = fmaf(b[j].x, rv[c][j].x, y0);
-                    y1 = fmaf(b[j].y, rv[c][j].y, y1);
-                    y0 = fmaf(b[j].z, rv[c][j].z, y0);
-                    y1 = fmaf(b[j].w, rv[c][j].w, y1);
-                }
-                sa[c] = x0 + x1;
-                sb[c] = y0 + y1;
+            for (int j = 0; j < NV; ++j) {
+                x0 = fmaf(a[j].x, rv[j].x, x0);
+                x1 = fmaf(a[j].y, rv[j].y, x1);
+                x0 = fmaf(a[j].z, rv[j].z, x0);
+                x1 = fmaf(a[j].w, rv[j].w, x1);
+                y0 = fmaf(b[j].x, rv[j].x, y0);
+                y1 = fmaf(b[j].y, rv[j].y, y1);
+                y0 = fmaf(b[j].z, rv[j].z, y0);
+                y1 = fmaf(b[j].w, rv[j].w, y1);
             }
+            float sa = x0 + x1, sb = y0 + y1;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-                for (int c = 0; c < NB; ++c) {
-                    sa[c] += __shfl_xor_sync(0xffffffffu, sa[c], off);
-                    sb[c] += __shfl_xor_sync(0xffffffffu, sb[c], off);
-                }
+                sa += __shfl_xor_sync(0xffffffffu, sa, off);
+                sb += __shfl_xor_sync(0xffffffffu, sb, off);
             }
-#pragma unroll
-            for (int c = 0; c < NB; ++c) {
-                if (c < ng) {
-                    if (WRITE_SCORES) {
-                        if (lane == 0) {
-                            const int ch = chlist ? chlist[g0 + c] : g0 + c;
-                            scores[(int64_t)ch * K + row] = sa[c];
-                            if (has2) scores[(int64_t)ch * K + row2] = sb[c];
-                        }
-                    } else {
-                        float x = fabsf(sa[c]);
-                        if (x > best[c]) {
-                            best[c] = x;
-                            bidx[c] = (uint32_t)row;
-                        }
-                        if (has2) {
-                            x = fabsf(sb[c]);
-                            if (x > best[c]) {
-                                best[c] = x;
-                                bidx[c] = (uint32_t)row2;
-                            }
-                        }
-                    }
+            float x = fabsf(sa);
+            if (x > best) {
+                best = x;
+                bidx = (uint32_t)row;
+            }
+            if (has2) {
+                x = fabsf(sb);
+                if (x > best) {
+                    best = x;
+                    bidx = (uint32_t)row2;
                 }
             }
         }
-
-        if (!WRITE_SCORES) {
-            if (lane == 0) {
-#pragma unroll
-                for (int c = 0; c < NB; ++c) {
-                    red_s[wid][c] = best[c];
-                    red_i[wid][c] = bidx[c];
-                }
-            }
-            __syncthreads();
-            if (threadIdx.x < ng) {
-                const int c = threadIdx.x;
-                float bs = -1.0f;
-                uint32_t bi = 0u;
-                for (int w = 0; w < kWarps; ++w) {
-                    const float s = red_s[w][c];
-                    const uint32_t i = red_i[w][c];
-                    if (s > bs || (s == bs && i < bi)) {
-                        bs = s;
-                        bi = i;
-                    }
-                }
-                if (bs >= 0.0f) {
-                    const int ch = chlist ? chlist[g0 + c] : g0 + c;
-                    atomicMax(keys + ch, pack_key(bs, bi));
-                }
-            }
+        if (lane == 0) {
+            red_s[wid] = best;
+            red_i[wid] = bidx;
         }
-        __syncthreads();  // shared residuals and reduction slots are reused by the next group
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            float bs = -1.0f;
+            uint32_t bi = 0u;
+            for (int w = 0; w < kWarps; ++w) {
+                const float s = red_s[w];
+                const uint32_t i = red_i[w];
+                if (s > bs || (s == bs && i < bi)) {
+                    bs = s;
+                    bi = i;
+                }
+            }
+            if (bs >= 0.0f) atomicMax(keys + ch, pack_key(bs, bi));
+        }
+        __syncthreads();  // the shared residual and reduction slots are reused by the next channel
     }
 }
 
-template <int NV, int NB, bool WS>
+template <int NV>
 static cudaError_t gemv_instance(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
-                                 const int *count_dev, unsigned long long *keys, float *scores, int *status,
-                                 int grid_ctas, unsigned long long wait_ns, cudaStream_t st, bool pdl) {
-    const size_t smem = (size_t)NB * Lp * sizeof(float);
-    return launch_kernel(k_gemv<NV, NB, WS>, dim3(grid_ctas), dim3(kGemvThreads), smem, st, pdl, D, K, Lp, R, B,
-                         chlist, count_dev, keys, scores, status, wait_ns);
-}
-
-template <bool WS>
-static cudaError_t gemv_dispatch(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
-                                 const int *count_dev, unsigned long long *keys, float *scores, int *status,
-                                 int grid_ctas, unsigned long long wait_ns, cudaStream_t st, bool pdl = false) {
-    const int nv = Lp / 128;
-    // Several channels per pass over D only when the count is known on the host.
-    const bool multi = (count_dev == nullptr) && B >= 4 && nv <= 4;
-#define ACT_GEMV_CASE(NVV)                                                                                 \
-    case NVV:                                                                                              \
-        return multi ? gemv_instance<NVV, 4, WS>(D, K, Lp, R, B, chlist, count_dev, keys, scores, status, \
-                                                 grid_ctas, wait_ns, st, pdl)                              \
-                     : gemv_instance<NVV, 1, WS>(D, K, Lp, R, B, chlist, count_dev, keys, scores, status, \
-                                                 grid_ctas, wait_ns, st, pdl);
-    switch (nv) {
-        ACT_GEMV_CASE(1)
-        ACT_GEMV_CASE(2)
-        ACT_GEMV_CASE(3)
-        ACT_GEMV_CASE(4)
-        case 8:
-            return gemv_instance<8, 1, WS>(D, K, Lp, R, B, chlist, count_dev, keys, scores, status, grid_ctas,
-                                           wait_ns, st, pdl);
-        case 16:
-            return gemv_instance<16, 1, WS>(D, K, Lp, R, B, chlist, count_dev, keys, scores, status, grid_ctas,
-                                            wait_ns, st, pdl);
-        default:
-            return cudaErrorInvalidValue;
-    }
-#undef ACT_GEMV_CASE
+                                 const int *count_dev, unsigned long long *keys, int *status, int grid_ctas,
+                                 unsigned long long wait_ns, cudaStream_t st, bool pdl) {
+    return launch_kernel(k_gemv<NV>, dim3(grid_ctas), dim3(kGemvThreads), (size_t)Lp * sizeof(float), st, pdl, D, K,
+                         Lp, R, B, chlist, count_dev, keys, status, wait_ns);
 }
 
 int gemv_ctas(int sm_count, int Lp) { return sm_count * gemv_max_ctas_per_sm(Lp); }
@@ -236,12 +159,12 @@ int gemv_max_ctas_per_sm(int Lp) {
     cudaError_t e = cudaErrorInvalidValue;
     const size_t smem = (size_t)Lp * sizeof(float);
     switch (nv) {
-        case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<1, 1, false>, kGemvThreads, smem); break;
-        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<2, 1, false>, kGemvThreads, smem); break;
-        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<3, 1, false>, kGemvThreads, smem); break;
-        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<4, 1, false>, kGemvThreads, smem); break;
-        case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<8, 1, false>, kGemvThreads, smem); break;
-        case 16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<16, 1, false>, kGemvThreads, smem); break;
+        case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<1>, kGemvThreads, smem); break;
+        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<2>, kGemvThreads, smem); break;
+        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<3>, kGemvThreads, smem); break;
+        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<4>, kGemvThreads, smem); break;
+        case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<8>, kGemvThreads, smem); break;
+        case 16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<16>, kGemvThreads, smem); break;
         default: break;
     }
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -252,13 +175,20 @@ int gemv_max_ctas_per_sm(int Lp) {
 cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
                                const int *count_dev, unsigned long long *keys, int *status, int grid_ctas,
                                cudaStream_t st, unsigned long long wait_ns, bool pdl) {
-    return gemv_dispatch<false>(D, K, Lp, R, B, chlist, count_dev, keys, nullptr, status, grid_ctas, wait_ns, st,
-                                pdl);
-}
-
-cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, int B, float *scores, int *status,
-                           int grid_ctas, cudaStream_t st, unsigned long long wait_ns) {
-    return gemv_dispatch<true>(D, K, Lp, R, B, nullptr, nullptr, nullptr, scores, status, grid_ctas, wait_ns, st);
+#define ACT_GEMV_CASE(NVV)                                                                                        \
+    case NVV:                                                                                                     \
+        return gemv_instance<NVV>(D, K, Lp, R, B, chlist, count_dev, keys, status, grid_ctas, wait_ns, st, pdl);
+    switch (Lp / 128) {
+        ACT_GEMV_CASE(1)
+        ACT_GEMV_CASE(2)
+        ACT_GEMV_CASE(3)
+        ACT_GEMV_CASE(4)
+        ACT_GEMV_CASE(8)
+        ACT_GEMV_CASE(16)
+        default:
+            return cudaErrorInvalidValue;
+    }
+#undef ACT_GEMV_CASE
 }
 
 }  // namespace act

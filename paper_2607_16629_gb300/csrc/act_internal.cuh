@@ -129,8 +129,14 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
                                const int *chlist, const int *count_dev, unsigned long long *keys,
                                int *status, int grid_ctas, cudaStream_t st,
                                unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
+// Several channels: up to 16 per pass over the dictionary (act_gemv_multi.cu);
+// the same scores and keys.
+cudaError_t launch_gemv_multi_argmax(const float *D, int64_t K, int Lp, const float *R, int B,
+                                     unsigned long long *keys, int *status, int sm_count, cudaStream_t st,
+                                     unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
+// Every score, scores[b * K + row], any number of channels.
 cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, int B, float *scores,
-                           int *status, int grid_ctas, cudaStream_t st, unsigned long long wait_ns = kWaitLimitNs);
+                           int *status, int sm_count, cudaStream_t st, unsigned long long wait_ns = kWaitLimitNs);
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
                           unsigned long long *keys, const GridAxes &ax, int k, int P, act_atom *atoms,
                           float *coefs, double *energy, int *fb_count, cudaStream_t st, bool pdl = false);
