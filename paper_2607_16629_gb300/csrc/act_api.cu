@@ -657,6 +657,7 @@ act_status act_grid_create(const act_grid_desc *desc, int32_t device, act_grid *
         return e == cudaErrorMemoryAllocation ? ACT_ERR_OOM : ACT_ERR_CUDA;
     }
     g->gemv_grid = gemv_ctas(g->sm_count, g->Lp);
+    g->gemv_stream = g->K * (int64_t)g->Lp * (int64_t)sizeof(float) >= kStreamMinDictBytes;
     act_lem_params lp;
     memset(&lp, 0, sizeof(lp));
     lp.top_k = 4;
