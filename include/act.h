@@ -79,8 +79,10 @@ typedef struct {
  *   ACT_DICT_FP32: D as FP32 [K][Lp] (Lp = L rounded up to 128), searched by
  *                  the FP32 GEMV / multi-channel GEMV.
  *   ACT_DICT_BF16: D as FP32 [K][Lp] plus BF16 [K][Lb] (Lb = L rounded up to
- *                  64) for the tensor-core search; FP32 rows are used to
- *                  rescore candidates and for the update.
+ *                  64) for the tensor-core search (and, where that search
+ *                  uses them and they fit, templates as for
+ *                  ACT_DICT_RECOMPUTE); FP32 rows are used to rescore
+ *                  candidates and for the update.
  *   ACT_DICT_AUTO: ACT_DICT_FP32 when the FP32 rows fit the grid's memory
  *                  budget (act_set_memory_budget; by default 90% of the
  *                  device memory free when the build starts), otherwise
@@ -112,7 +114,11 @@ typedef enum {
  *   ACT_SEARCH_FP32: FP32 GEMV with the argmax fused (CUDA cores).
  *   ACT_SEARCH_BF16: BF16 tcgen05 GEMM over all atoms (tensor cores, FP32
  *                    accumulation) reduced to the largest |score| per
- *                    tile and per 32-atom block; the blocks that an error
+ *                    tile and per 32-atom block (on grids of whole-sample
+ *                    time centres and 128 MiB of BF16 rows or more, where the
+ *                    templates of ACT_DICT_RECOMPUTE take little memory
+ *                    beside them, every atom is scored through its BF16
+ *                    template instead of its row); the blocks that an error
  *                    bound cannot exclude are rescored in FP32 (a channel
  *                    with more than 512 of them takes the FP32 search), so
  *                    the selection equals the FP32 search's bit for bit

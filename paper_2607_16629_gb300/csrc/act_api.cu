@@ -156,6 +156,8 @@ struct act_grid {
     Bf16Search *bf16 = nullptr;
     ShiftPlan shift;       // template dictionary (ACT_DICT_RECOMPUTE)
     ShiftTc *shift_tc = nullptr;  // its tensor-core search (ACT_SEARCH_SHIFT_BF16)
+    ShiftPlan screen;             // templates of a BF16 build's atoms, for its screening GEMM
+    ShiftTc *screen_tc = nullptr; // null: the dense GEMM over the BF16 rows screens
     int gemv_grid = 0;
     bool gemv_stream = false;  // FP32 search by the bulk-copy streaming GEMV (one CTA per SM)
     int refine_steps = 0;  // BFGS iterations per order (0: grid-only search)
@@ -218,6 +220,17 @@ void free_work(WorkBuffers &w) {
     shift_tc_scratch_free(w.stc);
 }
 
+void free_templates(ShiftPlan &sp) {
+    free_dev(sp.tpl);
+    free_dev(sp.scale);
+    free_dev(sp.tpl16);
+    free_dev(sp.scaleT);
+    free_dev(sp.eps_bits);
+    free_dev(sp.span);
+    free_dev(sp.blk_order);
+    sp = ShiftPlan();
+}
+
 void free_dictionary(act_grid *g) {
     if (g->bf16) bf16_search_free(g->bf16);
     g->bf16 = nullptr;
@@ -225,14 +238,10 @@ void free_dictionary(act_grid *g) {
     free_dev(g->d16);
     if (g->shift_tc) shift_tc_free(g->shift_tc);
     g->shift_tc = nullptr;
-    free_dev(g->shift.tpl);
-    free_dev(g->shift.scale);
-    free_dev(g->shift.tpl16);
-    free_dev(g->shift.scaleT);
-    free_dev(g->shift.eps_bits);
-    free_dev(g->shift.span);
-    free_dev(g->shift.blk_order);
-    g->shift = ShiftPlan();
+    free_templates(g->shift);
+    if (g->screen_tc) shift_tc_free(g->screen_tc);
+    g->screen_tc = nullptr;
+    free_templates(g->screen);
     g->built = -1;
     // the tensor-core search scratch is sized by the dictionary's shape
     bf16_scratch_free(g->w.b16);
@@ -310,7 +319,7 @@ act_status scratch_status(cudaError_t e, const char *what) {
 bool work_fits(const act_grid *g, const WorkBuffers &w, int B, int P, act_search_mode mode) {
     if (B > w.cap_B || P > w.cap_P) return false;
     if (mode == ACT_SEARCH_LEM && (w.lem.cap < lem_capacity(g->lem) || w.lem_B < B || !w.lem.cand)) return false;
-    if (mode == ACT_SEARCH_BF16 && w.b16.B_cap < B) return false;
+    if (mode == ACT_SEARCH_BF16 && (g->screen_tc ? w.stc.B_cap : w.b16.B_cap) < B) return false;
     if (mode == ACT_SEARCH_SHIFT_BF16 && w.stc.B_cap < B) return false;
     return true;
 }
@@ -337,7 +346,11 @@ act_status grow_work(const act_grid *g, WorkBuffers &w, int B, int P, act_search
             return s;
         }
     }
-    if (mode == ACT_SEARCH_BF16 && w.b16.B_cap < B) {
+    if (mode == ACT_SEARCH_BF16 && g->screen_tc && w.stc.B_cap < B) {
+        if ((s = scratch_status(shift_tc_reserve(g->screen_tc, g->screen, B, w.stc), "shift_tc_reserve")) != ACT_OK)
+            return s;
+    }
+    if (mode == ACT_SEARCH_BF16 && !g->screen_tc && w.b16.B_cap < B) {
         if ((s = scratch_status(bf16_scratch_reserve(g->bf16, B, w.b16), "bf16_scratch_reserve")) != ACT_OK)
             return s;
     }
@@ -435,7 +448,7 @@ cudaError_t launch_fp32_search(const act_grid *g, const WorkBuffers &w, int B, c
 act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_search_mode mode, GraphEntry &ge,
                             cudaStream_t st, bool profiling, bool allow_fused) {
     const bool bf16 = mode == ACT_SEARCH_BF16;
-    __nv_bfloat16 *R16 = bf16 ? w.R16 : nullptr;
+    __nv_bfloat16 *R16 = bf16 && !g->screen_tc ? w.R16 : nullptr;  // the dense GEMM's operand
     int kernels = 0;
     const int fctas = allow_fused ? fused_ctas(g, B, mode, profiling) : 0;
     if (fctas > 0) {  // the single-launch form (it also initialises the residuals)
@@ -474,6 +487,14 @@ act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_searc
             if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
             ACT_CK(launch_shift_tc_resolve(g->shift_tc, w.stc, g->shift, w.R, g->Lp, g->L, B, w.keys, w.fb_list,
                                            w.fb_count, g->stats, g->status, st, !profiling, g->wait_ns));
+            kernels += 5;
+        } else if (bf16 && g->screen_tc) {
+            ACT_CK(launch_shift_tc_gemm(g->screen_tc, w.stc, g->screen, w.R, g->Lp, g->L, B, g->stats, g->status, st,
+                                        !profiling, g->wait_ns, g->cta_pairs));
+            if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
+            ACT_CK(launch_shift_tc_resolve_rows(g->screen_tc, w.stc, g->screen, g->d32, g->K, w.R, g->Lp, g->L, B,
+                                                w.keys, w.fb_list, w.fb_count, g->stats, g->status, g->gemv_grid, st,
+                                                !profiling, g->wait_ns));
             kernels += 5;
         } else if (bf16) {
             ACT_CK(launch_bf16_gemm(g->bf16, w.b16, B, w.R16, g->status, st, g->wait_ns));
@@ -684,13 +705,11 @@ act_status act_grid_size(const act_grid *g, int64_t *n_atoms, int32_t *row_strid
     return ACT_OK;
 }
 
-// Template dictionary: per (fc, logDt, c) the samples the window can see,
-// and one FP32 scale per atom.
-static act_status build_templates(act_grid *g, cudaStream_t st) {
-    ShiftPlan sp;
-    if (shift_plan(sp, g->ax) != cudaSuccess) return ACT_ERR_UNSUPPORTED;
-    sp.Lp = g->Lp;
-    if (shift_default_config(sp, g->sm_count) != cudaSuccess) return ACT_ERR_UNSUPPORTED;
+// Allocates and builds the templates of g's atoms into sp (laid out by
+// shift_plan): per (fc, logDt, c) the samples the window can see, one FP32
+// scale per atom, and the tensor-core view where it exists.  On failure
+// nothing is kept.
+static cudaError_t make_templates(const act_grid *g, ShiftPlan &sp, unsigned long long *degenerate, cudaStream_t st) {
     const size_t bt = sizeof(float) * (size_t)sp.TB * sp.Sa * sp.rows * 32;
     const size_t bs = sizeof(float) * (size_t)sp.TB * sp.NtcP * 32;
     cudaError_t e = dev_alloc((void **)&sp.tpl, bt);
@@ -717,21 +736,27 @@ static act_status build_templates(act_grid *g, cudaStream_t st) {
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.scaleT, 0, bst, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.eps_bits, 0, sizeof(unsigned int), st);
     }
+    if (e == cudaSuccess) e = launch_shift_build(sp, g->ax, degenerate, g->sm_count, st);
     if (e != cudaSuccess) {
         cudaGetLastError();
-        free_dev(sp.tpl);
-        free_dev(sp.scale);
-        free_dev(sp.tpl16);
-        free_dev(sp.scaleT);
-        free_dev(sp.eps_bits);
-        free_dev(sp.span);
-        free_dev(sp.blk_order);
+        free_templates(sp);
+    }
+    return e;
+}
+
+// Template dictionary (ACT_DICT_RECOMPUTE).
+static act_status build_templates(act_grid *g, cudaStream_t st) {
+    ShiftPlan sp;
+    if (shift_plan(sp, g->ax) != cudaSuccess) return ACT_ERR_UNSUPPORTED;
+    sp.Lp = g->Lp;
+    if (shift_default_config(sp, g->sm_count) != cudaSuccess) return ACT_ERR_UNSUPPORTED;
+    ACT_CK(cudaMemsetAsync(g->degenerate, 0, sizeof(unsigned long long), st));
+    const cudaError_t e = make_templates(g, sp, g->degenerate, st);
+    if (e != cudaSuccess) {
         note_error("template dictionary", e);
-        return ACT_ERR_OOM;
+        return e == cudaErrorMemoryAllocation ? ACT_ERR_OOM : ACT_ERR_CUDA;
     }
     g->shift = sp;
-    ACT_CK(cudaMemsetAsync(g->degenerate, 0, sizeof(unsigned long long), st));
-    ACT_CK(launch_shift_build(g->shift, g->ax, g->degenerate, g->sm_count, st));
     g->built = ACT_DICT_RECOMPUTE;
     if (sp.tpl16 && shift_tc_prepare(&g->shift_tc, g->shift, g->sm_count) != cudaSuccess) {
         cudaGetLastError();
@@ -748,6 +773,26 @@ static uint64_t template_bytes(const act_grid *g) {
     uint64_t b = sizeof(float) * ((uint64_t)sp.TB * sp.Sa * sp.rows * 32 + (uint64_t)sp.TB * sp.NtcP * 32);
     if (sp.Kt > 0) b += sizeof(__nv_bfloat16) * (uint64_t)sp.T_pad * sp.Kt + sizeof(float) * (uint64_t)sp.NtcP * sp.T_pad;
     return b;
+}
+
+// The screening templates of a BF16 build (kScreenMinRowBytes).  Without
+// them, for want of memory too, the dense GEMM over the BF16 rows screens.
+static void build_screen(act_grid *g, cudaStream_t st) {
+    const int64_t row_bytes = (int64_t)sizeof(__nv_bfloat16) * g->K * g->Lb;
+    const uint64_t bt = template_bytes(g);
+    if (row_bytes < kScreenMinRowBytes || bt == 0 ||
+        bt > ((uint64_t)row_bytes + sizeof(float) * (uint64_t)g->K * (uint64_t)g->Lp) / 4)
+        return;
+    ShiftPlan sp;
+    if (shift_plan(sp, g->ax) != cudaSuccess || sp.Kt == 0) return;
+    sp.Lp = g->Lp;
+    if (make_templates(g, sp, nullptr, st) != cudaSuccess) return;
+    g->screen = sp;
+    if (shift_tc_prepare(&g->screen_tc, g->screen, g->sm_count) != cudaSuccess) {
+        cudaGetLastError();
+        g->screen_tc = nullptr;
+        free_templates(g->screen);
+    }
 }
 
 // ACT_DICT_AUTO: the FP32 rows when they fit the memory budget, else the
@@ -826,6 +871,7 @@ act_status act_dictionary_build(act_grid *g, act_dict_mode mode, void *cuda_stre
             free_dictionary(g);
             return pe == cudaErrorNotSupported ? ACT_ERR_UNSUPPORTED : ACT_ERR_CUDA;
         }
+        build_screen(g, st);
     }
     g->built = mode;
     return ACT_OK;
@@ -1022,7 +1068,16 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {  // pass 0 warms up
             e = cudaEventRecord(e0, st);
             for (int r = 0; r < reps && e == cudaSuccess; ++r) {
-                if (use_bf16) {
+                if (use_bf16 && g->screen_tc) {
+                    e = cudaMemsetAsync(g->w.fb_count, 0, 2 * sizeof(int), st);
+                    if (e == cudaSuccess)
+                        e = launch_shift_tc_gemm(g->screen_tc, g->w.stc, g->screen, g->w.R, g->Lp, g->L, channels,
+                                                 g->stats, g->status, st, false, g->wait_ns, g->cta_pairs);
+                    if (e == cudaSuccess)
+                        e = launch_shift_tc_resolve_rows(g->screen_tc, g->w.stc, g->screen, g->d32, g->K, g->w.R,
+                                                         g->Lp, g->L, channels, g->w.keys, g->w.fb_list, g->w.fb_count,
+                                                         g->stats, g->status, g->gemv_grid, st, false, g->wait_ns);
+                } else if (use_bf16) {
                     e = cudaMemsetAsync(g->w.fb_count, 0, 2 * sizeof(int), st);
                     if (e == cudaSuccess)
                         e = launch_bf16_gemm(g->bf16, g->w.b16, channels, g->w.R16, g->status, st, g->wait_ns);
@@ -1049,7 +1104,9 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
     int best_grid = g->gemv_grid;
     bool best_stream = false;
     g->gemv_stream = false;
-    const int max_per_sm = gemv_max_ctas_per_sm(g->Lp);
+    // (several channels have one form; its time, the one-channel forms as they are by load streaming)
+    if (channels > 1) err = time_search(false, &best32);
+    const int max_per_sm = channels > 1 ? 0 : gemv_max_ctas_per_sm(g->Lp);
     for (int per_sm = 1; per_sm <= max_per_sm && err == cudaSuccess; ++per_sm) {
         g->gemv_grid = g->sm_count * per_sm;
         double ms = 0.0;
@@ -1060,7 +1117,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         }
     }
     g->gemv_grid = best_grid;
-    if (err == cudaSuccess) {
+    if (err == cudaSuccess && channels == 1) {
         g->gemv_stream = true;
         double ms = 0.0;
         err = time_search(false, &ms);
@@ -1070,9 +1127,11 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         }
     }
     g->gemv_stream = best_stream;
-    // tensor-core search: tile width x pipeline depth
+    // tensor-core search: tile width x pipeline depth of the dense GEMM, or,
+    // where the templates screen, that search as it is
     double best16 = 1e30;
-    if (bf16 && err == cudaSuccess) {
+    if (bf16 && g->screen_tc && err == cudaSuccess) err = time_search(true, &best16);
+    if (bf16 && !g->screen_tc && err == cudaSuccess) {
         int best_bn = 256, best_st = 0;
         const int widths[2] = {128, 256};
         for (int wi = 0; wi < 2 && err == cudaSuccess; ++wi) {

@@ -363,7 +363,11 @@ __global__ void __launch_bounds__(256) k_select(int64_t ntiles, int bpt, const f
 __global__ void __launch_bounds__(256) k_rescan(const float *__restrict__ D32, int64_t K, int Lp, int tile_atoms,
                                                 const float *__restrict__ R, const int *__restrict__ pairs,
                                                 const int *__restrict__ counters,
-                                                unsigned long long *__restrict__ keys) {
+                                                unsigned long long *__restrict__ keys, int T, int n_blocks) {
+    // (a programmatic dependent of the kernel that flagged the items, where
+    // the template GEMM screens)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ float red_s[8];
     __shared__ uint32_t red_i[8];
     const int n_items = counters[1];
@@ -372,18 +376,23 @@ __global__ void __launch_bounds__(256) k_rescan(const float *__restrict__ D32, i
     const int rows_per_warp = tile_atoms / 8;
     for (int w = blockIdx.x; w < n_items; w += gridDim.x) {
         const int b = pairs[2 * w];
-        const int64_t tile = pairs[2 * w + 1];
+        const int item = pairs[2 * w + 1];
+        // T > 0: item = time centre * n_blocks + 32-template block, its atoms
+        // the rows from (time centre) T + 32 block on, up to that centre's T
+        const int64_t base = T > 0 ? (int64_t)(item / n_blocks) * T + (int64_t)(item % n_blocks) * 32
+                                   : (int64_t)item * tile_atoms;
+        const int64_t row_end = T > 0 ? (int64_t)(item / n_blocks + 1) * T : K;
         const float4 *res = reinterpret_cast<const float4 *>(R + (size_t)b * Lp);
         float best = -1.0f;
         uint32_t bidx = 0u;
-        const int64_t row0 = tile * tile_atoms + warp * rows_per_warp;
-        // four rows in flight per step; rows past K (last tile) are skipped
+        const int64_t row0 = base + warp * rows_per_warp;
+        // four rows in flight per step; rows past the end are skipped
         for (int i = 0; i < rows_per_warp; i += 4) {
             float sc[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int64_t row = row0 + i + u;
-                sc[u] = row < K ? fabsf(row_score(reinterpret_cast<const float4 *>(D32 + (size_t)row * Lp), res, nv,
+                sc[u] = row < row_end ? fabsf(row_score(reinterpret_cast<const float4 *>(D32 + (size_t)row * Lp), res, nv,
                                                   lane))
                                 : -1.0f;
             }
@@ -555,11 +564,18 @@ cudaError_t launch_bf16_resolve(const Bf16Search *s, const Bf16Scratch &x, int B
                                 fb_count, x.pairs, stats);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_rescan<<<2 * s->sm_count, 256, 0, st>>>(D32, s->K, Lp, 32, R, x.pairs, fb_count, keys);
+    k_rescan<<<2 * s->sm_count, 256, 0, st>>>(D32, s->K, Lp, 32, R, x.pairs, fb_count, keys, 0, 0);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // FP32 full search for the channels with too many flagged blocks
     return launch_gemv_argmax(D32, s->K, Lp, R, B, fb_list, fb_count, keys, status, gemv_grid, st, wait_ns);
+}
+
+cudaError_t launch_rows_rescan(const float *D32, int64_t K, int Lp, const float *R, const int *items,
+                               const int *counters, unsigned long long *keys, int T, int n_blocks, int sm_count,
+                               cudaStream_t st) {
+    return launch_kernel(k_rescan, dim3(2 * sm_count), dim3(256), 0, st, true, D32, K, Lp, 32, R, items, counters,
+                         keys, T, n_blocks);
 }
 
 }  // namespace act

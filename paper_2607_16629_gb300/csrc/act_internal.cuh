@@ -323,6 +323,29 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
                                     int Lp, int L, int B, unsigned long long *keys, int *fb_list, int *counters,
                                     long long *stats, int *status, cudaStream_t st, bool pdl = false,
                                     unsigned long long wait_ns = kWaitLimitNs);
+// The same selection for a stored dictionary D32 whose atoms the templates
+// of sp are (whole-sample time centres, a BF16 build): the flagged items are
+// scored from D32's rows with the FP32 GEMV's arithmetic, a channel with more
+// than 512 of them is queued for that GEMV, so the selection equals the FP32
+// search's over D32 bit for bit.
+cudaError_t launch_shift_tc_resolve_rows(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp,
+                                         const float *D32, int64_t K, const float *R, int Lp, int L, int B,
+                                         unsigned long long *keys, int *fb_list, int *counters, long long *stats,
+                                         int *status, int gemv_grid, cudaStream_t st, bool pdl = false,
+                                         unsigned long long wait_ns = kWaitLimitNs);
+// FP32 scores of the flagged (time centre, 32-template block) items' rows,
+// folded into keys; a programmatic dependent of the flagging.
+cudaError_t launch_rows_rescan(const float *D32, int64_t K, int Lp, const float *R, const int *items,
+                               const int *counters, unsigned long long *keys, int T, int n_blocks, int sm_count,
+                               cudaStream_t st);
+// A BF16 build screens with the template GEMM where its time centres are
+// whole samples, its BF16 rows take at least this many bytes and its
+// templates at most a quarter of the rows'.  Measured, dense against template
+// screening in us per order: 2.1 GB (EEG-like grid) 319 and 31 at 1 channel,
+// 337 and 98 at 64, 480 and 197 at 160; 393 MB 86 and 49 at 64; 268 MB 67 and
+// 51; 236 MB 63 and 45; below L2's size the dense GEMM's stream costs nothing
+// and its fewer lags win: 69 MB 34 and 37, 58 MB 28 and 43.
+constexpr int64_t kScreenMinRowBytes = 128ll << 20;
 
 // ---- tensor-core search (act_gemm.cu) -------------------------------------
 // Bf16Search holds what a BF16 dictionary build fixes (tensor maps, tile

@@ -93,6 +93,7 @@ struct ShiftTile {
                                        ((uint32_t)((PAIR ? 2 * kBM : kBM) >> 4) << 24);
 };
 constexpr int kMaxItems = 1024;    // flagged (lag, block) items per channel before the full FP32 search
+constexpr int kMaxRowItems = 512;  // the same where the items are rows of a stored dictionary
 constexpr int kRescanWarps = 4;     // independent warps per rescore block
 
 struct Smem {
@@ -618,7 +619,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 // bf16(r) - r, the Kt term bounds FP32 accumulation in the tensor core, the
 // factor the scale product).  As for the dense BF16 search, the FP32 argmax
 // lies in an item whose largest |h| is >= hmax - 2 delta - 2 eps_r.
-__global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int Kt, int L,
+// max_items: flagged items per channel before the full FP32 search;
+// err_terms: the rounding terms of that search's score (eps_r).
+__global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int Kt, int err_terms, int max_items,
                                                     const float *__restrict__ tile_max,
                                                     const float *__restrict__ blk_max,
                                                     const double2 *__restrict__ chan_norm,
@@ -638,7 +641,7 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
         const double rr = rn + drn;
         const double ulp = 1.1920928955078125e-07;  // 2^-23
         const double delta = (1.0 + 1e-5) * (eps_u * rr + drn + (double)Kt * ulp * (1.0 + eps_u) * rr);
-        const double eps_r = (double)(L + 4) * ulp * rn;
+        const double eps_r = (double)err_terms * ulp * rn;
         const double thr = (double)__uint_as_float(chmax[b]) - 2.0 * delta - 2.0 * eps_r;
         // FP32 compare against the threshold rounded down: a superset of the items
         thr_sh = __double2float_rd(thr);
@@ -657,12 +660,12 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
             for (int k = 0; k < bpt; ++k) {
                 if (bm[k] < thr_f) continue;
                 const int pos = atomicAdd(chcount + b, 1);
-                if (pos < kMaxItems) {
+                if (pos < max_items) {
                     const int at = atomicAdd(&counters[1], 1);
                     items[2 * at] = b;
                     items[2 * at + 1] = j * n_blocks + blk_order[tile * bpt + k];  // the templates' own block
                     atomicAdd((unsigned long long *)&stats[2], 1ull);
-                } else if (pos == kMaxItems) {
+                } else if (pos == max_items) {
                     // too many: the FP32 template search scores this channel in full
                     fb_list[atomicAdd(&counters[0], 1)] = b;
                     atomicAdd((unsigned long long *)&stats[1], 1ull);
@@ -1020,26 +1023,33 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
                          (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
 }
 
-cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, const float *R,
-                                    int Lp, int L, int B, unsigned long long *keys, int *fb_list, int *counters,
-                                    long long *stats, int *status, cudaStream_t st, bool pdl,
-                                    unsigned long long wait_ns) {
-    if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
+// Flags the items of every channel (first step of either resolve).
+static cudaError_t launch_flag(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, int B, int err_terms,
+                               int max_items, int *fb_list, int *counters, long long *stats, cudaStream_t st,
+                               bool pdl) {
     const RowTiling tl = make_tiling(sp, B);
     int stages = 0, threads = 0;
     size_t smem = 0;
     bool pair = false;
-    const int bn = shift_tc_bn(s, sp, tl, false, &stages, &smem, &pair, &threads);  // the GEMM's tile width for B channels
+    const int bn = shift_tc_bn(s, sp, tl, false, &stages, &smem, &pair, &threads);  // the GEMM's tile width
     const int n_tiles = sp.T_pad / bn;
     const int entries = sp.Ntc * n_tiles;
     int slices = (entries + 255) / 256;
     const int max_slices = (4 * s->sm_count + B - 1) / B;
     if (slices > max_slices) slices = max_slices;
-    cudaError_t e = launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32,
-                                  sp.Kt, L, (const float *)x.tile_max, (const float *)x.blk_max,
-                                  (const double2 *)x.chan_norm, (const unsigned int *)x.chmax,
-                                  (const unsigned int *)sp.eps_bits, (const int *)sp.blk_order, x.chcount, fb_list, counters,
-                                  x.items, stats);
+    return launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32, sp.Kt, err_terms,
+                         max_items, (const float *)x.tile_max, (const float *)x.blk_max,
+                         (const double2 *)x.chan_norm, (const unsigned int *)x.chmax,
+                         (const unsigned int *)sp.eps_bits, (const int *)sp.blk_order, x.chcount, fb_list, counters,
+                         x.items, stats);
+}
+
+cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, const float *R,
+                                    int Lp, int L, int B, unsigned long long *keys, int *fb_list, int *counters,
+                                    long long *stats, int *status, cudaStream_t st, bool pdl,
+                                    unsigned long long wait_ns) {
+    if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
+    cudaError_t e = launch_flag(s, x, sp, B, L + 4, kMaxItems, fb_list, counters, stats, st, pdl);
     if (e != cudaSuccess) return e;
     e = launch_kernel(k_shift_rescan, dim3(s->sm_count * s->rescan_blocks_per_sm), dim3(s->rescan_warps * 32),
                       s->rescan_smem, st, true, (const float *)sp.tpl, (const float *)sp.scale, sp.S, sp.Sa, sp.P,
@@ -1053,5 +1063,19 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
     return launch_shift_search(sp, R, Lp, L, B, keys, nullptr, status, true, st, fb_list, &counters[0], wait_ns);
 }
 
+cudaError_t launch_shift_tc_resolve_rows(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp,
+                                         const float *D32, int64_t K, const float *R, int Lp, int L, int B,
+                                         unsigned long long *keys, int *fb_list, int *counters, long long *stats,
+                                         int *status, int gemv_grid, cudaStream_t st, bool pdl,
+                                         unsigned long long wait_ns) {
+    if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
+    // |f - s| of the GEMV: its sum's rounding, and the row's own (the
+    // template's sample times the FP32 scale, both rounded) beside it
+    cudaError_t e = launch_flag(s, x, sp, B, L + 8, kMaxRowItems, fb_list, counters, stats, st, pdl);
+    if (e == cudaSuccess)
+        e = launch_rows_rescan(D32, K, Lp, R, x.items, counters, keys, sp.T, sp.T_pad / 32, s->sm_count, st);
+    if (e != cudaSuccess) return e;
+    return launch_gemv_argmax(D32, K, Lp, R, B, fb_list, &counters[0], keys, status, gemv_grid, st, wait_ns, true);
+}
 
 }  // namespace act
