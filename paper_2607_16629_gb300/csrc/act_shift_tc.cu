@@ -77,6 +77,7 @@ constexpr int kStepsPerChunk = kBK / kUmmaK;
 constexpr int kMaxThreads = 384;  // two epilogue groups
 constexpr int kAChunkBytes = kBM * kBK * 2;  // 16 KB
 constexpr int kMaxStages = 6;
+constexpr unsigned kAccPause = 64;  // ns between an epilogue group's looks at its accumulator
 constexpr int kUnitTab = 1024;  // row units whose lag range is tabulated in shared memory
 constexpr int kTileTab = 512;   // template tiles whose lag span is
 
@@ -522,7 +523,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
                 epilogue_bar(bar_id);
             }
             const uint32_t acc = local & 1u, aph = (local >> 1) & 1u;
-            const bool landed = mbar_poll<PAIR>(&sm.bar_acc_full[acc], aph, wait_ns, 256);
+            const bool landed = mbar_poll<PAIR>(&sm.bar_acc_full[acc], aph, wait_ns, kAccPause);
             const int failed = (*abort_flag || !landed) ? 1 : 0;
             if (epilogue_bar_or(bar_id, failed)) {  // the group's warps leave together
                 *abort_flag = 1;
@@ -538,16 +539,23 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
             float *bm = blk_max + ((size_t)(valid ? b : 0) * Ntc + (valid ? j : 0)) * (T_pad / 32) +
                         (size_t)nt * (BN / 32);
             float mx = 0.0f, bmv[BN / 32];
+            // the next 32 columns are on their way while these are scaled
+            const uint32_t cols = tmem + ((uint32_t)(q * 32) << 16) + acc * BN;
+            uint32_t v[2][32];
+            tmem_load32(cols, v[0]);
 #pragma unroll
             for (int c = 0; c < BN / 32; ++c) {
-                float v[32];
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + acc * BN + c * 32, v);
+                tmem_wait32(v[c & 1]);
+                if (c + 1 < BN / 32) tmem_load32(cols + (c + 1) * 32, v[(c + 1) & 1]);
+                const uint32_t(&x)[32] = v[c & 1];
                 float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const float4 s = valid ? sc4[c * 8 + e] : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float2 p01 = mul_f32x2(v[4 * e], v[4 * e + 1], s.x, s.y);
-                    const float2 p23 = mul_f32x2(v[4 * e + 2], v[4 * e + 3], s.z, s.w);
+                    const float2 p01 =
+                        mul_f32x2(__uint_as_float(x[4 * e]), __uint_as_float(x[4 * e + 1]), s.x, s.y);
+                    const float2 p23 =
+                        mul_f32x2(__uint_as_float(x[4 * e + 2]), __uint_as_float(x[4 * e + 3]), s.z, s.w);
                     m0 = max_abs3(m0, p01.x, p01.y);
                     m1 = max_abs3(m1, p23.x, p23.y);
                 }
