@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
         uint32_t s = 0, ph = 0;  // the ring's stage and its phase parity
         for (int64_t w = unit0; w < items && !*abort_flag; w += n_units) {
-            const int u = (int)(w / n_tiles), nt = (int)(w % n_tiles);
+            const int u = (int)((uint32_t)w / (uint32_t)n_tiles), nt = (int)((uint32_t)w % (uint32_t)n_tiles);
             // this CTA's row tile (PAIR: past the last tile, load the last one again)
             const int mt = PAIR ? min(2 * u + (int)rank, tl.m_tiles - 1) : u;
             int ks_lo, ks_hi;
@@ -437,8 +437,18 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         // MMA per 128 cycles): no divisions, descriptors formed once per stage
         const bool issuer = elect_one();
         uint32_t s = 0, ph = 0, local = 0;
+        auto test_full = [&](uint32_t st, uint32_t parity) {
+            return PAIR ? mbar_test_wait_cluster(&sm.bar_full[st], parity) : mbar_test_wait(&sm.bar_full[st], parity);
+        };
+        bool landed = false;  // the stage about to be multiplied was seen complete a stage ago
         for (int64_t w = unit0; w < items; w += n_units, ++local) {
             const uint32_t acc = local & 1u, aph = (local >> 1) & 1u;
+            int ks_lo, ks_hi;
+            const int u = (int)((uint32_t)w / (uint32_t)n_tiles), nt = (int)(w - (int64_t)u * n_tiles);
+            item_steps(u < kUnitTab ? sm.unit_steps[u] : unit_steps(tl, PAIR, u),
+                       nt < kTileTab ? sm.tile_steps[nt] : tile_steps<BN>(span, nt), ks_lo, ks_hi);
+            ks_lo = __shfl_sync(0xffffffffu, ks_lo, 0);
+            ks_hi = __shfl_sync(0xffffffffu, ks_hi, 0);
             const bool ok = PAIR ? mbar_wait_cluster(&sm.bar_acc_empty[acc], aph ^ 1u, wait_ns)
                                  : mbar_wait(&sm.bar_acc_empty[acc], aph ^ 1u, wait_ns);
             if (!__all_sync(0xffffffffu, ok && !*abort_flag)) {
@@ -447,31 +457,40 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
             }
             tc_fence_after();
             const uint32_t d_tmem = tmem + acc * BN;
-            int ks_lo, ks_hi;
-            const int u = (int)(w / n_tiles), nt = (int)(w - (int64_t)u * n_tiles);
-            item_steps(u < kUnitTab ? sm.unit_steps[u] : unit_steps(tl, PAIR, u),
-                       nt < kTileTab ? sm.tile_steps[nt] : tile_steps<BN>(span, nt), ks_lo, ks_hi);
-            ks_lo = __shfl_sync(0xffffffffu, ks_lo, 0);
-            ks_hi = __shfl_sync(0xffffffffu, ks_hi, 0);
             const int kc_lo = ks_lo / kStepsPerChunk, kc_hi = ks_hi / kStepsPerChunk;
             bool all = true;
             for (int kc = kc_lo; kc <= kc_hi; ++kc) {
-                all = __all_sync(0xffffffffu, mbar_poll<PAIR>(&sm.bar_full[s], ph, wait_ns, 0));
-                if (!all) break;
+                if (!landed) {
+                    all = __all_sync(0xffffffffu, mbar_poll<PAIR>(&sm.bar_full[s], ph, wait_ns, 0));
+                    if (!all) break;
+                }
                 tc_fence_after();
+                const uint32_t s1 = s + 1 == (uint32_t)stages ? 0u : s + 1, ph1 = s1 == 0u ? ph ^ 1u : ph;
+                // look at the next stage's barrier now: the answer is there when
+                // these MMAs are issued (a look took some 290 cycles, now 170;
+                // 64 EEG-like channels 1.88 -> 1.81 ms with this, whole chunks
+                // issued without a test per step and 32-bit divisions)
+                const bool next = test_full(s1, ph1);
                 const uint32_t b0 = base + s * (uint32_t)kStageBytes;
-                const uint64_t bdesc = smem_desc(b0), adesc = smem_desc(b0 + kBChunkBytes);
                 // only the chunk's steps inside [ks_lo, ks_hi]
-                const int k_lo = ks_lo - kc * kStepsPerChunk, k_hi = ks_hi - kc * kStepsPerChunk;
+                const int k0 = max(ks_lo - kc * kStepsPerChunk, 0);
+                const int n = min(ks_hi - kc * kStepsPerChunk, kStepsPerChunk - 1) - k0 + 1;
+                const uint64_t bdesc = smem_desc_k(smem_desc(b0), k0);
+                const uint64_t adesc = smem_desc_k(smem_desc(b0 + kBChunkBytes), k0);
                 if (issuer) {
-#pragma unroll
-                    for (int k = 0; k < kStepsPerChunk; ++k) {
-                        if (k < k_lo || k > k_hi) continue;
-                        const uint32_t accum = kc != kc_lo || k != k_lo ? 1u : 0u;
+                    auto mma = [&](int k, bool accum) {
                         if constexpr (PAIR)
-                            tc_mma_pair(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum);
+                            tc_mma_pair(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum ? 1u : 0u);
                         else
-                            tc_mma(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum);
+                            tc_mma(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum ? 1u : 0u);
+                    };
+                    mma(0, kc != kc_lo);
+                    if (n == kStepsPerChunk) {
+#pragma unroll
+                        for (int k = 1; k < kStepsPerChunk; ++k) mma(k, true);
+                    } else {
+                        if (n > 1) mma(1, true);
+                        if (n > 2) mma(2, true);
                     }
                     if constexpr (PAIR)
                         tc_commit_pair(&sm.bar_empty[s], 0x3);
@@ -479,10 +498,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
                         tc_commit(&sm.bar_empty[s]);
                 }
                 __syncwarp();
-                if (++s == (uint32_t)stages) {
-                    s = 0;
-                    ph ^= 1u;
-                }
+                landed = __all_sync(0xffffffffu, next);
+                s = s1;
+                ph = ph1;
             }
             if (!all) {
                 *abort_flag = 1;
@@ -506,7 +524,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
                        (size_t)eg * tl.Jt * kScaleLd;
         uint32_t local = (uint32_t)eg;
         for (int64_t w = unit0 + eg * n_units; w < items; w += n_eg * n_units, local += n_eg) {
-            const int unit = (int)(w / n_tiles), nt = (int)(w % n_tiles);
+            const int unit = (int)((uint32_t)w / (uint32_t)n_tiles), nt = (int)((uint32_t)w % (uint32_t)n_tiles);
             const int mt = PAIR ? 2 * unit + (int)rank : unit;  // PAIR: may be one past the last tile (no rows)
             // the tile's Jt scale rows (j0 .. j0 + Jt - 1, those below Ntc), BN each
             {
