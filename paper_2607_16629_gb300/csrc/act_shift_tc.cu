@@ -657,10 +657,11 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
                                                     int *__restrict__ counters, int *__restrict__ items,
                                                     long long *__restrict__ stats) {
     const int b = blockIdx.y;
-    __shared__ float thr_sh;
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the GEMM's maxima
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (threadIdx.x == 0) {  // the bound in FP64, once per block
+    __shared__ float bound_sh;
+    // The bound, in FP64 by one thread, while the GEMM still runs: it lets
+    // this kernel launch only after its own wait for the rows kernel that
+    // wrote the norms.  One FP32 difference is left behind the wait.
+    if (threadIdx.x == 0) {
         const double2 nr = chan_norm[b];
         const double rn = nr.x, drn = nr.y;
         const double eps_u = (double)__uint_as_float(*eps_bits);
@@ -668,37 +669,50 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
         const double ulp = 1.1920928955078125e-07;  // 2^-23
         const double delta = (1.0 + 1e-5) * (eps_u * rr + drn + (double)Kt * ulp * (1.0 + eps_u) * rr);
         const double eps_r = (double)err_terms * ulp * rn;
-        const double thr = (double)__uint_as_float(chmax[b]) - 2.0 * delta - 2.0 * eps_r;
-        // FP32 compare against the threshold rounded down: a superset of the items
-        thr_sh = __double2float_rd(thr);
+        bound_sh = __double2float_ru(2.0 * delta + 2.0 * eps_r);
     }
     __syncthreads();
-    const float thr_f = thr_sh;
+    const float bound = bound_sh;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the GEMM's maxima
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the threshold rounded down: a superset of the items
+    const float thr_f = __fsub_rd(__uint_as_float(chmax[b]), bound);
     // scan the tile maxima; a tile at or above the threshold is narrowed to
     // its 32-template blocks at or above it (the items: j * n_blocks + block)
     const float *tm = tile_max + (size_t)b * Ntc * n_tiles;
     const int n_entries = Ntc * n_tiles;
     const int n_blocks = n_tiles * bpt;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_entries; i += gridDim.x * blockDim.x) {
-        if (tm[i] >= thr_f) {
-            const int j = i / n_tiles, tile = i - j * n_tiles;
-            const float *bm = blk_max + ((size_t)b * Ntc + j) * n_blocks + (size_t)tile * bpt;
-            for (int k = 0; k < bpt; ++k) {
-                if (bm[k] < thr_f) continue;
-                const int pos = atomicAdd(chcount + b, 1);
-                if (pos < max_items) {
-                    const int at = atomicAdd(&counters[1], 1);
-                    items[2 * at] = b;
-                    items[2 * at + 1] = j * n_blocks + blk_order[tile * bpt + k];  // the templates' own block
-                    atomicAdd((unsigned long long *)&stats[2], 1ull);
-                } else if (pos == max_items) {
-                    // too many: the FP32 template search scores this channel in full
-                    fb_list[atomicAdd(&counters[0], 1)] = b;
-                    atomicAdd((unsigned long long *)&stats[1], 1ull);
-                    atomicAdd((unsigned long long *)&stats[0], ~0ull);  // -1: not resolved by the items
-                }
-            }
+        if (!(tm[i] >= thr_f)) continue;
+        const int j = i / n_tiles, tile = i - j * n_tiles;
+        const float4 *bm4 =
+            reinterpret_cast<const float4 *>(blk_max + ((size_t)b * Ntc + j) * n_blocks + (size_t)tile * bpt);
+        float bm[8];  // bpt is 4 or 8
+        *reinterpret_cast<float4 *>(bm) = bm4[0];
+        *reinterpret_cast<float4 *>(bm + 4) = bpt > 4 ? bm4[1] : make_float4(-1.f, -1.f, -1.f, -1.f);
+        int hits = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) hits += k < bpt && bm[k] >= thr_f;
+        if (hits == 0) continue;
+        const int pos = atomicAdd(chcount + b, hits);
+        const int take = max(0, min(hits, max_items - pos));
+        if (pos <= max_items && pos + hits > max_items) {
+            // too many: the FP32 search scores this channel in full
+            fb_list[atomicAdd(&counters[0], 1)] = b;
+            atomicAdd((unsigned long long *)&stats[1], 1ull);
+            atomicAdd((unsigned long long *)&stats[0], ~0ull);  // -1: not resolved by the items
         }
+        if (take == 0) continue;
+        int at = atomicAdd(&counters[1], take);
+        const int end = at + take;
+        atomicAdd((unsigned long long *)&stats[2], (unsigned long long)take);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k < bpt && bm[k] >= thr_f && at < end) {
+                items[2 * at] = b;
+                items[2 * at + 1] = j * n_blocks + blk_order[tile * bpt + k];  // the templates' own block
+                ++at;
+            }
     }
 }
 
