@@ -72,7 +72,7 @@ __device__ __forceinline__ float warp_sum_32(float (&v)[32], int lane) {
 // older copy is still in flight, and a parity wait would let it pass.
 template <int N8, int N4, bool WRITE_SCORES>
 __global__ void __launch_bounds__(kMultiThreads, 1)
-    k_gemv_multi(const float *__restrict__ D, int64_t K, int Lp, const float *__restrict__ R, int ng,
+    k_gemv_multi(const float *__restrict__ D, int64_t K, int Lp, const float *R, int ng,
                  unsigned long long *__restrict__ keys, float *__restrict__ scores, int tiles, int stages, int *status,
                  unsigned long long wait_ns) {
     constexpr int NCH = 8 * N8 + 4 * N4, G = N8 + N4;

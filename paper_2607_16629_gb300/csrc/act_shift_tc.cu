@@ -96,6 +96,13 @@ struct ShiftTile {
 constexpr int kMaxItems = 1024;    // flagged (lag, block) items per channel before the full FP32 search
 constexpr int kMaxRowItems = 512;  // the same where the items are rows of a stored dictionary
 constexpr int kRescanWarps = 4;     // independent warps per rescore block
+constexpr int kRescanBufs = 8;      // phase buffers per warp, at most
+// Bytes of a warp's buffers where it has more than two: with few channels
+// (few items) one or two warps an SM with every phase in flight, with many
+// four warps an SM.  One EEG-like channel 536 -> 511 us per decomposition, 64
+// of them 1,730 us with two buffers a warp and 1,768 with four.
+constexpr int kRescanFewBytes = 108 * 1024;
+constexpr int kRescanFewChannels = 16;
 
 struct Smem {
     uint64_t bar_full[kMaxStages];
@@ -648,10 +655,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 // max_items: flagged items per channel before the full FP32 search;
 // err_terms: the rounding terms of that search's score (eps_r).
 __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int Kt, int err_terms, int max_items,
-                                                    const float *__restrict__ tile_max,
-                                                    const float *__restrict__ blk_max,
-                                                    const double2 *__restrict__ chan_norm,
-                                                    const unsigned int *__restrict__ chmax,
+                                                    const float *tile_max, const float *blk_max,
+                                                    const double2 *__restrict__ chan_norm, const unsigned int *chmax,
                                                     const unsigned int *__restrict__ eps_bits,
                                                     const int *__restrict__ blk_order, int *__restrict__ chcount, int *__restrict__ fb_list,
                                                     int *__restrict__ counters, int *__restrict__ items,
@@ -676,7 +681,9 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the GEMM's maxima
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the threshold rounded down: a superset of the items
-    const float thr_f = __fsub_rd(__uint_as_float(chmax[b]), bound);
+    // (what the GEMM writes is read through pointers without __restrict__: a
+    // load that the compiler may take for constant could move before the wait)
+    const float thr_f = __fsub_rd(__uint_as_float(*(const volatile unsigned int *)&chmax[b]), bound);
     // scan the tile maxima; a tile at or above the threshold is narrowed to
     // its 32-template blocks at or above it (the items: j * n_blocks + block)
     const float *tm = tile_max + (size_t)b * Ntc * n_tiles;
@@ -717,96 +724,94 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
 }
 
 // FP32 rescore, one warp per flagged (lag, 32-template block) item.  Lane =
-// template.  Per phase
-// a, the P template rows the FP32 template search reads for this lag
-// (contiguous, P x 128 bytes) arrive by a bulk copy into one of the warp's
-// two buffers (the next phase's copy is in flight while this one is used);
-// each lane runs the FP32 search's FMA chain over them in its order and
-// scales the sum the same way.  Each warp owns its barriers, buffers and
-// residual phases; warps never wait on one another.
+// template.  Per phase a, the P template rows the FP32 template search reads
+// for this lag (contiguous, P x 128 bytes) arrive by a bulk copy into one of
+// the warp's nb buffers (the copies of the next nb - 1 phases are in flight
+// while this one is used); each lane runs the FP32 search's FMA chain over
+// them in its order and scales the sum the same way.  Each warp owns its
+// barriers, buffers and residual phases; warps never wait on one another.
+// Bound by latency: the item, the copies (all at once where nb = Sa) and the
+// chain of L dependent FMAs.
 __global__ void __launch_bounds__(kRescanWarps * 32) k_shift_rescan(
     const float *__restrict__ tpl, const float *__restrict__ scale, int S, int Sa, int P, int rows, int NtcP,
-    int Ntc, int T, int n_blocks, int Lp, int L, const float *__restrict__ R, const int *__restrict__ items,
-    const int *__restrict__ counters, unsigned long long *__restrict__ keys, int *status,
+    int Ntc, int T, int n_blocks, int Lp, int L, const float *R, const int2 *items, int64_t max_tasks, int nb,
+    const int *counters, unsigned long long *__restrict__ keys, int *status,
     unsigned long long wait_ns) {
-    extern __shared__ __align__(128) float sm[];  // per warp: the residual [Lp], then 2 x [P][32] rows
-    __shared__ __align__(8) uint64_t bar[kRescanWarps][2];
+    extern __shared__ __align__(128) float sm[];  // per warp: the residual [Lp], then nb x [P][32] rows
+    __shared__ __align__(8) uint64_t bar[kRescanWarps][kRescanBufs];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t warp_floats = (size_t)Lp + 2 * (size_t)P * 32;
+    const size_t buf_floats = (size_t)P * 32, warp_floats = (size_t)Lp + nb * buf_floats;
     float *rres = sm + warp * warp_floats;
     float *buf0 = rres + Lp;
     const uint32_t bytes = (uint32_t)P * 128u;
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the flagged items
-    const int n_tasks = counters[1];  // at most kMaxItems per channel
-    // the fallback search behind this kernel may launch now: it reads
-    // nothing of ours before its wait for our completion
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int nw = (int)(blockDim.x >> 5);
-    if (lane == 0) {
-        mbar_init(&bar[warp][0], 1);
-        mbar_init(&bar[warp][1], 1);
-        fence_mbar_init();
-    }
+    if (lane < nb) mbar_init(&bar[warp][lane], 1);
+    fence_mbar_init();
     __syncwarp();
-    uint32_t uses[2] = {0u, 0u};
-    int cur_b = -1;
     // tasks go to the first warp of every block before the second (one task
     // per SM while there are fewer tasks than SMs)
     const int64_t stride = (int64_t)gridDim.x * nw;
-    for (int64_t task = (int64_t)warp * gridDim.x + blockIdx.x; task < n_tasks; task += stride) {
-        const int b = items[2 * task];
-        const int e = items[2 * task + 1];  // j * n_blocks + block
-        const int j = e / n_blocks, tb = e % n_blocks;
+    int64_t task = (int64_t)warp * gridDim.x + blockIdx.x;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the flagged items
+    // the first item is read beside the number of items, which says whether it
+    // is one (neither may move before the wait: volatile, and no __restrict__)
+    const volatile int2 *item_v = items;
+    int2 item = make_int2(0, 0);
+    if (task < max_tasks) item = make_int2(item_v[task].x, item_v[task].y);
+    const int n_tasks = *(const volatile int *)&counters[1];  // at most kMaxItems per channel
+    // the fallback search behind this kernel may launch now: it reads
+    // nothing of ours before its wait for our completion
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    uint32_t par = 0u;  // bit i: the parity buffer i's next copy completes
+    int cur_b = -1;
+    for (bool first = true; task < n_tasks; task += stride, first = false) {
+        if (!first) item = items[task];
+        const int b = item.x;
+        const int j = item.y / n_blocks, tb = item.y % n_blocks;
         if (tb * 32 >= T) continue;  // past the last template
         const float *src = tpl + ((size_t)tb * Sa * rows + (size_t)(NtcP - 1 - j)) * 32;
+        auto copy = [&](int a, uint32_t more) {  // lane 0: phase a's rows into buffer a % nb
+            uint64_t *br = &bar[warp][a % nb];
+            mbar_expect_tx(br, bytes + more);
+            bulk_g2s(buf0 + (size_t)(a % nb) * buf_floats, src + (size_t)a * rows * 32, bytes, br);
+        };
         __syncwarp();
-        if (lane == 0) {  // phase 0's rows and, for a new channel, its residual on the same barrier
+        if (lane == 0) {  // a new channel's residual with phase 0's rows
             const bool new_b = b != cur_b;
-            mbar_expect_tx(&bar[warp][0], bytes + (new_b ? (uint32_t)Lp * 4u : 0u));
-            bulk_g2s(buf0, src, bytes, &bar[warp][0]);
+            copy(0, new_b ? (uint32_t)Lp * 4u : 0u);
             if (new_b) bulk_g2s(rres, R + (size_t)b * Lp, (uint32_t)Lp * 4u, &bar[warp][0]);
+            for (int a = 1; a < nb && a < Sa; ++a) copy(a, 0u);
         }
         cur_b = b;
+        // the scale is needed last: on its way meanwhile
+        const float sc = scale[((size_t)tb * NtcP + j) * 32 + lane];
         float acc = 0.0f;
-        int ok = 1, fail_a = 0;
-        for (int a = 0; a < Sa; ++a) {
-            const int cb = a & 1;
-            if (a + 1 < Sa && lane == 0) {
-                // the other buffer was released by the __syncwarp ending phase a - 1
-                mbar_expect_tx(&bar[warp][cb ^ 1], bytes);
-                bulk_g2s(buf0 + (size_t)(cb ^ 1) * P * 32, src + (size_t)(a + 1) * rows * 32, bytes,
-                         &bar[warp][cb ^ 1]);
-            }
-            ok = mbar_wait(&bar[warp][cb], uses[cb] & 1u, wait_ns) ? 1 : 0;
-            ++uses[cb];
+        for (int a = 0, cb = 0; a < Sa; ++a) {
+            const int ok = mbar_wait(&bar[warp][cb], par >> cb & 1u, wait_ns) ? 1 : 0;
             if (!__all_sync(0xffffffffu, ok)) {
-                ok = 0;
-                fail_a = a;
-                break;
+                if (lane == 0) {
+                    atomicOr(status, kFlagTimeout);
+                    // bounded: let the copies in flight land before the warp leaves
+                    for (int f = a; f < Sa && f < a + nb; ++f) mbar_drain(&bar[warp][f % nb], par >> (f % nb) & 1u);
+                }
+                return;
             }
+            par ^= 1u << cb;
             // sample n = a + S p of the window (0 past it, as in the FP32 search's phases)
-            const float *bp = buf0 + (size_t)cb * P * 32 + lane;
+            const float *bp = buf0 + (size_t)cb * buf_floats + lane;
 #pragma unroll 8
             for (int p = 0; p < P; ++p) {
                 const int n = a + S * p;
                 acc = fmaf(n < L ? rres[n] : 0.0f, bp[p * 32], acc);
             }
             __syncwarp();
-        }
-        if (!ok) {
-            if (lane == 0) {
-                atomicOr(status, kFlagTimeout);
-                // bounded: let the copies in flight land before the warp leaves
-                const int cb = fail_a & 1;
-                mbar_drain(&bar[warp][cb], (uses[cb] - 1) & 1u);
-                if (fail_a + 1 < Sa) mbar_drain(&bar[warp][cb ^ 1], uses[cb ^ 1] & 1u);
-            }
-            return;
+            if (a + nb < Sa && lane == 0) copy(a + nb, 0u);  // into the buffer just used
+            if (++cb == nb) cb = 0;
         }
         const int t = tb * 32 + lane;
         unsigned long long key = 0ull;
         if (t < T) {
-            const float sv = acc * scale[((size_t)tb * NtcP + j) * 32 + lane];
+            const float sv = acc * sc;
             const float x = fabsf(sv);
             if (x == x) key = pack_key(x, (uint32_t)j * (uint32_t)T + (uint32_t)t);
         }
@@ -829,8 +834,10 @@ struct ShiftTc {
     CUtensorMap mapB[2];    // box heights 128 and 256
     int nkc = 0, sm_count = 0, T_pad = 0;
     int pair_clusters = 0;  // co-resident CTA pairs of the paired GEMM (0: not available)
-    int rescan_warps = 0, rescan_blocks_per_sm = 0;
-    size_t rescan_smem = 0;
+    struct {
+        int bufs = 0, warps = 0, blocks_per_sm = 0;
+        size_t smem = 0;
+    } rescan[2];  // few channels, many
 };
 
 cudaError_t shift_tc_prepare(ShiftTc **out, const ShiftPlan &sp, int sm_count) {
@@ -874,19 +881,28 @@ cudaError_t shift_tc_prepare(ShiftTc **out, const ShiftPlan &sp, int sm_count) {
         }
         s->pair_clusters = clusters;
     }
-    // rescore: per warp the residual and two P-row buffers; as many warps per
+    // rescore: per warp the residual and its P-row buffers; as many warps per
     // block (up to kRescanWarps) as fit
-    const size_t per_warp = sizeof(float) * ((size_t)sp.Lp + 2 * (size_t)sp.P * 32);
-    int rw = kRescanWarps;
-    while (rw > 1 && rw * per_warp > (size_t)kSmemBudget) --rw;
-    s->rescan_warps = rw;
-    s->rescan_smem = rw * per_warp;
-    if (e == cudaSuccess && s->rescan_smem > (size_t)kSmemBudget) e = cudaErrorNotSupported;
-    if (e == cudaSuccess) e = allow_max_smem((const void *)k_shift_rescan, s->rescan_smem);
-    if (e == cudaSuccess) {
+    const size_t buf = (size_t)sp.P * 128, res = sizeof(float) * (size_t)sp.Lp;
+    size_t most = 0;
+    for (int i = 0; i < 2; ++i) {
+        int nb = 2;
+        while (i == 0 && nb < sp.Sa && nb < kRescanBufs && res + (nb + 1) * buf <= (size_t)kRescanFewBytes) ++nb;
+        const size_t per_warp = res + nb * buf;
+        int rw = kRescanWarps;
+        while (rw > 1 && rw * per_warp > (size_t)kSmemBudget) --rw;
+        s->rescan[i].bufs = nb;
+        s->rescan[i].warps = rw;
+        s->rescan[i].smem = rw * per_warp;
+        most = s->rescan[i].smem > most ? s->rescan[i].smem : most;
+        if (e == cudaSuccess && s->rescan[i].smem > (size_t)kSmemBudget) e = cudaErrorNotSupported;
+    }
+    if (e == cudaSuccess) e = allow_max_smem((const void *)k_shift_rescan, most);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shift_rescan, rw * 32, s->rescan_smem);
-        s->rescan_blocks_per_sm = per_sm < 1 ? 1 : per_sm;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shift_rescan, s->rescan[i].warps * 32,
+                                                          s->rescan[i].smem);
+        s->rescan[i].blocks_per_sm = per_sm < 1 ? 1 : per_sm;
     }
     if (e != cudaSuccess) {
         delete s;
@@ -1091,10 +1107,11 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
     if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
     cudaError_t e = launch_flag(s, x, sp, B, L + 4, kMaxItems, fb_list, counters, stats, st, pdl);
     if (e != cudaSuccess) return e;
-    e = launch_kernel(k_shift_rescan, dim3(s->sm_count * s->rescan_blocks_per_sm), dim3(s->rescan_warps * 32),
-                      s->rescan_smem, st, true, (const float *)sp.tpl, (const float *)sp.scale, sp.S, sp.Sa, sp.P,
-                      sp.rows, sp.NtcP, sp.Ntc, sp.T, sp.T_pad / 32, Lp, L, R, (const int *)x.items,
-                      (const int *)counters, keys, status, wait_ns);
+    const auto &rc = s->rescan[B <= kRescanFewChannels ? 0 : 1];
+    e = launch_kernel(k_shift_rescan, dim3(s->sm_count * rc.blocks_per_sm), dim3(rc.warps * 32), rc.smem, st, true,
+                      (const float *)sp.tpl, (const float *)sp.scale, sp.S, sp.Sa, sp.P, sp.rows, sp.NtcP, sp.Ntc,
+                      sp.T, sp.T_pad / 32, Lp, L, R, reinterpret_cast<const int2 *>(x.items),
+                      (int64_t)x.B_cap * kMaxItems, rc.bufs, (const int *)counters, keys, status, wait_ns);
     if (e != cudaSuccess) return e;
     // channels with more than kMaxItems flagged items: the FP32 template
     // search over the queue, launched early (its CTAs become resident while
