@@ -167,7 +167,7 @@ cudaError_t launch_init(const float *sig, int B, int L, int Lp, float *R, __nv_b
 // float pairs and returned in FP64, the selected atom's parameters decoded
 // from its flat index, the key cleared for the next order.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kUpdateThreads) k_update(const float *__restrict__ D32, int Lp, int L,
+__global__ void __launch_bounds__(kUpdateThreads + 32) k_update(const float *__restrict__ D32, int Lp, int L,
                                                            float *__restrict__ R, __nv_bfloat16 *__restrict__ R16,
                                                            int Lb, unsigned long long *__restrict__ keys,
                                                            GridAxes ax, int k, int P,
@@ -186,18 +186,34 @@ __global__ void __launch_bounds__(kUpdateThreads) k_update(const float *__restri
     float *r = R + (int64_t)b * Lp;
 
     float part = 0.0f;
-    for (int n = threadIdx.x; n < L; n += blockDim.x) part = fmaf(g[n], r[n], part);
+    // the atom's and the residual's samples stay in registers between the passes
+    constexpr int kPer = kMaxSamples / kUpdateThreads;
+    float gv[kPer], rv[kPer];
+    const bool record = threadIdx.x >= kUpdateThreads;  // the extra warp: the atom's record (FP64), no samples
+    if (record) write_atom_lanes(ax, idx, atoms + (int64_t)b * P + k);
+    const int n0 = record ? L : (int)threadIdx.x;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int n = n0 + i * kUpdateThreads;
+        gv[i] = n < L ? g[n] : 0.0f;
+        rv[i] = n < L ? r[n] : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < kPer; ++i)
+        if (n0 + i * kUpdateThreads < L) part = fmaf(gv[i], rv[i], part);
     const float c = block_sum(part, shf);
 
     ff e = {0.0f, 0.0f};  // |r_{k+1}|^2 as a float pair (about 2^-44 relative)
-    for (int n = threadIdx.x; n < L; n += blockDim.x) {
-        const float v = fmaf(-c, g[n], r[n]);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int n = n0 + i * kUpdateThreads;
+        if (n >= L) continue;
+        const float v = fmaf(-c, gv[i], rv[i]);
         r[n] = v;
         ff_add_square(e, v);
         if (R16) R16[(int64_t)b * Lb + n] = __float2bfloat16_rn(v);
     }
     const ff tot = block_sum_ff(e, shp);
-    if (threadIdx.x < 32) write_atom_lanes(ax, idx, atoms + (int64_t)b * P + k);
     if (threadIdx.x == 0) {
         coefs[(int64_t)b * P + k] = c;
         energy[(int64_t)b * (P + 1) + k + 1] = ff_to_double(tot);
@@ -212,7 +228,7 @@ __global__ void __launch_bounds__(kUpdateThreads) k_update(const float *__restri
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
                           unsigned long long *keys, const GridAxes &ax, int k, int P, act_atom *atoms, float *coefs,
                           double *energy, int *fb_count, cudaStream_t st, bool pdl) {
-    return launch_kernel(k_update, dim3(B), dim3(kUpdateThreads), 0, st, pdl, D32, Lp, L, R, R16, Lb, keys, ax, k, P,
+    return launch_kernel(k_update, dim3(B), dim3(kUpdateThreads + 32), 0, st, pdl, D32, Lp, L, R, R16, Lb, keys, ax, k, P,
                          atoms, coefs, energy, fb_count);
 }
 
