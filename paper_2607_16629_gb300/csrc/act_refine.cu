@@ -303,7 +303,14 @@ __device__ __forceinline__ void eval_warp_scatter(const EvalAcc &a, int lane, fl
 // Partial sums go to red[warp]; after the barrier the group's first warp
 // adds its warps' sums in warp order and finishes on the FP32 pipes.
 // Returned in every lane of each group's first warp: the score s and
-// component (lane & 3) of its gradient (zeros elsewhere).
+// component (lane & 3) of its gradient (zeros elsewhere).  kSpan: samples a
+// thread evaluates at once, 2 where L <= 512, else 4 (with 4 there, half of
+// the evaluations and more were of samples past the window: 64 EEG-like
+// channels, hierarchical search, 6.48 -> 6.27 ms).  kShort (L <= 256): the
+// second is passed over too (a 256-sample epoch 1.11 -> 1.01 ms).  With kSpan
+// 1 the compiler fuses products and sums differently, and a trajectory
+// changes with its last bits; this form keeps them.
+template <int kSpan, bool kShort>
 __device__ __forceinline__ void eval_cands(const EvalConst *ec, const float *__restrict__ r, int L, float (*red)[12],
                                            ff *s_out, float *gi_out) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -313,13 +320,14 @@ __device__ __forceinline__ void eval_cands(const EvalConst *ec, const float *__r
         // kSpan samples of the thread at once: their evaluations are
         // independent (the latency of one overlaps the others), then they
         // are accumulated in sample order
-        constexpr int kStride = 32 * kCandWarps, kSpan = 4;
+        constexpr int kStride = 32 * kCandWarps;
         const EvalConst e = ec[h];
         for (int n0 = t; n0 < L; n0 += kSpan * kStride) {
             float u[kSpan], du[kSpan][4], rv[kSpan];
 #pragma unroll
             for (int k = 0; k < kSpan; ++k) {
                 const int n = n0 + k * kStride;
+                if (kShort && k > 0 && n0 - t + k * kStride >= L) break;  // the same for all threads
                 rv[k] = n < L ? r[n] : 0.0f;
                 eval_sample(n < L ? n : 0, e, u[k], du[k]);
             }
@@ -393,6 +401,7 @@ __device__ __forceinline__ void eval_cands(const EvalConst *ec, const float *__r
 // halvings.  Then the BFGS inverse update (when <y, s> > 0).  It stops early
 // when no step is accepted.  Bookkeeping runs on warp 0 (lane & 3 =
 // parameter, the 4 x 4 update on 16 lanes); the other warps only evaluate.
+template <int kSpan, bool kShort>
 __global__ void __launch_bounds__(kBfgsThreads) k_refine(GridAxes ax, RefineBox box, int steps, int Lp,
                                                           const float *__restrict__ R,
                                                           const unsigned long long *__restrict__ keys,
@@ -455,7 +464,7 @@ __global__ void __launch_bounds__(kBfgsThreads) k_refine(GridAxes ax, RefineBox 
     {  // the start point (every group of every CTA of the cluster evaluates it, with the same bits)
         ff s0;
         float g0;
-        eval_cands(slot_ec, r, L, red, &s0, &g0);
+        eval_cands<kSpan, kShort>(slot_ec, r, L, red, &s0, &g0);
         if (warp == 0 && lane < 4) {
             const float sg = s0.hi < 0.0f ? -1.0f : 1.0f;
             gz[pi] = -sg * g0 * wf[pi];
@@ -515,7 +524,7 @@ __global__ void __launch_bounds__(kBfgsThreads) k_refine(GridAxes ax, RefineBox 
         const int s0 = slot0;
         ff sc;
         float gi;
-        eval_cands(slot_ec + s0, r, L, red, &sc, &gi);
+        eval_cands<kSpan, kShort>(slot_ec + s0, r, L, red, &sc, &gi);
         if (warp % kCandWarps == 0 && lane < 4 * C) {
             // lane = (destination CTA, parameter): this candidate into every
             // CTA's list of the round
@@ -716,6 +725,10 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
         box.zlo[i] = box.lo[i] / box.w[i];
         box.zhi[i] = box.hi[i] / box.w[i];
     }
+    void (*kern)(GridAxes, RefineBox, int, int, const float *, const unsigned long long *, const double *, int, double *,
+                 int) = k_refine<4, false>;
+    if (ax.L <= 64 * kCandWarps) kern = k_refine<2, false>;
+    if (ax.L <= 32 * kCandWarps) kern = k_refine<2, true>;
     // a cluster of C CTAs per channel: the largest C of kRefineCluster, 2, 1
     // for which every channel's cluster is resident at once (measured: 64
     // channels refine 23 % faster on clusters of 2 in one wave than on
@@ -738,7 +751,7 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
         cfg.gridDim = dim3((unsigned)(B * c));
         cfg.numAttrs = 1;
         int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, k_refine, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess) {
             cudaGetLastError();
             clusters = 0;
         }
@@ -752,7 +765,7 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
         int per_sm = 0, sms = 0, dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_refine, kBfgsThreads, 0);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBfgsThreads, 0);
         if (e != cudaSuccess) cudaGetLastError();
         // one CTA per channel when that puts every channel on at once (or no
         // cluster can be placed), else full clusters over several waves
@@ -766,7 +779,7 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
         cfg.gridDim = dim3((unsigned)B);
         cfg.numAttrs = 0;
     }
-    return cudaLaunchKernelEx(&cfg, k_refine, ax, box, steps, Lp, R, keys, theta_in, theta_in_stride, theta_out, C);
+    return cudaLaunchKernelEx(&cfg, kern, ax, box, steps, Lp, R, keys, theta_in, theta_in_stride, theta_out, C);
 }
 
 cudaError_t launch_update_refined(int Lp, float *R, __nv_bfloat16 *R16, int Lb, int B, unsigned long long *keys,
