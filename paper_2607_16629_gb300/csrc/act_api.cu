@@ -135,6 +135,7 @@ struct WorkBuffers {
     int lem_B = 0;
     Bf16Scratch b16;                  // dense tensor-core search maxima and rescan lists (on first use)
     ShiftTcScratch stc;               // tensor-core template search rows, maxima, items (on first use)
+    bool dense16 = false;             // no memory for a BF16 build's template screening: the dense GEMM screens
 };
 
 struct act_grid {
@@ -158,6 +159,7 @@ struct act_grid {
     ShiftTc *shift_tc = nullptr;  // its tensor-core search (ACT_SEARCH_SHIFT_BF16)
     ShiftPlan screen;             // templates of a BF16 build's atoms, for its screening GEMM
     ShiftTc *screen_tc = nullptr; // null: the dense GEMM over the BF16 rows screens
+    int screen_channels = 0;      // most channels of a call that the templates screen
     int gemv_grid = 0;
     bool gemv_stream = false;  // FP32 search by the bulk-copy streaming GEMV (one CTA per SM)
     int refine_steps = 0;  // BFGS iterations per order (0: grid-only search)
@@ -246,6 +248,7 @@ void free_dictionary(act_grid *g) {
     // the tensor-core search scratch is sized by the dictionary's shape
     bf16_scratch_free(g->w.b16);
     shift_tc_scratch_free(g->w.stc);
+    g->w.dense16 = false;
 }
 
 #define ACT_AL(ptr, bytes)                                                          \
@@ -315,11 +318,17 @@ act_status scratch_status(cudaError_t e, const char *what) {
     return e == cudaErrorMemoryAllocation ? ACT_ERR_OOM : ACT_ERR_CUDA;
 }
 
+// Whether a BF16 search of B channels on w screens through the templates
+// (else by the dense GEMM over the BF16 rows).
+bool screens(const act_grid *g, const WorkBuffers &w, int B) {
+    return g->screen_tc && !w.dense16 && B <= g->screen_channels;
+}
+
 // Whether w holds everything `mode` needs for B channels and P orders.
 bool work_fits(const act_grid *g, const WorkBuffers &w, int B, int P, act_search_mode mode) {
     if (B > w.cap_B || P > w.cap_P) return false;
     if (mode == ACT_SEARCH_LEM && (w.lem.cap < lem_capacity(g->lem) || w.lem_B < B || !w.lem.cand)) return false;
-    if (mode == ACT_SEARCH_BF16 && (g->screen_tc ? w.stc.B_cap : w.b16.B_cap) < B) return false;
+    if (mode == ACT_SEARCH_BF16 && (screens(g, w, B) ? w.stc.B_cap : w.b16.B_cap) < B) return false;
     if (mode == ACT_SEARCH_SHIFT_BF16 && w.stc.B_cap < B) return false;
     return true;
 }
@@ -346,11 +355,11 @@ act_status grow_work(const act_grid *g, WorkBuffers &w, int B, int P, act_search
             return s;
         }
     }
-    if (mode == ACT_SEARCH_BF16 && g->screen_tc && w.stc.B_cap < B) {
-        if ((s = scratch_status(shift_tc_reserve(g->screen_tc, g->screen, B, w.stc), "shift_tc_reserve")) != ACT_OK)
-            return s;
-    }
-    if (mode == ACT_SEARCH_BF16 && !g->screen_tc && w.b16.B_cap < B) {
+    // (without the memory for its scratch, these buffers' searches take the
+    // dense GEMM, whose scratch is smaller, from here on)
+    if (mode == ACT_SEARCH_BF16 && screens(g, w, B) && w.stc.B_cap < B)
+        w.dense16 = shift_tc_reserve(g->screen_tc, g->screen, B, w.stc) != cudaSuccess;
+    if (mode == ACT_SEARCH_BF16 && !screens(g, w, B) && w.b16.B_cap < B) {
         if ((s = scratch_status(bf16_scratch_reserve(g->bf16, B, w.b16), "bf16_scratch_reserve")) != ACT_OK)
             return s;
     }
@@ -448,7 +457,7 @@ cudaError_t launch_fp32_search(const act_grid *g, const WorkBuffers &w, int B, c
 act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_search_mode mode, GraphEntry &ge,
                             cudaStream_t st, bool profiling, bool allow_fused) {
     const bool bf16 = mode == ACT_SEARCH_BF16;
-    __nv_bfloat16 *R16 = bf16 && !g->screen_tc ? w.R16 : nullptr;  // the dense GEMM's operand
+    __nv_bfloat16 *R16 = bf16 && !screens(g, w, B) ? w.R16 : nullptr;  // the dense GEMM's operand
     int kernels = 0;
     const int fctas = allow_fused ? fused_ctas(g, B, mode, profiling) : 0;
     if (fctas > 0) {  // the single-launch form (it also initialises the residuals)
@@ -488,7 +497,7 @@ act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_searc
             ACT_CK(launch_shift_tc_resolve(g->shift_tc, w.stc, g->shift, w.R, g->Lp, g->L, B, w.keys, w.fb_list,
                                            w.fb_count, g->stats, g->status, st, !profiling, g->wait_ns));
             kernels += 5;
-        } else if (bf16 && g->screen_tc) {
+        } else if (bf16 && screens(g, w, B)) {
             ACT_CK(launch_shift_tc_gemm(g->screen_tc, w.stc, g->screen, w.R, g->Lp, g->L, B, g->stats, g->status, st,
                                         !profiling, g->wait_ns, g->cta_pairs));
             if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
@@ -778,11 +787,18 @@ static uint64_t template_bytes(const act_grid *g) {
 // The screening templates of a BF16 build (kScreenMinRowBytes).  Without
 // them, for want of memory too, the dense GEMM over the BF16 rows screens.
 static void build_screen(act_grid *g, cudaStream_t st) {
-    const int64_t row_bytes = (int64_t)sizeof(__nv_bfloat16) * g->K * g->Lb;
+    const uint64_t row16 = sizeof(__nv_bfloat16) * (uint64_t)g->K * (uint64_t)g->Lb;
+    const uint64_t all_rows = row16 + sizeof(float) * (uint64_t)g->K * (uint64_t)g->Lp;
     const uint64_t bt = template_bytes(g);
-    if (row_bytes < kScreenMinRowBytes || bt == 0 ||
-        bt > ((uint64_t)row_bytes + sizeof(float) * (uint64_t)g->K * (uint64_t)g->Lp) / 4)
+    if (row16 < (uint64_t)kScreenMinRowBytes || bt == 0 || bt > all_rows / 4) return;
+    // at most a quarter of what the rows left free: the rest is for the work
+    // buffers and for the caller's own memory
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        cudaGetLastError();
         return;
+    }
+    if (bt > free_bytes / 4) return;
     ShiftPlan sp;
     if (shift_plan(sp, g->ax) != cudaSuccess || sp.Kt == 0) return;
     sp.Lp = g->Lp;
@@ -792,7 +808,14 @@ static void build_screen(act_grid *g, cudaStream_t st) {
         cudaGetLastError();
         g->screen_tc = nullptr;
         free_templates(g->screen);
+        return;
     }
+    // channels whose scratch (maxima and shifted residual rows) takes no more
+    // than the rows do, within the launch limit of the template GEMM
+    const uint64_t per_channel = (uint64_t)sp.Ntc * (sizeof(float) * (uint64_t)(sp.T_pad / 128 + sp.T_pad / 32) +
+                                                     sizeof(__nv_bfloat16) * (uint64_t)sp.Kt);
+    const uint64_t most = all_rows / per_channel;
+    g->screen_channels = most < 65535 ? (int)most : 65535;
 }
 
 // ACT_DICT_AUTO: the FP32 rows when they fit the memory budget, else the
@@ -1068,7 +1091,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {  // pass 0 warms up
             e = cudaEventRecord(e0, st);
             for (int r = 0; r < reps && e == cudaSuccess; ++r) {
-                if (use_bf16 && g->screen_tc) {
+                if (use_bf16 && screens(g, g->w, channels)) {
                     e = cudaMemsetAsync(g->w.fb_count, 0, 2 * sizeof(int), st);
                     if (e == cudaSuccess)
                         e = launch_shift_tc_gemm(g->screen_tc, g->w.stc, g->screen, g->w.R, g->Lp, g->L, channels,
@@ -1130,8 +1153,9 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
     // tensor-core search: tile width x pipeline depth of the dense GEMM, or,
     // where the templates screen, that search as it is
     double best16 = 1e30;
-    if (bf16 && g->screen_tc && err == cudaSuccess) err = time_search(true, &best16);
-    if (bf16 && !g->screen_tc && err == cudaSuccess) {
+    const bool dense = bf16 && !screens(g, g->w, channels);
+    if (bf16 && !dense && err == cudaSuccess) err = time_search(true, &best16);
+    if (dense && err == cudaSuccess) {
         int best_bn = 256, best_st = 0;
         const int widths[2] = {128, 256};
         for (int wi = 0; wi < 2 && err == cudaSuccess; ++wi) {

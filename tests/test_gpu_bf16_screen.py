@@ -101,3 +101,20 @@ def test_uneven_batch_and_a_later_larger_call():
         act.act_ragged_plan_destroy(plan)
         for h in hs:
             act.act_destroy(h)
+
+
+def test_more_channels_than_the_templates_screen():
+    """Past the channel count whose screening scratch would outgrow the rows
+    (1,980 on this grid) the dense GEMM screens; calls on either side of it
+    alternate on one grid."""
+    g = GRIDS["mid"]
+    sig = torch.tensor(synth.random_signals(11, 2100, g.n_samples), dtype=torch.float32, device="cuda")
+    h = act.act_grid_create(g, 0)
+    try:
+        act.act_dictionary_build(h, act.ACT_DICT_BF16)
+        want = run(h, act.ACT_SEARCH_FP32, sig, 2)
+        for B in (3, 2100, 1900, 2100, 3):
+            for x, y in zip(run(h, act.ACT_SEARCH_BF16, sig[:B], 2), want):
+                assert torch.equal(x, y[:B])
+    finally:
+        act.act_destroy(h)
