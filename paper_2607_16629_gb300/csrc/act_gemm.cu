@@ -361,16 +361,17 @@ __global__ void __launch_bounds__(256) k_select(int64_t ntiles, int bpt, const f
 // into keys[b] with the packed atomicMax (largest |score|, then lowest
 // index).  One block of 8 warps per pair.
 __global__ void __launch_bounds__(256) k_rescan(const float *__restrict__ D32, int64_t K, int Lp, int tile_atoms,
-                                                const float *__restrict__ R, const int *__restrict__ pairs,
-                                                const int *__restrict__ counters,
+                                                const float *__restrict__ R, const int *pairs, const int *counters,
                                                 unsigned long long *__restrict__ keys, int T, int n_blocks) {
     // (a programmatic dependent of the kernel that flagged the items, where
-    // the template GEMM screens)
+    // the template GEMM screens: their number and the items are read without
+    // __restrict__, which would let those loads move ahead of the wait; what
+    // R is read at depends on them)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     __shared__ float red_s[8];
     __shared__ uint32_t red_i[8];
-    const int n_items = counters[1];
+    const int n_items = *(const volatile int *)&counters[1];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nv = Lp / 128;
     const int rows_per_warp = tile_atoms / 8;
@@ -392,9 +393,8 @@ __global__ void __launch_bounds__(256) k_rescan(const float *__restrict__ D32, i
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int64_t row = row0 + i + u;
-                sc[u] = row < row_end ? fabsf(row_score(reinterpret_cast<const float4 *>(D32 + (size_t)row * Lp), res, nv,
-                                                  lane))
-                                : -1.0f;
+                const float4 *a = reinterpret_cast<const float4 *>(D32 + (size_t)row * Lp);
+                sc[u] = row < row_end ? fabsf(row_score(a, res, nv, lane)) : -1.0f;
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u)

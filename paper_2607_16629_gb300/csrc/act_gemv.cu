@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
     constexpr int kWarps = kGemvThreads / 32;
     const int64_t gw = (int64_t)blockIdx.x * kWarps + wid;
     const int64_t nw = (int64_t)gridDim.x * kWarps;
-    const int count = count_dev ? *count_dev : B;
+    const int count = count_dev ? *(const volatile int *)count_dev : B;  // not before the wait
     const int Lp4 = Lp >> 2;
     const float4 *D4 = reinterpret_cast<const float4 *>(D);
 

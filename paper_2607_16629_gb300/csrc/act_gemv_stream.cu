@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int count = count_dev ? *count_dev : B;
+    const int count = count_dev ? *(const volatile int *)count_dev : B;  // not before the wait
     // this CTA's chunks: k-th is chunk blockIdx.x + k gridDim.x of the dictionary
     const int64_t total_chunks = (K + rows_per_chunk - 1) / rows_per_chunk;
     const int64_t n_chunks =

@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(kUpdateThreads + 32) k_update(const float *__r
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
                           unsigned long long *keys, const GridAxes &ax, int k, int P, act_atom *atoms, float *coefs,
                           double *energy, int *fb_count, cudaStream_t st, bool pdl) {
-    return launch_kernel(k_update, dim3(B), dim3(kUpdateThreads + 32), 0, st, pdl, D32, Lp, L, R, R16, Lb, keys, ax, k, P,
-                         atoms, coefs, energy, fb_count);
+    return launch_kernel(k_update, dim3(B), dim3(kUpdateThreads + 32), 0, st, pdl, D32, Lp, L, R, R16, Lb, keys, ax, k,
+                         P, atoms, coefs, energy, fb_count);
 }
 
 }  // namespace act

@@ -155,9 +155,11 @@ __device__ __forceinline__ void lem_neighbour(const double *__restrict__ th, int
 // so large that FP64 does not hold it, c is infinite: k_lem_pick then always
 // projects the candidate again.
 // Bound by the special-function pipe (two a sample, 16 cycles a warp, and
-// about as many other issues): SCREEN_US for 64 channels x 2,048 candidates x
-// 512 samples, where the float-float projection of all took 230 us (118
-// instructions a sample).
+// about as many other issues): 44 us for 64 channels x 2,048 candidates x 512
+// samples, where the float-float projection of all took 230 us (118
+// instructions a sample).  The cosine as a polynomial on the FMA pipe instead
+// was 6 % slower over the whole search (packed FP32 FMAs take two passes of
+// that pipe), for one sample in four neither faster nor slower.
 constexpr float kScreenX = 5.8f;
 constexpr int kScreenCands = 64;
 constexpr float kScreenWide = 2.0f;
@@ -229,7 +231,8 @@ __global__ void __launch_bounds__(kLemThreads) k_lem_screen(int cap, int level, 
         k.dx = dx * kScale;
         k.xs = (float)((double)(32 * k.row_lo) - p[0]) * k.dx;
         const float K = (float)(k.row_hi - k.row_lo), w = x0 + 1.5f;
-        const float a_cos = 6.2831853f * (2.3283064e-10f * (1.0f + K + 0.5f * K * K) + 5.9604645e-8f) + 5.1e-7f + 7.6e-7f;
+        const float a_phase = 6.2831853f * (2.3283064e-10f * (1.0f + K + 0.5f * K * K) + 5.9604645e-8f);
+        const float a_cos = a_phase + 5.1e-7f + 7.6e-7f;
         const float a_env = w * 1.7e-6f + w * w * 8e-7f + 5e-7f;
         k.c_u = 2.0f * 2.0f * (a_cos + a_env + 2e-6f) * sqrtf(1.7724539f / dx + 1.0f);
         k.c_s = 2.0f * 2.0f * (K + 40.0f) * 5.9604645e-8f;

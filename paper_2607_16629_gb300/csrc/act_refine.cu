@@ -725,8 +725,7 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
         box.zlo[i] = box.lo[i] / box.w[i];
         box.zhi[i] = box.hi[i] / box.w[i];
     }
-    void (*kern)(GridAxes, RefineBox, int, int, const float *, const unsigned long long *, const double *, int, double *,
-                 int) = k_refine<4, false>;
+    auto *kern = k_refine<4, false>;
     if (ax.L <= 64 * kCandWarps) kern = k_refine<2, false>;
     if (ax.L <= 32 * kCandWarps) kern = k_refine<2, true>;
     // a cluster of C CTAs per channel: the largest C of kRefineCluster, 2, 1

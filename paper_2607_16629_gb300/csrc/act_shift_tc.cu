@@ -325,7 +325,8 @@ template <int BN, bool PAIR>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     k_shift_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowTiling tl,
                  int n_tiles, int nkc, int stages, int T_pad, const short2 *__restrict__ span,
-                 const float *__restrict__ scaleT, float *__restrict__ tile_max, float *__restrict__ blk_max, unsigned int *__restrict__ chmax,
+                 const float *__restrict__ scaleT, float *__restrict__ tile_max, float *__restrict__ blk_max,
+                 unsigned int *__restrict__ chmax,
                  int *status, unsigned long long wait_ns) {
     // shared memory: stages, then the item's scales [Jt][BN + 4] (the +4
     // floats of padding spread the Jt rows a warp reads over the banks)
@@ -486,10 +487,11 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
                 const uint64_t adesc = smem_desc_k(smem_desc(b0 + kBChunkBytes), k0);
                 if (issuer) {
                     auto mma = [&](int k, bool accum) {
+                        const uint64_t da = smem_desc_k(adesc, k), db = smem_desc_k(bdesc, k);
                         if constexpr (PAIR)
-                            tc_mma_pair(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum ? 1u : 0u);
+                            tc_mma_pair(d_tmem, da, db, Cfg::kIdesc, accum ? 1u : 0u);
                         else
-                            tc_mma(d_tmem, smem_desc_k(adesc, k), smem_desc_k(bdesc, k), Cfg::kIdesc, accum ? 1u : 0u);
+                            tc_mma(d_tmem, da, db, Cfg::kIdesc, accum ? 1u : 0u);
                     };
                     mma(0, kc != kc_lo);
                     if (n == kStepsPerChunk) {
@@ -658,7 +660,8 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
                                                     const float *tile_max, const float *blk_max,
                                                     const double2 *__restrict__ chan_norm, const unsigned int *chmax,
                                                     const unsigned int *__restrict__ eps_bits,
-                                                    const int *__restrict__ blk_order, int *__restrict__ chcount, int *__restrict__ fb_list,
+                                                    const int *__restrict__ blk_order, int *__restrict__ chcount,
+                                                    int *__restrict__ fb_list,
                                                     int *__restrict__ counters, int *__restrict__ items,
                                                     long long *__restrict__ stats) {
     const int b = blockIdx.y;
@@ -1075,8 +1078,8 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
     const int grid = (int)(items < s->sm_count ? items : s->sm_count);
     // a programmatic dependent of the shifted-row build (set-up overlaps it)
     return launch_kernel(bn == 256 ? k_shift_gemm<256, false> : k_shift_gemm<128, false>, dim3(grid), dim3(threads),
-                         smem, st, true, mapA, s->mapB[i], tl, n_tiles, s->nkc, stages, sp.T_pad, (const short2 *)sp.span,
-                         (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
+                         smem, st, true, mapA, s->mapB[i], tl, n_tiles, s->nkc, stages, sp.T_pad,
+                         (const short2 *)sp.span, (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
 }
 
 // Flags the items of every channel (first step of either resolve).
@@ -1093,8 +1096,8 @@ static cudaError_t launch_flag(const ShiftTc *s, const ShiftTcScratch &x, const 
     int slices = (entries + 255) / 256;
     const int max_slices = (4 * s->sm_count + B - 1) / B;
     if (slices > max_slices) slices = max_slices;
-    return launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32, sp.Kt, err_terms,
-                         max_items, (const float *)x.tile_max, (const float *)x.blk_max,
+    return launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32, sp.Kt,
+                         err_terms, max_items, (const float *)x.tile_max, (const float *)x.blk_max,
                          (const double2 *)x.chan_norm, (const unsigned int *)x.chmax,
                          (const unsigned int *)sp.eps_bits, (const int *)sp.blk_order, x.chcount, fb_list, counters,
                          x.items, stats);

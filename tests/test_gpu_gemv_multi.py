@@ -27,8 +27,9 @@ def grid(n, tc, fc, c):
 
 # row widths 128 .. 2048 floats; atoms: fewer than a tile, one more than a
 # chunk, more chunks than SMs, none a multiple of the tile
-GRIDS = {"n37": grid(37, 1, 2, 1), "n100": grid(100, 11, 37, 5), "n256": grid(256, 13, 41, 7), "n300": grid(300, 9, 33, 5),
-         "n512": grid(512, 17, 29, 7), "n1024": grid(1024, 5, 23, 3), "n2048": grid(2048, 7, 31, 3)}
+GRIDS = {"n37": grid(37, 1, 2, 1), "n100": grid(100, 11, 37, 5), "n256": grid(256, 13, 41, 7),
+         "n300": grid(300, 9, 33, 5), "n512": grid(512, 17, 29, 7), "n1024": grid(1024, 5, 23, 3),
+         "n2048": grid(2048, 7, 31, 3)}
 
 
 @pytest.mark.parametrize("channels", [2, 3, 4, 5, 8, 9, 12, 13, 16, 17, 29])

@@ -49,7 +49,8 @@ def test_screened_selection_is_the_oracles(name):
     lo, hi = (np.array([f(a.lo, a.lo + (a.count - 1) * a.step) for a in axes]) for f in (min, max))
     params = oracle.lem_params(n_coarse, top_k, levels, STEPS, RADIUS)
     B, seed = 3, 99
-    sig = np.stack([synth.eeg_like_signal(2, 200 + b, n_samples=g.n_samples, fs=g.fs)[0] for b in range(B)]).astype(np.float32)
+    sig = np.stack([synth.eeg_like_signal(2, 200 + b, n_samples=g.n_samples, fs=g.fs)[0] for b in range(B)])
+    sig = sig.astype(np.float32)
     sig[1] = 0.0
     h = act.act_grid_create(g, 0)
     try:
