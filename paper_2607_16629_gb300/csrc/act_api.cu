@@ -480,7 +480,7 @@ act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_searc
             ACT_CK(cudaEventRecordWithFlags(ev[0], st, cudaEventRecordExternal));
         }
         if (mode == ACT_SEARCH_LEM) {
-            ACT_CK(launch_lem_select(g->lem, B, k, w.R, g->Lp, g->L, g->desc.fs, w.lem, st));
+            ACT_CK(launch_lem_select(g->lem, B, k, w.R, g->Lp, g->L, g->desc.fs, w.lem, st, !profiling));
             if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
             kernels += lem_kernels(g->lem);
         } else if (mode == ACT_SEARCH_SHIFT) {
@@ -523,7 +523,7 @@ act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_searc
             ACT_CK(launch_refine(g->ax, g->refine_steps, g->Lp, w.R, nullptr, w.lem.kept, 4 * g->lem.top_k, B,
                                  w.theta, st));
             ACT_CK(launch_update_refined(g->Lp, w.R, nullptr, g->Lb, B, nullptr, g->ax, w.theta, k, P, w.atoms,
-                                         w.coefs, w.energy, nullptr, st));
+                                         w.coefs, w.energy, nullptr, st, !profiling));
             kernels += 2;
         } else if (g->refine_steps > 0) {
             ACT_CK(launch_refine(g->ax, g->refine_steps, g->Lp, w.R, w.keys, nullptr, 0, B, w.theta, st));

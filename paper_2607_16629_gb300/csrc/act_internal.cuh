@@ -202,7 +202,7 @@ struct LemBuffers {
     int *nkept = nullptr;         // [B]
 };
 cudaError_t launch_lem_select(const LemConfig &cfg, int B, int order, const float *R, int Lp, int L, double fs,
-                              const LemBuffers &lb, cudaStream_t st);
+                              const LemBuffers &lb, cudaStream_t st, bool pdl = false);
 int lem_kernels(const LemConfig &cfg);
 
 // ---- off-grid refinement (act_refine.cu) ----------------------------------
@@ -214,7 +214,7 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
                           const double *theta_in, int theta_in_stride, int B, double *theta_out, cudaStream_t st);
 cudaError_t launch_update_refined(int Lp, float *R, __nv_bfloat16 *R16, int Lb, int B, unsigned long long *keys,
                                   const GridAxes &ax, const double *theta, int k, int P, act_atom *atoms, float *coefs,
-                                  double *energy, int *fb_count, cudaStream_t st);
+                                  double *energy, int *fb_count, cudaStream_t st, bool pdl = false);
 
 // ---- template (shift-correlation) dictionary and search (act_shift.cu) ----
 struct ShiftPlan {
