@@ -117,7 +117,8 @@ typedef enum {
  *                    tile and per 32-atom block (on grids of whole-sample
  *                    time centres and 128 MiB of BF16 rows or more, where the
  *                    templates of ACT_DICT_RECOMPUTE take little memory
- *                    beside them, every atom is scored through its BF16
+ *                    beside them, and while the call's scratch does not
+ *                    outgrow the rows, every atom is scored through its BF16
  *                    template instead of its row); the blocks that an error
  *                    bound cannot exclude are rescored in FP32 (a channel
  *                    with more than 512 of them takes the FP32 search), so
@@ -362,11 +363,14 @@ ACT_API act_status act_chirplet_score(int32_t n_samples, double fs, const double
  * on this grid's dictionary with the caller's `channels` signals
  * [channels][n_samples] (device or host memory) as residuals, keeps the
  * fastest, and returns its time per order in *best_ms (may be NULL).
- * Candidates: resident CTAs per SM of the FP32 GEMV (1..4, as occupancy
- * allows), the bulk-copy streaming GEMV and, when the grid holds a BF16 dictionary,
- * tile width (128 or 256 atoms) x pipeline depth (2 .. what fits in shared
- * memory) of the tensor-core GEMM, each timed with its tile selection and
- * rescan; with an ACT_DICT_RECOMPUTE build, every valid (lags per thread,
+ * Candidates: with one channel, resident CTAs per SM of the load-streaming
+ * FP32 GEMV (1..4, as occupancy allows) and the bulk-copy streaming GEMV
+ * (several channels have one FP32 form, which is only timed: a call with one
+ * channel then takes the load-streaming GEMV); when the grid holds a BF16
+ * dictionary, tile width (128 or 256 atoms) x pipeline depth (2 .. what fits
+ * in shared memory) of the tensor-core GEMM over its rows, each timed with
+ * its tile selection and rescan (where templates screen, that search is only
+ * timed); with an ACT_DICT_RECOMPUTE build, every valid (lags per thread,
  * warps, stages, CTAs per SM) combination of the template search instead
  * (act_set_shift_tuning).
  * Results never depend on the configuration, only the speed does.
@@ -375,13 +379,15 @@ ACT_API act_status act_chirplet_score(int32_t n_samples, double fs, const double
 ACT_API act_status act_autotune(act_grid *grid, const float *signals, int32_t channels, void *cuda_stream,
                                 double *best_ms);
 
-/* The configuration in use: FP32 GEMV grid size in CTAs (-1: the
- * bulk-copy streaming GEMV, one CTA per SM), tensor-core tile width in atoms
- * and pipeline stages (0 and 0 without a BF16 dictionary). */
+/* The configuration in use: grid size in CTAs of the one-channel FP32 GEMV
+ * (-1: the bulk-copy streaming GEMV, one CTA per SM; the initial choice where
+ * the FP32 rows take 64 MiB or more), tensor-core tile width in atoms
+ * and pipeline stages of the GEMM over BF16 rows (0 and 0 without a BF16
+ * dictionary). */
 ACT_API act_status act_get_tuning(const act_grid *grid, int32_t *gemv_ctas, int32_t *bf16_tile_atoms,
                                   int32_t *bf16_stages);
 
-/* Sets the configuration by hand: gemv_ctas > 0 sets the FP32 GEMV grid
+/* Sets the configuration by hand: gemv_ctas > 0 sets the one-channel FP32 GEMV grid
  * (at most the resident limit), -1 selects the bulk-copy streaming GEMV (the
  * dictionary brought into shared memory by TMA bulk copies, one CTA per SM;
  * same scores and selections), 0 keeps the current choice;

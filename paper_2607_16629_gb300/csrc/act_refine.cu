@@ -18,10 +18,10 @@
 // this GPU).
 //
 // Refinement.  BFGS on f(z) = -|s(w (.) z)| in coordinates scaled by the
-// grid steps w, one cluster of 4 CTAs per channel: p = -H grad f (H reset to
-// I when p is not a descent direction), a first step of at most half a grid
-// step, Armijo backtracking (c1 = 1e-4, up to 20 halvings, evaluated four
-// step sizes at a time, one per CTA), the standard BFGS inverse update when
+// grid steps w, a cluster of up to 4 CTAs per channel: p = -H grad f (H reset
+// to I when p is not a descent direction), a first step of at most half a grid
+// step, Armijo backtracking (c1 = 1e-4, up to 20 halvings, evaluated two step
+// sizes per CTA at a time), the standard BFGS inverse update when
 // <y, s> > 0, parameters clamped to the grid box widened by one step; it
 // stops early when no step is accepted.
 #include <cuda_runtime.h>
@@ -736,9 +736,10 @@ cudaError_t launch_refine(const GridAxes &ax, int steps, int Lp, const float *R,
     if (ax.L <= 64 * kCandWarps) kern = k_refine<2, false>;
     if (ax.L <= 32 * kCandWarps) kern = k_refine<2, true>;
     // a cluster of C CTAs per channel: the largest C of kRefineCluster, 2, 1
-    // for which every channel's cluster is resident at once (measured: 64
-    // channels refine 23 % faster on clusters of 2 in one wave than on
-    // clusters of 4 in two; 32 channels fastest on clusters of 4); when no
+    // for which every channel's cluster is resident at once (measured: 32
+    // radar-like channels 3.65 ms per decomposition on clusters of 4 and 3.92
+    // on clusters of 2; 64 EEG-like channels, two CTAs of a 4-cluster an SM,
+    // 6.19 either way; clusters of 4 in two waves were 23 % slower); when no
     // size fits, clusters of kRefineCluster.  Every size takes the same
     // steps (the first that satisfies the Armijo condition), so the results
     // do not depend on it.

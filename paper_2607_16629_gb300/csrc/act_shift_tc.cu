@@ -7,9 +7,11 @@
 //     residual rows (M = 128 rows per tile), K = Kt lags.  A tile multiplies
 //     only the lags that its rows' windows see and its templates span
 //     (k_shift_spans).  That is bounded by the tensor pipe and the issue of
-//     its MMAs, so fewer lags is what helps: 256 uneven EMG-like channels
-//     (atoms of 9-111 samples in windows of 256-2,048) 57.8 -> 34.6 ms per
-//     30-order decomposition, 32 radar-like channels 4.54 -> 4.17 ms;
+//     its MMAs, so fewer lags is what helps: by that alone 256 uneven EMG-like
+//     channels (atoms of 9-111 samples in windows of 256-2,048) went from 57.8
+//     to 34.6 ms per 30-order decomposition, 32 radar-like channels from 4.54
+//     to 4.17 ms (with the issue loop and the epilogue below now 25.2 and
+//     3.64; 64 EEG-like channels 2.40 and now 1.73);
 //  2. the tcgen05 GEMM scales every accumulator by its atom's 1/|u| and keeps,
 //     per row, the largest |score| of every template tile and of every
 //     32-template block;
