@@ -161,18 +161,21 @@ __device__ __forceinline__ void lem_neighbour(const double *__restrict__ th, int
 // Where x0 > 2, or the sums are so small that squares vanish, or the phase
 // so large that FP64 does not hold it, c is infinite: k_lem_pick then always
 // projects the candidate again.
-// Bound by the special-function pipe (two a sample, 16 cycles a warp, and
-// about as many other issues): 44 us for 64 channels x 2,048 candidates x 512
-// samples, where the float-float projection of all took 230 us (118
-// instructions a sample).  The cosine as a polynomial on the FMA pipe instead
-// was 6 % slower over the whole search (packed FP32 FMAs take two passes of
-// that pipe), for one sample in four neither faster nor slower.
+// Bound by instruction issue (three slots of four busy; the special-function
+// pipe is a quarter used) beside the FP64 set-up of a block's candidates: 44
+// us for 64 channels x 2,048 candidates x 512 samples, where the float-float
+// projection of all took 230 us (118 instructions a sample).  The phase's
+// products are formed once per candidate, a lane adds its own few (6.19 ->
+// 6.13 ms per decomposition of 20 orders).  Slower or no faster: the cosine as
+// a polynomial on the FMA pipe (6 %), two samples to a packed instruction (48
+// registers: fewer warps), 32 candidates a block, 32 registers a thread.
 constexpr float kScreenX = 5.8f;
 constexpr int kScreenCands = 64;
 constexpr float kScreenWide = 2.0f;
 
 struct ScreenConst {
-    uint64_t A, B, C;     // phase of sample n: A + B n + C n^2, in 2^-64 cycles
+    uint64_t P, P1, C;    // phase of sample 32 row_lo + l: P + P1 l + C l^2, in 2^-64 cycles
+    uint64_t D32;         // its difference over 32 samples, at l = 0
     float xs, dx;         // sqrt(log2(e) / 2) x of sample 32 row_lo, and its step per sample
     int row_lo, row_hi;   // rows of 32 samples projected
     float c_u, c_s;       // error bound: (c_u / |u| + c_s) |r|
@@ -223,9 +226,7 @@ __global__ void __launch_bounds__(kLemThreads) k_lem_screen(int cap, int level, 
         ScreenConst k;
         const double g = p[3] * inv_fs * inv_fs, f = p[1] * inv_fs, gt = g * p[0];
         const double alpha = (gt - f) * p[0], beta = f - 2.0 * gt;
-        k.A = cycles64(alpha);
-        k.B = cycles64(beta);
-        k.C = cycles64(g);
+        const uint64_t A = cycles64(alpha), B = cycles64(beta), C = cycles64(g);
         const float big = (float)(fabs(gt * p[0]) + fabs(f * p[0]) + fabs(beta) * L) + fabsf((float)g) * L * (float)L;
         // 1 / dt = exp(-logdt), the argument's rounding made good
         const float ah = (float)-p[2], al = (float)(-p[2] - (double)ah);
@@ -237,6 +238,11 @@ __global__ void __launch_bounds__(kLemThreads) k_lem_screen(int cap, int level, 
         k.row_lo = lo > 0.0f ? (lo < (float)L ? (int)lo >> 5 : L) : 0;
         k.row_hi = hi < (float)L ? (hi >= 0.0f ? ((int)hi + 1 >> 5) + 1 : 0) : (L + 31) >> 5;
         k.row_hi = min(k.row_hi, (L + 31) >> 5);
+        const uint64_t n0 = 32ull * (uint64_t)k.row_lo;
+        k.P = A + (B + C * n0) * n0;
+        k.P1 = B + 2ull * C * n0;
+        k.C = C;
+        k.D32 = 32ull * (B + C * (2ull * n0 + 32ull));
         constexpr float kScale = 0.84932180f;  // sqrt(log2(e) / 2)
         k.dx = dx * kScale;
         k.xs = (float)((double)(32 * k.row_lo) - p[0]) * k.dx;
@@ -255,12 +261,13 @@ __global__ void __launch_bounds__(kLemThreads) k_lem_screen(int cap, int level, 
     for (int n = threadIdx.x; n < rows * 32; n += blockDim.x) r_sm[n] = n < L ? r[n] : 0.0f;
     __syncthreads();
     constexpr int kWarps = kLemThreads / 32;
+    const uint64_t lu = (uint64_t)lane;
     for (int q = warp; q < n_here; q += kWarps) {
         const ScreenConst k = ks[q];
-        const uint64_t n0 = (uint64_t)(32 * k.row_lo + lane);
-        // phase of the lane's first sample and its differences over 32 and 32 samples
-        uint32_t ph = (uint32_t)((k.A + (k.B + k.C * n0) * n0) >> 32) + 256u;  // + 256: the shift below rounds
-        uint32_t d1 = (uint32_t)((32ull * k.B + k.C * (64ull * n0 + 1024ull)) >> 32);
+        // phase of the lane's first sample and its differences over 32 and 32
+        // samples (+ 256: the shift below rounds)
+        uint32_t ph = (uint32_t)((k.P + lu * k.P1 + (lu * lu) * k.C) >> 32) + 256u;
+        uint32_t d1 = (uint32_t)((k.D32 + (64ull * lu) * k.C) >> 32);
         const uint32_t d2 = (uint32_t)((2048ull * k.C) >> 32);
         const float x_lane = fmaf((float)lane, k.dx, k.xs), step = 32.0f * k.dx;
         float ru = 0.0f, uu = 0.0f;
