@@ -566,9 +566,7 @@ def _targets(roofline, shift, bf16):
     search on tensor cores against the dense BF16 peak (>= 0.50).  For 64
     EEG-like channels the tensor-core search is the template form (BF16
     templates x shifted BF16 residual rows, FP32 accumulate, FP32 rescore);
-    the stored-dictionary BF16 GEMM is HBM-bound at that batch (2 B flop per
-    2 bytes of dictionary = 64 flop/byte, below the tensor ridge), so its
-    fraction is stated against HBM."""
+    the search of a stored BF16 dictionary screens with the same GEMM."""
     out = {"fp32_gemv_hbm": {"target": 0.70, "frac": roofline.get("frac"), "kernel": roofline.get("kernel"),
                              "peak": "measured hbm_gbs"}}
     ch64 = (shift or {}).get("channels_64")
@@ -579,9 +577,8 @@ def _targets(roofline, shift, bf16):
                                       "ms_per_step": ch64["tensor_ms_per_step"]}
     if bf16:
         r = bf16["roofline"]
-        out["bf16_dense_gemm_hbm"] = {"frac": r["frac"], "tensor_frac": r["tensor_frac_of_bf16_peak"],
-                                      "kernel": r["kernel"], "ms_per_step": bf16["ms_per_step"],
-                                      "note": "64 flop/byte at 64 channels: bound by HBM, not by the tensor pipe"}
+        out["bf16_stored_tensor"] = {"target": 0.50, "frac": r["frac"], "kernel": r["kernel"],
+                                     "peak": r["peak_source"], "ms_per_step": bf16["ms_per_step"]}
     return out
 
 
@@ -648,30 +645,6 @@ def _time_decompose(act, torch, h, sig, P, steps, stream, dev):
     return ms, search / max(1, n), core / max(1, n), kernels, n, [o.clone() for o in out]
 
 
-def _tc_mma_flops(grid, B):
-    """MMA flops one tensor-core template GEMM executes for B channels: the
-    library's row tiling (Bg channels x Jt time centres per 128-row tile,
-    only the 64-lag chunks the tile's windows touch), over 256-template
-    tiles (128 when those would leave SMs idle, the same count of flops)."""
-    S, tc0, Ntc, L = int(grid.tc.step), int(grid.tc.lo), grid.tc.count, grid.n_samples
-    T = grid.fc.count * grid.logdt.count * grid.c.count
-    t_pad = (T + 255) // 256 * 256
-    bg = 1
-    while bg < B and bg < 32:
-        bg <<= 1
-    n2 = 1
-    while n2 < Ntc:
-        n2 <<= 1
-    jt = min(128 // bg, n2)
-    n_cb = (B + 128 // jt - 1) // (128 // jt)
-    span0 = S * (Ntc - 1)
-    chunks = 0
-    for g in range((Ntc + jt - 1) // jt):
-        jf, jl = g * jt, min(g * jt + jt, Ntc) - 1
-        chunks += ((L - 1 + span0 - S * jf) // 64 - (span0 - S * jl) // 64 + 1) * n_cb
-    return 2.0 * 128 * t_pad * 64 * chunks
-
-
 def bench_shift(args, dev, stream, fp32_ms_per_step, fp32_atoms, clocks, peaks, peak_kind, checks):
     """Template dictionary (no atom rows stored; every atom formed in-kernel
     from its (fc, logDt, c) template) on the headline workload (one EEG-like
@@ -734,8 +707,10 @@ def bench_shift(args, dev, stream, fp32_ms_per_step, fp32_atoms, clocks, peaks, 
     alu = 2.0 * K * L / (f1[2] / 1e3) / 1e12
     tc_peak = peaks["bf16_tflops"]  # burst: the timed region is a few ms, not a seconds-long loop
     alg64 = 2.0 * B * K * L / (t64[2] / 1e3) / 1e12
-    mma_flops = _tc_mma_flops(grid, B)
-    mma64 = mma_flops / (t64[2] / 1e3) / 1e12
+    tc_files = ["paper_2607_16629_gb300/csrc/act_shift_tc.cu", "paper_2607_16629_gb300/csrc/act_tc.cuh",
+                "paper_2607_16629_gb300/csrc/act_device.cuh"]
+    mma_flops = _profile_value("shift_gemm_tc_eeg_b64.md", "mma_flops_per_launch", tc_files)
+    mma64 = mma_flops / (t64[2] / 1e3) / 1e12 if mma_flops else None
     fb = [y - x for x, y in zip(st0, st1)]
     return {"workload": "eeg_like_n512_k2097152_p20: 1 channel (the headline signal) and 64 channels",
             "value": K * P / (t1[0] / 1e3), "unit": UNIT, "ms_per_step": t1[0],
@@ -768,25 +743,27 @@ def bench_shift(args, dev, stream, fp32_ms_per_step, fp32_atoms, clocks, peaks, 
                 "resolved_items_fallbacks": fb,
                 "roofline": {"bound": "tensor", "achieved": alg64, "peak": tc_peak, "unit": "TFLOP/s",
                              "frac": alg64 / tc_peak,
-                             "traffic": _profile_traffic("shift_gemm_tc_eeg_b64.md",
-                                                         ["paper_2607_16629_gb300/csrc/act_shift_tc.cu",
-                                                          "paper_2607_16629_gb300/csrc/act_tc.cuh",
-                                                          "paper_2607_16629_gb300/csrc/act_device.cuh"]),
+                             "traffic": _profile_traffic("shift_gemm_tc_eeg_b64.md", tc_files),
                              "kernel": "k_shift_rows + k_shift_gemm<256, pair> (BF16 tcgen05 on CTA pairs, "
                                        "scaled tile maxima)",
                              "algorithmic_flops_per_launch": 2.0 * B * K * L,
                              "mma_flops_per_launch": mma_flops, "mma_tflops": mma64,
-                             "mma_frac": mma64 / tc_peak, "avg_launch_ms": t64[2],
+                             "mma_frac": mma64 / tc_peak if mma64 else None, "avg_launch_ms": t64[2],
                              "peak_source": f"{peak_kind} bf16_tflops (burst: a decomposition takes ms)",
-                             "note": "each 128-row tile (32 channels x 4 time centres) multiplies the 64-lag "
-                                     "chunks its windows touch (9 of Kt / 64 = 16): achieved counts 2 K L flops "
-                                     "per channel, mma_tflops everything the tensor cores execute; timed by an "
-                                     "event pair around the shifted-row build and the GEMM"}}}
+                             "note": "a tile (32 channels x 4 time centres x 256 templates) multiplies the lags "
+                                     "that its windows see and its templates span (the rest of every atom's "
+                                     "energy, 2^-23 a side, is in the error bound): achieved counts 2 K L flops "
+                                     "per channel as if every lag were multiplied, mma_tflops what the tensor "
+                                     "cores execute; timed by an event pair around the shifted-row build and "
+                                     "the GEMM"}}}
 
 
 def bench_bf16(args, dev, stream, peaks, peak_kind, checks):
-    """64 EEG-like channels, BF16 tensor-core search with FP32 rescore,
-    against the plain FP32 path run channel by channel."""
+    """64 EEG-like channels on the stored dictionary, BF16 tensor-core search
+    (its atoms' templates screen: the time centres are whole samples) with
+    FP32 rescore of the rows, against the plain FP32 path run channel by
+    channel.  The GEMM over the BF16 rows, which screens where there are no
+    templates, is in the channel sweep."""
     import torch
 
     from paper_2607_16629_gb300 import act, synth
@@ -805,7 +782,6 @@ def bench_bf16(args, dev, stream, peaks, peak_kind, checks):
            torch.empty((B, P + 1), dtype=torch.float64, device=dev)]
     act.act_set_search(h, act.ACT_SEARCH_BF16)
     tune_ms = act.act_autotune(h, sig, B, stream)
-    gemv_ctas, tile_atoms, stages_used = act.act_get_tuning(h)
     steps = max(3, args.steps // 2)
     for _ in range(3):
         act.act_decompose(h, sig, B, P, *out, stream)
@@ -852,27 +828,19 @@ def bench_bf16(args, dev, stream, peaks, peak_kind, checks):
     value = B * K * P * steps / (ms / 1e3)
     avg = search_ms / max(1, search_n)
     avg_gemm = gemm_ms / max(1, search_n)
-    bytes_per = K * L * 2
     flops_per = 2.0 * K * L * B
-    bw = bytes_per / (avg_gemm / 1e3) / 1e9
     tflops = flops_per / (avg_gemm / 1e3) / 1e12
     return {"workload": f"eeg_like_bf16_{B}ch_n512_grid128x64x8x32_k2097152_p20", "value": value, "unit": UNIT,
             "atoms_per_s": B * P * steps / (ms / 1e3), "ms_per_step": ms / steps, "steps": steps,
             "dtype": "bf16 x bf16 -> f32 (tensor cores), f32 tile rescan",
-            "roofline": {"bound": "hbm", "kernel": "k_gemm_tilemax (tcgen05 BF16 GEMM + per-tile and per-block maxima)",
-                         "achieved": bw, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": bw / peaks["hbm_gbs"],
-                         "traffic": _profile_traffic("gemm_tilemax_bf16_eeg_b64.md",
-                                                     ["paper_2607_16629_gb300/csrc/act_gemm.cu",
-                                                      "paper_2607_16629_gb300/csrc/act_tc.cuh",
-                                                      "paper_2607_16629_gb300/csrc/act_device.cuh"]),
-                         "peak_source": f"{peak_kind} hbm_gbs", "avg_gemm_ms": avg_gemm,
-                         "algorithmic_bytes_per_launch": bytes_per,
-                         "tensor_tflops": tflops,
-                         "tensor_frac_of_bf16_peak": tflops / peaks["bf16_tflops"],
-                         "tensor_peak_source": f"{peak_kind} bf16_tflops (burst)",
-                         "avg_search_ms_per_order": avg,
-                         "search_frac_of_hbm_roofline": bytes_per / (avg / 1e3) / 1e9 / peaks["hbm_gbs"]},
-            "autotuned": {"tile_atoms": tile_atoms, "stages": stages_used, "search_ms_per_order": tune_ms},
+            "roofline": {"bound": "tensor", "kernel": "k_shift_rows + k_shift_gemm<256, pair> (BF16 tcgen05, the "
+                                                      "stored atoms' templates)",
+                         "achieved": tflops, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
+                         "frac": tflops / peaks["bf16_tflops"], "traffic": None,
+                         "peak_source": f"{peak_kind} bf16_tflops (burst)", "avg_gemm_ms": avg_gemm,
+                         "algorithmic_flops_per_launch": flops_per, "avg_search_ms_per_order": avg,
+                         "note": "2 K L flops per channel, as if every lag were multiplied"},
+            "search_ms_per_order_tuned": tune_ms,
             "orders_resolved_by_block_rescan": c1 - c0, "blocks_rescanned": s1 - s0,
             "orders_full_fp32_fallback": f1 - f0,
             "fp32_plain_per_channel": {"value": B * K * P / (fp32_ms / 1e3), "ms": fp32_ms},
@@ -966,8 +934,8 @@ def bench_ragged(args, dev, stream, peaks, peak_kind, checks):
     its length, 30 orders, all length groups in one CUDA graph.  Two builds:
     template dictionaries (atoms generated in-kernel from per-(fc, logDt, c)
     templates, tensor-core template search), the configuration's own
-    "generated in-kernel" reading; and stored BF16 + FP32 dictionaries (108 GB)
-    with the dense BF16 tensor-core search."""
+    "generated in-kernel" reading; and stored BF16 + FP32 dictionaries (108 GB,
+    and their atoms' templates, which screen)."""
     import torch
 
     from paper_2607_16629_gb300 import act, synth
@@ -1002,8 +970,8 @@ def bench_ragged(args, dev, stream, peaks, peak_kind, checks):
                          "algorithmic_flops_per_step": flops,
                          "peak_source": f"{peak_kind} bf16_tflops (burst: a decomposition takes tens of ms)",
                          "note": "achieved = 2 K sum(N_i) flops per order x 30 orders / the event-timed "
-                                 "decomposition, every kernel of the step included: a lower bound on the "
-                                 "GEMM's own fraction"},
+                                 "decomposition, every kernel of the step included, as if every lag were "
+                                 "multiplied (the GEMM multiplies those its templates span)"},
             "stored_bf16_dictionaries": {
                 "value": C * K * P / (d_ms / 1e3), "unit": UNIT, "ms_per_step": d_ms,
                 "dictionary_build_s": d_build, "device_bytes": d_bytes, "gpu_launches": d_kernels * steps,
@@ -1285,19 +1253,19 @@ def bench_lem(args, dev, stream, peaks, peak_kind, checks):
     samples = cand * B * L
     files = ["paper_2607_16629_gb300/csrc/act_lem.cu", "paper_2607_16629_gb300/csrc/act_ff.cuh",
              "paper_2607_16629_gb300/csrc/act_device.cuh"]
-    ips = _profile_value("lem_score_eeg_b64.md", "inst_per_sample", files)
+    ips = _profile_value("lem_screen_eeg_b64.md", "inst_per_sample", files)
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     roof = sms * 4 * 32 * 2.07 / ips if ips else None  # G samples/s at the issue roof
     got = samples / (res["lem"]["search_ms_per_order"] / 1e3) / 1e9
     lem_roof = {"bound": "alu", "unit": "G samples/s", "achieved": got, "peak": roof,
                 "frac": got / roof if roof else None,
-                "traffic": _profile_traffic("lem_score_eeg_b64.md", files),
-                "kernel": "hierarchical search per order (k_lem_lhs, k_lem_score x 3 levels, k_lem_topk, k_lem_neigh)",
+                "traffic": _profile_traffic("lem_screen_eeg_b64.md", files),
+                "kernel": "hierarchical search per order (k_lem_lhs, then k_lem_screen and k_lem_pick on 3 levels)",
                 "samples_per_order": samples, "inst_per_sample": ips,
-                "peak_source": f"issue roof of k_lem_score: {sms} SMs x 4 schedulers x 32 lanes x 2.07 GHz / "
+                "peak_source": f"issue roof of k_lem_screen: {sms} SMs x 4 schedulers x 32 lanes x 2.07 GHz / "
                                "its warp instructions per sample (ncu)",
                 "timing": "event pair around the whole hierarchical search of every order in the graph: a lower "
-                          "bound on the scoring kernel's own fraction"}
+                          "bound on the screening kernel's own fraction"}
     return {"workload": "eeg_like_64ch_n512_box128x64x8x32_p20_bfgs20", "lem": res["lem"],
             "dense_bf16": res["dense_bf16"], "roofline": lem_roof,
             "lem_settings": "paper EEG settings: top_k 4, 2 levels, steps (64,2,2,5)/(32,1,1,2.5)/(16,.5,.5,.5), "
@@ -1312,7 +1280,8 @@ def bench_sweep(args, dev, stream, peaks, peak_kind):
     event pairs inside the graph), the GEMM's algorithmic tensor throughput
     2 B K N / t against the burst BF16 peak, and for the dense dictionary its
     stream rate 2 K Lb / t against the HBM copy peak (the batch at which the
-    GEMM turns from HBM- to tensor-bound, Sec. V-A's channel scaling)."""
+    GEMM turns from HBM- to tensor-bound, Sec. V-A's channel scaling).  The
+    dense dictionary's time centres lie between samples (no templates)."""
     import torch
 
     from paper_2607_16629_gb300 import act, synth
@@ -1326,7 +1295,7 @@ def bench_sweep(args, dev, stream, peaks, peak_kind):
            "peak_source": f"{peak_kind} bf16_tflops (burst) and hbm_gbs", "dense_bf16": [], "template_bf16": []}
     for name, build, search in (("dense_bf16", act.ACT_DICT_BF16, act.ACT_SEARCH_BF16),
                                 ("template_bf16", act.ACT_DICT_RECOMPUTE, act.ACT_SEARCH_SHIFT_BF16)):
-        h = act.act_grid_create(grid, dev.index)
+        h = act.act_grid_create(_between_samples(grid) if name == "dense_bf16" else grid, dev.index)
         try:
             act.act_dictionary_build(h, build, stream)
             act.act_set_search(h, search)
@@ -1340,20 +1309,25 @@ def bench_sweep(args, dev, stream, peaks, peak_kind):
                 if name == "dense_bf16":
                     gbs = 2.0 * K * L / (core_ms / 1e3) / 1e9
                     row.update({"gemm_gbs": gbs, "hbm_frac": gbs / peaks["hbm_gbs"]})
-                else:
-                    mma = _tc_mma_flops(grid, B) / (core_ms / 1e3) / 1e12
-                    row.update({"gemm_tflops_executed": mma, "executed_tensor_frac": mma / tc_peak})
                 out[name].append(row)
         finally:
             act.act_destroy(h)
     return out
 
 
+def _between_samples(grid):
+    """The same grid with its time centres a quarter of a sample later."""
+    from paper_2607_16629_gb300 import synth
+    tc = synth.Axis(grid.tc.lo + 0.25, grid.tc.step, grid.tc.count)
+    return synth.Grid(grid.n_samples, grid.fs, tc, grid.fc, grid.logdt, grid.c)
+
+
 def run_profile_case(args):
     """Small, self-checking cases for ncu captures: a few launches of one
     search kernel on a dictionary larger than L2 but a few GB at most.
       gemv_small: FP32 GEMV over 1,048,576 EEG-grid atoms (2.1 GB), 1 channel.
-      bf16_small: BF16 GEMM search over the same atoms, 64 channels.
+      bf16_small: BF16 GEMM search over as many atoms (time centres between
+        samples), 64 channels.
       fused_check: the 16,384-atom check workload (5 orders), one cooperative
         launch per decomposition."""
     import torch
@@ -1386,14 +1360,17 @@ def run_profile_case(args):
     grid = synth.Grid(full.n_samples, full.fs, synth.Axis(full.tc.lo, full.tc.step, 64), full.fc, full.logdt,
                       full.c)
     B = 1 if args.case == "gemv_small" else 64
+    if B > 1:
+        grid = _between_samples(grid)
     sig = torch.tensor(np.stack([synth.eeg_like_signal(2, b)[0] for b in range(B)]), dtype=torch.float32,
                        device="cuda")
     h = act.act_grid_create(grid, 0)
     try:
         act.act_dictionary_build(h, act.ACT_DICT_FP32 if B == 1 else act.ACT_DICT_BF16)
         act.act_set_search(h, act.ACT_SEARCH_FP32 if B == 1 else act.ACT_SEARCH_BF16)
-        if B == 1 and args.gemv == "stream":
-            act.act_set_tuning(h, -1)
+        if B == 1:
+            sms = torch.cuda.get_device_properties(0).multi_processor_count
+            act.act_set_tuning(h, -1 if args.gemv == "stream" else 4 * sms)
         for _ in range(args.steps):
             act.decompose(h, sig, 3)
         torch.cuda.synchronize()
