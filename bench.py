@@ -952,7 +952,6 @@ def bench_ragged(args, dev, stream, peaks, peak_kind, checks):
     checks["ragged_uneven_batch"] = payload
     d_ms, d_build, d_bytes, _, d_kernels, d_idx, _ = _ragged_run(act, torch, synth, sigs, lengths, offsets, P,
                                                                   act.ACT_DICT_BF16, steps, dev, stream)
-    bf16_bytes = sum(K * L * 2 for L in lengths)
     counts = {L: sum(1 for x in sigs if len(x) == L) for L in lengths}
     # algorithmic flops of the projections P = D X^T: 2 K N per channel and order
     flops = 2.0 * K * float(sum(len(x) for x in sigs)) * P
@@ -975,7 +974,6 @@ def bench_ragged(args, dev, stream, peaks, peak_kind, checks):
             "stored_bf16_dictionaries": {
                 "value": C * K * P / (d_ms / 1e3), "unit": UNIT, "ms_per_step": d_ms,
                 "dictionary_build_s": d_build, "device_bytes": d_bytes, "gpu_launches": d_kernels * steps,
-                "hbm_frac_of_bf16_dictionary_stream": bf16_bytes * P / (d_ms / 1e3) / 1e9 / peaks["hbm_gbs"],
                 "same_selections_as_template_search": float(np.mean(d_idx == t_idx)),
                 "dtype": "bf16 x bf16 -> f32 (tensor cores), f32 tile rescan"},
             "dtype": "bf16 x bf16 -> f32 (tensor cores), f32 rescore"}
