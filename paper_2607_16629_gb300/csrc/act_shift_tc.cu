@@ -10,8 +10,8 @@
 //     its MMAs, so fewer lags is what helps: by that alone 256 uneven EMG-like
 //     channels (atoms of 9-111 samples in windows of 256-2,048) went from 57.8
 //     to 34.6 ms per 30-order decomposition, 32 radar-like channels from 4.54
-//     to 4.17 ms (with the issue loop and the epilogue below now 25.2 and
-//     3.64; 64 EEG-like channels 2.40 and now 1.73);
+//     to 4.17 ms (with the issue loop, the epilogue and the row tiles below now
+//     21.3 and 3.64; 64 EEG-like channels 2.40 and now 1.74);
 //  2. the tcgen05 GEMM scales every accumulator by its atom's 1/|u| and keeps,
 //     per row, the largest |score| of every template tile and of every
 //     32-template block;
@@ -152,22 +152,30 @@ __device__ __forceinline__ float max_abs3(float a, float b, float c) {
 // the 32 rows an epilogue warp holds share one time centre (its scale loads
 // are broadcasts).  Rows of one tile see the window only over
 // L + (Jt - 1) S lags instead of Kt; outside them every product is zero.
+// A few channels past the whole blocks of 32 have tiles of their own behind
+// the others, from m_main on: Bg2 channels (B_main ..) x Jt2 time centres
+// (make_tiling).
 struct RowTiling {
     int B, Ntc, Jt, Bg, n_cb, m_tiles;
     int S, L, span0;  // span0 = -m_lo - tc0 = S (Ntc - 1); sample n at time centre j sits at lag n + span0 - S j
+    int m_main, B_main, Jt2, Bg2;
 };
 
-__host__ __device__ inline void tile_row(const RowTiling &t, int mt, int lr, int &b, int &j) {
-    const int g = mt / t.n_cb, cb = mt - g * t.n_cb;
-    b = cb * t.Bg + lr % t.Bg;
-    j = g * t.Jt + lr / t.Bg;
+// Row tile mt: channels b0 .. b0 + Bg - 1, time centres j0 .. j0 + Jt - 1.
+struct TileGeo {
+    int Bg, Jt, b0, j0;
+};
+__host__ __device__ inline TileGeo tile_geo(const RowTiling &t, int mt) {
+    if (t.Jt2 > 0 && mt >= t.m_main) return {t.Bg2, t.Jt2, t.B_main, (mt - t.m_main) * t.Jt2};
+    const int g = mt / t.n_cb;
+    return {t.Bg, t.Jt, (mt - g * t.n_cb) * t.Bg, g * t.Jt};
 }
 
 // The lags row tile mt's windows see, in steps of 16 (one MMA).
 __host__ __device__ inline void row_steps(const RowTiling &t, int mt, int &lo, int &hi) {
-    const int g = mt / t.n_cb;
-    const int j_first = g * t.Jt;
-    const int j_last = min(j_first + t.Jt, t.Ntc) - 1;
+    const TileGeo geo = tile_geo(t, mt);
+    const int j_first = geo.j0;
+    const int j_last = min(j_first + geo.Jt, t.Ntc) - 1;
     const int kk_min = t.span0 - t.S * j_last;           // sample 0 at the last time centre
     const int kk_max = t.L - 1 + t.span0 - t.S * j_first;  // sample L - 1 at the first
     lo = kk_min / kUmmaK;
@@ -297,10 +305,13 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
     const uint4 *cp16 = reinterpret_cast<const uint4 *>(rows_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c0 = k0 >> 3, c1 = k1 >> 3;
-    const int cb = b / t.Bg, bl = b - cb * t.Bg;
+    // this channel's tiles: every n_cb-th from first on
+    const bool main = b < t.B_main;
+    const int Jt = main ? t.Jt : t.Jt2, Bg = main ? t.Bg : t.Bg2, n_cb = main ? t.n_cb : 1;
+    const int cb = main ? b / Bg : 0, bl = main ? b - cb * Bg : b - t.B_main, first = main ? cb : t.m_main;
     for (int jj = warp; jj < nj; jj += blockDim.x >> 5) {
-        const int j = j0 + jj, gt = j / t.Jt, jl = j - gt * t.Jt;
-        const int row = (gt * t.n_cb + cb) * kBM + jl * t.Bg + bl;
+        const int j = j0 + jj, gt = j / Jt, jl = j - gt * Jt;
+        const int row = (gt * n_cb + first) * kBM + jl * Bg + bl;
         uint4 *out = reinterpret_cast<uint4 *>(X + (size_t)row * Kt);
         for (int c = c0 + lane; c < c1; c += 32) {
             const int o = S * jj + 8 * c - k0, sft = o & 7;
@@ -532,15 +543,16 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         const int et = threadIdx.x & 127, bar_id = 1 + eg;
         constexpr int kScaleLd = BN + 4;
         float *sc_sm = reinterpret_cast<float *>(dyn_raw + (base - smem_u32(dyn_raw)) + (size_t)stages * kStageBytes) +
-                       (size_t)eg * tl.Jt * kScaleLd;
+                       (size_t)eg * max(tl.Jt, tl.Jt2) * kScaleLd;
         uint32_t local = (uint32_t)eg;
         for (int64_t w = unit0 + eg * n_units; w < items; w += n_eg * n_units, local += n_eg) {
             const int unit = (int)((uint32_t)w / (uint32_t)n_tiles), nt = (int)((uint32_t)w % (uint32_t)n_tiles);
             const int mt = PAIR ? 2 * unit + (int)rank : unit;  // PAIR: may be one past the last tile (no rows)
             // the tile's Jt scale rows (j0 .. j0 + Jt - 1, those below Ntc), BN each
+            const TileGeo geo = tile_geo(tl, mt);
             {
-                const int j0 = (mt / tl.n_cb) * tl.Jt;
-                const int rows = min(tl.Jt, Ntc - j0);
+                const int j0 = geo.j0;
+                const int rows = min(geo.Jt, Ntc - j0);
                 const int per_row = BN / 4;  // 16-byte pieces
                 for (int i = et; i < rows * per_row; i += 128) {
                     const int rr = i / per_row, cc = i % per_row;
@@ -560,10 +572,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
             }
             tc_fence_after();
             const int lr = q * 32 + lane;
-            int b, j;
-            tile_row(tl, mt, lr, b, j);
+            const int jl = lr / geo.Bg, bl = lr - jl * geo.Bg;
+            const int b = geo.b0 + bl, j = geo.j0 + jl;
             const bool valid = mt < tl.m_tiles && b < tl.B && j < Ntc;
-            const float4 *sc4 = reinterpret_cast<const float4 *>(sc_sm + (valid ? lr / tl.Bg : 0) * kScaleLd);
+            const float4 *sc4 = reinterpret_cast<const float4 *>(sc_sm + (valid ? jl : 0) * kScaleLd);
             // per 32-template block and per tile: the largest scaled |score|
             float *bm = blk_max + ((size_t)(valid ? b : 0) * Ntc + (valid ? j : 0)) * (T_pad / 32) +
                         (size_t)nt * (BN / 32);
@@ -610,15 +622,15 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
             // the warp, then across the warps in shared memory; one global
             // atomic per channel and tile
             unsigned bits = valid ? __float_as_uint(mx) : 0u;
-            for (int off = 16; off >= tl.Bg; off >>= 1) {
+            for (int off = 16; off >= geo.Bg; off >>= 1) {
                 const unsigned o = __shfl_xor_sync(0xffffffffu, bits, off);
                 bits = o > bits ? o : bits;
             }
             unsigned int *cm = sm.chan_max[eg];
-            if (tl.Bg >= 32 || lane < tl.Bg) atomicMax(cm + lr % tl.Bg, bits);
+            if (geo.Bg >= 32 || lane < geo.Bg) atomicMax(cm + bl, bits);
             epilogue_bar(bar_id);  // also: the scale rows are reloaded for the next item
-            if (et < tl.Bg) {
-                const int bc = (mt % tl.n_cb) * tl.Bg + et;
+            if (et < geo.Bg) {
+                const int bc = geo.b0 + et;
                 if (bc < tl.B) atomicMax(chmax + bc, cm[et]);
                 cm[et] = 0u;  // the next item adds to it after the barrier that follows its scale rows
             }
@@ -932,7 +944,14 @@ void shift_tc_scratch_free(ShiftTcScratch &x) {
 
 // Row tiling for B channels: Bg channels x Jt time centres per 128-row tile,
 // Jt as small as B allows (fewer lag chunks per tile), at most the time
-// centres (rounded up to a power of two).
+// centres (rounded up to a power of two).  Up to 16 channels past whole
+// blocks of 32 take tiles of 8 or 16 channels x 16 or 8 time centres instead
+// of one more block that is mostly padding, unless the time centres lie so
+// far apart that such a tile's windows see over a quarter more lags.  Row
+// build + GEMM in us per order, EEG-like grid: 33 channels 67.5 -> 49.2, 48
+// 68.3 -> 57.5, 66 97 -> 80; EMG-like, 2,048 samples: 160 -> 116, 167 -> 141,
+// 237 -> 197; the uneven EMG-like batch (66, 60, 73 and 57 channels) 25.1 ->
+// 21.3 ms.
 static RowTiling make_tiling(const ShiftPlan &sp, int B) {
     RowTiling t;
     int bg = 1;
@@ -944,7 +963,20 @@ static RowTiling make_tiling(const ShiftPlan &sp, int B) {
     t.B = B;
     t.Ntc = sp.Ntc;
     t.n_cb = (B + t.Bg - 1) / t.Bg;
-    t.m_tiles = ((sp.Ntc + t.Jt - 1) / t.Jt) * t.n_cb;
+    t.B_main = t.n_cb * t.Bg;
+    t.Jt2 = t.Bg2 = 0;
+    const int rest = B % 32;
+    if (B > 32 && t.Bg == 32 && rest > 0 && rest <= 16) {
+        const int bg2 = rest <= 8 ? 8 : 16, jt2 = kBM / bg2;
+        if (jt2 <= ntc2 && 4 * (int64_t)(jt2 - 1) * sp.S <= sp.L) {
+            t.n_cb = B / 32;
+            t.B_main = t.n_cb * 32;
+            t.Bg2 = bg2;
+            t.Jt2 = jt2;
+        }
+    }
+    t.m_main = ((sp.Ntc + t.Jt - 1) / t.Jt) * t.n_cb;
+    t.m_tiles = t.m_main + (t.Jt2 ? (sp.Ntc + t.Jt2 - 1) / t.Jt2 : 0);
     t.S = sp.S;
     t.L = sp.L;
     t.span0 = -sp.m_lo - sp.tc0;
@@ -990,7 +1022,7 @@ cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, Shift
 static int shift_tc_bn(const ShiftTc *s, const ShiftPlan &sp, const RowTiling &tl, bool pairs_allowed, int *stages,
                        size_t *smem, bool *pair, int *threads) {
     auto smem_for = [&](int bn, int stage_bytes, int *stg_out) {
-        const size_t sc = (size_t)tl.Jt * (bn + 4) * sizeof(float);
+        const size_t sc = (size_t)(tl.Jt > tl.Jt2 ? tl.Jt : tl.Jt2) * (bn + 4) * sizeof(float);
         int groups = 2;
         int stg = (int)((kSmemBudget - 2 * (int64_t)sc) / stage_bytes);
         if (stg < 4) {
