@@ -152,8 +152,8 @@ __device__ __forceinline__ float max_abs3(float a, float b, float c) {
 // the 32 rows an epilogue warp holds share one time centre (its scale loads
 // are broadcasts).  Rows of one tile see the window only over
 // L + (Jt - 1) S lags instead of Kt; outside them every product is zero.
-// A few channels past the whole blocks of 32 have tiles of their own behind
-// the others, from m_main on: Bg2 channels (B_main ..) x Jt2 time centres
+// A few channels past the whole blocks have tiles of their own behind the
+// others, from m_main on: Bg2 channels (B_main ..) x Jt2 time centres
 // (make_tiling).
 struct RowTiling {
     int B, Ntc, Jt, Bg, n_cb, m_tiles;
@@ -945,12 +945,12 @@ void shift_tc_scratch_free(ShiftTcScratch &x) {
 // Row tiling for B channels: Bg channels x Jt time centres per 128-row tile,
 // Jt as small as B allows (fewer lag chunks per tile), at most the time
 // centres (rounded up to a power of two).  Up to 16 channels past whole
-// blocks of 32 take tiles of 8 or 16 channels x 16 or 8 time centres instead
-// of one more block that is mostly padding, unless the time centres lie so
+// blocks of 32 (up to 8 past one block of 16) take tiles of 8 or 16 channels x
+// 16 or 8 time centres instead of one more block that is mostly padding, unless the time centres lie so
 // far apart that such a tile's windows see over a quarter more lags.  Row
-// build + GEMM in us per order, EEG-like grid: 33 channels 67.5 -> 49.2, 48
-// 68.3 -> 57.5, 66 97 -> 80; EMG-like, 2,048 samples: 160 -> 116, 167 -> 141,
-// 237 -> 197; the uneven EMG-like batch (66, 60, 73 and 57 channels) 25.1 ->
+// build + GEMM in us per order, EEG-like grid: 17 channels 41.0 -> 36.7, 33
+// 67.5 -> 49.2, 48 68.3 -> 57.5, 66 97 -> 80; EMG-like, 2,048 samples: 90 ->
+// 78, 160 -> 116, 167 -> 141, 237 -> 197; the uneven EMG-like batch (66, 60, 73 and 57 channels) 25.1 ->
 // 21.3 ms.
 static RowTiling make_tiling(const ShiftPlan &sp, int B) {
     RowTiling t;
@@ -965,12 +965,14 @@ static RowTiling make_tiling(const ShiftPlan &sp, int B) {
     t.n_cb = (B + t.Bg - 1) / t.Bg;
     t.B_main = t.n_cb * t.Bg;
     t.Jt2 = t.Bg2 = 0;
-    const int rest = B % 32;
-    if (B > 32 && t.Bg == 32 && rest > 0 && rest <= 16) {
+    const int block = B > 32 ? 32 : 16, rest = B % block;
+    if (B > 16 && t.Bg == 32 && rest > 0 && rest <= block / 2) {
         const int bg2 = rest <= 8 ? 8 : 16, jt2 = kBM / bg2;
         if (jt2 <= ntc2 && 4 * (int64_t)(jt2 - 1) * sp.S <= sp.L) {
-            t.n_cb = B / 32;
-            t.B_main = t.n_cb * 32;
+            t.Bg = block;
+            t.Jt = kBM / block;
+            t.n_cb = B / block;
+            t.B_main = t.n_cb * block;
             t.Bg2 = bg2;
             t.Jt2 = jt2;
         }

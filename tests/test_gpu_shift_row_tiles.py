@@ -51,7 +51,7 @@ def test_equals_fp32_template_search(name):
         want = run(act.ACT_SEARCH_SHIFT, 113)
         for pairs in (True, False):
             act.act_set_cta_pairs(h, pairs)
-            for B in (33, 113, 40, 41, 48, 49, 64, 65, 73, 80, 81, 32):
+            for B in (33, 113, 40, 41, 48, 49, 64, 65, 73, 80, 81, 32, 17, 24, 25):
                 for x, y in zip(run(act.ACT_SEARCH_SHIFT_BF16, B), want):
                     assert torch.equal(x, y[:B]), (pairs, B)
     finally:
