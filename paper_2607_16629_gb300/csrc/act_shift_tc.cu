@@ -1115,7 +1115,8 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
     // a programmatic dependent of the shifted-row build (set-up overlaps it)
     return launch_kernel(bn == 256 ? k_shift_gemm<256, false> : k_shift_gemm<128, false>, dim3(grid), dim3(threads),
                          smem, st, true, mapA, s->mapB[i], tl, n_tiles, s->nkc, stages, sp.T_pad,
-                         (const short2 *)sp.span, (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status, wait_ns);
+                         (const short2 *)sp.span, (const float *)sp.scaleT, x.tile_max, x.blk_max, x.chmax, status,
+                         wait_ns);
 }
 
 // Flags the items of every channel (first step of either resolve).
