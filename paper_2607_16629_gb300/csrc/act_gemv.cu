@@ -20,13 +20,15 @@ namespace act {
 // warp-shuffle reduction gives every lane the row's score; the warp keeps its
 // best |score| (lowest row on ties, rows are visited in increasing order),
 // the block combines its warps and issues one 64-bit atomicMax of the packed
-// key per channel.
-template <int NV>
+// key per channel.  With WRITE every score is stored instead (scores[row]):
+// the projection of one channel on up to kProjectOneBytes of rows.
+template <int NV, bool WRITE>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__ D, int64_t K, int Lp,
                                                        const float *__restrict__ R, int B,
                                                        const int *__restrict__ chlist,
                                                        const int *__restrict__ count_dev,
-                                                       unsigned long long *__restrict__ keys, int *status,
+                                                       unsigned long long *__restrict__ keys,
+                                                       float *__restrict__ scores, int *status,
                                                        unsigned long long wait_ns) {
     extern __shared__ __align__(128) float smem_r[];  // Lp floats
     __shared__ __align__(8) uint64_t bar;
@@ -108,19 +110,27 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
                 sa += __shfl_xor_sync(0xffffffffu, sa, off);
                 sb += __shfl_xor_sync(0xffffffffu, sb, off);
             }
-            float x = fabsf(sa);
-            if (x > best) {
-                best = x;
-                bidx = (uint32_t)row;
-            }
-            if (has2) {
-                x = fabsf(sb);
+            if (WRITE) {
+                if (lane == 0) {
+                    scores[row] = sa;
+                    if (has2) scores[row2] = sb;
+                }
+            } else {
+                float x = fabsf(sa);
                 if (x > best) {
                     best = x;
-                    bidx = (uint32_t)row2;
+                    bidx = (uint32_t)row;
+                }
+                if (has2) {
+                    x = fabsf(sb);
+                    if (x > best) {
+                        best = x;
+                        bidx = (uint32_t)row2;
+                    }
                 }
             }
         }
+        if (WRITE) return;  // one channel
         if (lane == 0) {
             red_s[wid] = best;
             red_i[wid] = bidx;
@@ -145,10 +155,11 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
 
 template <int NV>
 static cudaError_t gemv_instance(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
-                                 const int *count_dev, unsigned long long *keys, int *status, int grid_ctas,
-                                 unsigned long long wait_ns, cudaStream_t st, bool pdl) {
-    return launch_kernel(k_gemv<NV>, dim3(grid_ctas), dim3(kGemvThreads), (size_t)Lp * sizeof(float), st, pdl, D, K,
-                         Lp, R, B, chlist, count_dev, keys, status, wait_ns);
+                                 const int *count_dev, unsigned long long *keys, float *scores, int *status,
+                                 int grid_ctas, unsigned long long wait_ns, cudaStream_t st, bool pdl) {
+    return launch_kernel(scores ? k_gemv<NV, true> : k_gemv<NV, false>, dim3(grid_ctas), dim3(kGemvThreads),
+                         (size_t)Lp * sizeof(float), st, pdl, D, K, Lp, R, B, chlist, count_dev, keys, scores, status,
+                         wait_ns);
 }
 
 int gemv_ctas(int sm_count, int Lp) { return sm_count * gemv_max_ctas_per_sm(Lp); }
@@ -159,12 +170,12 @@ int gemv_max_ctas_per_sm(int Lp) {
     cudaError_t e = cudaErrorInvalidValue;
     const size_t smem = (size_t)Lp * sizeof(float);
     switch (nv) {
-        case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<1>, kGemvThreads, smem); break;
-        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<2>, kGemvThreads, smem); break;
-        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<3>, kGemvThreads, smem); break;
-        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<4>, kGemvThreads, smem); break;
-        case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<8>, kGemvThreads, smem); break;
-        case 16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<16>, kGemvThreads, smem); break;
+        case 1: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<1, false>, kGemvThreads, smem); break;
+        case 2: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<2, false>, kGemvThreads, smem); break;
+        case 3: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<3, false>, kGemvThreads, smem); break;
+        case 4: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<4, false>, kGemvThreads, smem); break;
+        case 8: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<8, false>, kGemvThreads, smem); break;
+        case 16: e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_gemv<16, false>, kGemvThreads, smem); break;
         default: break;
     }
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -172,12 +183,13 @@ int gemv_max_ctas_per_sm(int Lp) {
     return per_sm;
 }
 
-cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
-                               const int *count_dev, unsigned long long *keys, int *status, int grid_ctas,
-                               cudaStream_t st, unsigned long long wait_ns, bool pdl) {
+static cudaError_t launch_gemv(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
+                               const int *count_dev, unsigned long long *keys, float *scores, int *status,
+                               int grid_ctas, cudaStream_t st, unsigned long long wait_ns, bool pdl) {
 #define ACT_GEMV_CASE(NVV)                                                                                        \
     case NVV:                                                                                                     \
-        return gemv_instance<NVV>(D, K, Lp, R, B, chlist, count_dev, keys, status, grid_ctas, wait_ns, st, pdl);
+        return gemv_instance<NVV>(D, K, Lp, R, B, chlist, count_dev, keys, scores, status, grid_ctas, wait_ns, st, \
+                                  pdl);
     switch (Lp / 128) {
         ACT_GEMV_CASE(1)
         ACT_GEMV_CASE(2)
@@ -189,6 +201,18 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
             return cudaErrorInvalidValue;
     }
 #undef ACT_GEMV_CASE
+}
+
+cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
+                               const int *count_dev, unsigned long long *keys, int *status, int grid_ctas,
+                               cudaStream_t st, unsigned long long wait_ns, bool pdl) {
+    return launch_gemv(D, K, Lp, R, B, chlist, count_dev, keys, nullptr, status, grid_ctas, st, wait_ns, pdl);
+}
+
+cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, float *scores, int *status,
+                               int sm_count, cudaStream_t st, unsigned long long wait_ns) {
+    return launch_gemv(D, K, Lp, R, 1, nullptr, nullptr, nullptr, scores, status, gemv_ctas(sm_count, Lp), st, wait_ns,
+                       false);
 }
 
 }  // namespace act

@@ -134,7 +134,15 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
 cudaError_t launch_gemv_multi_argmax(const float *D, int64_t K, int Lp, const float *R, int B,
                                      unsigned long long *keys, int *status, int sm_count, cudaStream_t st,
                                      unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
-// Every score, scores[b * K + row], any number of channels.
+// Every score of one channel by the load-streaming GEMV.
+cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, float *scores, int *status,
+                               int sm_count, cudaStream_t st, unsigned long long wait_ns);
+// Every score, scores[b * K + row], any number of channels.  One channel takes
+// the load-streaming GEMV up to this many bytes of rows: us per call of it and
+// of the several-channel form at 17 MB 12.2 and 14.2, 72 MB (N = 300) 16.5 and
+// 20.6, 98 MB (N = 512) 27.7 and 24.7, 170 MB (N = 300) 33.0 and 39.4, 584 MB
+// 112 and 100, 4.3 GB 739 and 627.
+constexpr int64_t kProjectOneBytes = 256ll << 20;
 cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, int B, float *scores,
                            int *status, int sm_count, cudaStream_t st, unsigned long long wait_ns = kWaitLimitNs);
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
