@@ -491,15 +491,16 @@ act_status record_decompose(act_grid *g, WorkBuffers &w, int B, int P, act_searc
             kernels += 1;
         } else if (mode == ACT_SEARCH_SHIFT_BF16) {
             // programmatic dependents between kernel nodes only (not next to profiling events)
-            ACT_CK(launch_shift_tc_gemm(g->shift_tc, w.stc, g->shift, w.R, g->Lp, g->L, B, g->stats, g->status, st,
-                                        !profiling, g->wait_ns, g->cta_pairs));
+            ACT_CK(launch_shift_tc_gemm(g->shift_tc, w.stc, g->shift, w.R, g->Lp, g->L, B,
+                                        template_err_terms(g->L), g->stats, g->status, st, !profiling, g->wait_ns,
+                                        g->cta_pairs));
             if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
             ACT_CK(launch_shift_tc_resolve(g->shift_tc, w.stc, g->shift, w.R, g->Lp, g->L, B, w.keys, w.fb_list,
                                            w.fb_count, g->stats, g->status, st, !profiling, g->wait_ns));
             kernels += 5;
         } else if (bf16 && screens(g, w, B)) {
-            ACT_CK(launch_shift_tc_gemm(g->screen_tc, w.stc, g->screen, w.R, g->Lp, g->L, B, g->stats, g->status, st,
-                                        !profiling, g->wait_ns, g->cta_pairs));
+            ACT_CK(launch_shift_tc_gemm(g->screen_tc, w.stc, g->screen, w.R, g->Lp, g->L, B, row_err_terms(g->L),
+                                        g->stats, g->status, st, !profiling, g->wait_ns, g->cta_pairs));
             if (profiling) ACT_CK(cudaEventRecordWithFlags(ev[1], st, cudaEventRecordExternal));
             ACT_CK(launch_shift_tc_resolve_rows(g->screen_tc, w.stc, g->screen, g->d32, g->K, w.R, g->Lp, g->L, B,
                                                 w.keys, w.fb_list, w.fb_count, g->stats, g->status, g->gemv_grid, st,
@@ -1095,7 +1096,8 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
                     e = cudaMemsetAsync(g->w.fb_count, 0, 2 * sizeof(int), st);
                     if (e == cudaSuccess)
                         e = launch_shift_tc_gemm(g->screen_tc, g->w.stc, g->screen, g->w.R, g->Lp, g->L, channels,
-                                                 g->stats, g->status, st, false, g->wait_ns, g->cta_pairs);
+                                                 row_err_terms(g->L), g->stats, g->status, st, false, g->wait_ns,
+                                                 g->cta_pairs);
                     if (e == cudaSuccess)
                         e = launch_shift_tc_resolve_rows(g->screen_tc, g->w.stc, g->screen, g->d32, g->K, g->w.R,
                                                          g->Lp, g->L, channels, g->w.keys, g->w.fb_list, g->w.fb_count,

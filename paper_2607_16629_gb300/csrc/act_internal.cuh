@@ -298,7 +298,7 @@ struct ShiftTcScratch {
     float *blk_max = nullptr;       // [rows][T_pad / 32] maxima per 32-template block
     int *items = nullptr;           // [B_cap * 1024][2] flagged (channel, item) pairs
     __nv_bfloat16 *X = nullptr;     // [rows_alloc][Kt] shifted BF16 residual rows
-    double2 *chan_norm = nullptr;   // [B_cap] |r|, |bf16(r) - r|
+    float *bound = nullptr;         // [B_cap] error bound of the screened scores, this order
     unsigned int *chmax = nullptr;  // [B_cap] largest tile maximum (float bits)
     int *chcount = nullptr;         // [B_cap] items flagged this order
     int B_cap = 0;
@@ -324,9 +324,17 @@ void shift_tc_scratch_free(ShiftTcScratch &x);
 // Whether a B-channel launch runs the paired-SM GEMM.
 bool shift_tc_uses_pairs(const ShiftTc *s, const ShiftPlan &sp, int B, bool pairs_allowed);
 // pairs_allowed: the paired-SM GEMM (cta_group::2) may be chosen where it applies.
+// err_terms: the roundings of the score that the flagged items are resolved
+// by, over its L products: template_err_terms before launch_shift_tc_resolve
+// (the sum, the scale, the final product), row_err_terms before
+// launch_shift_tc_resolve_rows (the GEMV's sum and the row's own: the
+// template's sample times the FP32 scale, both rounded).
+constexpr int template_err_terms(int L) { return L + 4; }
+constexpr int row_err_terms(int L) { return L + 8; }
 cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, const float *R,
-                                 int Lp, int L, int B, long long *stats, int *status, cudaStream_t st, bool pdl = false,
-                                 unsigned long long wait_ns = kWaitLimitNs, bool pairs_allowed = true);
+                                 int Lp, int L, int B, int err_terms, long long *stats, int *status, cudaStream_t st,
+                                 bool pdl = false, unsigned long long wait_ns = kWaitLimitNs,
+                                 bool pairs_allowed = true);
 cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, const float *R,
                                     int Lp, int L, int B, unsigned long long *keys, int *fb_list, int *counters,
                                     long long *stats, int *status, cudaStream_t st, bool pdl = false,

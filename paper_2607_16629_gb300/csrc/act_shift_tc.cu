@@ -231,11 +231,27 @@ __device__ __forceinline__ void item_steps(short2 rows, short2 tpls, int &lo, in
 // o = S jj + kk - k0, are one aligned 16-byte load from copy o & 7.  Padding
 // rows (b >= B or j >= Ntc) are not written (the GEMM's epilogue ignores
 // them).  Block (0, b) also prepares channel b's selection for this order:
-// |r| and |bf16(r) - r| (for the error bound), the channel maximum and item
-// count cleared.
+// the error bound of its scores (k_shift_flag), the channel maximum and item
+// count cleared.  The bound is formed here because its residual sums are, and
+// its FP64 steps take a warp that few channels leave without rows; the flag
+// kernel reads it, as all that earlier kernels write, behind its own wait.
+//
+// With s the exact score, f the FP32 search's score and h the tensor-core
+// score of an atom,
+//   |f - s| <= eps_r = err_terms 2^-23 |r|
+// (template search: one FP32 chain of L products, the FP32 scale and the
+// final product; a stored row: the GEMV's sum and the row's own two
+// roundings), and
+//   |h - s| <= delta = (1 + 1e-5) [eps_u (|r| + |dr|) + |dr|
+//                                  + Kt 2^-23 (1 + eps_u)(|r| + |dr|)]
+// (eps_u = largest |u~ - u| / |u| over the atoms' windows, u~ = the BF16
+// template as multiplied, zero outside its tile's span; dr =
+// bf16(r) - r, the Kt term bounds FP32 accumulation in the tensor core, the
+// factor the scale product).  bound = 2 delta + 2 eps_r, rounded up.
 __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__restrict__ R, int Lp, int tc0,
                                                     int m_lo, int Kt, int RJ, int KSEG, int n_seg, int span_pad,
-                                                    __nv_bfloat16 *__restrict__ X, double2 *__restrict__ chan_norm,
+                                                    int err_terms, const unsigned int *__restrict__ eps_bits,
+                                                    __nv_bfloat16 *__restrict__ X, float *__restrict__ bound,
                                                     unsigned int *__restrict__ chmax, int *__restrict__ chcount,
                                                     long long *__restrict__ stats) {
     extern __shared__ __align__(16) uint8_t rows_raw[];
@@ -249,6 +265,7 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
     const int k0 = seg * KSEG, k1 = min(Kt, k0 + KSEG);
     const int L = t.L, S = t.S;
     const float *r = R + (size_t)b * Lp;
+    float te = 0.0f, tde = 0.0f;  // block (0, b): |r|^2 and |bf16(r) - r|^2
     if (blockIdx.x == 0) {
         // FP32 sums of at most 2048 squares are within 2048 * 2^-24 < 1.3e-4
         // (relative) of the exact ones: inflated by 1e-3 they bound them
@@ -259,10 +276,9 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
             e = fmaf(x, x, e);
             de = fmaf(d, d, de);
         }
-        const float te = block_sum(e, sh);
-        const float tde = block_sum(de, sh);
+        te = block_sum(e, sh);
+        tde = block_sum(de, sh);
         if (threadIdx.x == 0) {
-            chan_norm[b] = make_double2(sqrt((double)te * (1.0 + 1e-3)), sqrt((double)tde * (1.0 + 1e-3)));
             chmax[b] = 0u;
             chcount[b] = 0;
             atomicAdd((unsigned long long *)&stats[0], 1ull);
@@ -304,6 +320,16 @@ __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__
     __syncthreads();
     const uint4 *cp16 = reinterpret_cast<const uint4 *>(rows_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // (block (0, b) always gets here: it has rows and lags)
+    if (blockIdx.x == 0 && threadIdx.x == blockDim.x - 32) {
+        const double rn = sqrt((double)te * (1.0 + 1e-3)), drn = sqrt((double)tde * (1.0 + 1e-3));
+        const double eps_u = (double)__uint_as_float(*eps_bits);
+        const double rr = rn + drn;
+        const double ulp = 1.1920928955078125e-07;  // 2^-23
+        const double delta = (1.0 + 1e-5) * (eps_u * rr + drn + (double)Kt * ulp * (1.0 + eps_u) * rr);
+        const double eps_r = (double)err_terms * ulp * rn;
+        bound[b] = __double2float_ru(2.0 * delta + 2.0 * eps_r);
+    }
     const int c0 = k0 >> 3, c1 = k1 >> 3;
     // this channel's tiles: every n_cb-th from first on
     const bool main = b < t.B_main;
@@ -657,50 +683,24 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 }
 
 // Item selection for channel b (blockIdx.y; blockIdx.x slices its entries).
-// With s the exact score, f the
-// FP32 template search's score and h the tensor-core score of an atom,
-//   |f - s| <= eps_r = (L + 4) 2^-23 |r|
-// (one FP32 chain of L products, the FP32 scale and the final product), and
-//   |h - s| <= delta = (1 + 1e-5) [eps_u (|r| + |dr|) + |dr|
-//                                  + Kt 2^-23 (1 + eps_u)(|r| + |dr|)]
-// (eps_u = largest |u~ - u| / |u| over the atoms' windows, u~ = the BF16
-// template as multiplied, zero outside its tile's span; dr =
-// bf16(r) - r, the Kt term bounds FP32 accumulation in the tensor core, the
-// factor the scale product).  As for the dense BF16 search, the FP32 argmax
-// lies in an item whose largest |h| is >= hmax - 2 delta - 2 eps_r.
-// max_items: flagged items per channel before the full FP32 search;
-// err_terms: the rounding terms of that search's score (eps_r).
-__global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int Kt, int err_terms, int max_items,
-                                                    const float *tile_max, const float *blk_max,
-                                                    const double2 *__restrict__ chan_norm, const unsigned int *chmax,
-                                                    const unsigned int *__restrict__ eps_bits,
-                                                    const int *__restrict__ blk_order, int *__restrict__ chcount,
-                                                    int *__restrict__ fb_list,
+// With bound[b] = 2 delta + 2 eps_r (k_shift_rows), as for the dense BF16
+// search, the FP32 argmax lies in an item whose largest |h| is
+// >= hmax - bound[b].  max_items: flagged items per channel before the full
+// FP32 search.
+__global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int max_items,
+                                                    const float *tile_max, const float *blk_max, const float *bound,
+                                                    const unsigned int *chmax, const int *__restrict__ blk_order,
+                                                    int *__restrict__ chcount, int *__restrict__ fb_list,
                                                     int *__restrict__ counters, int *__restrict__ items,
                                                     long long *__restrict__ stats) {
     const int b = blockIdx.y;
-    __shared__ float bound_sh;
-    // The bound, in FP64 by one thread, while the GEMM still runs: it lets
-    // this kernel launch only after its own wait for the rows kernel that
-    // wrote the norms.  One FP32 difference is left behind the wait.
-    if (threadIdx.x == 0) {
-        const double2 nr = chan_norm[b];
-        const double rn = nr.x, drn = nr.y;
-        const double eps_u = (double)__uint_as_float(*eps_bits);
-        const double rr = rn + drn;
-        const double ulp = 1.1920928955078125e-07;  // 2^-23
-        const double delta = (1.0 + 1e-5) * (eps_u * rr + drn + (double)Kt * ulp * (1.0 + eps_u) * rr);
-        const double eps_r = (double)err_terms * ulp * rn;
-        bound_sh = __double2float_ru(2.0 * delta + 2.0 * eps_r);
-    }
-    __syncthreads();
-    const float bound = bound_sh;
-    asm volatile("griddepcontrol.wait;" ::: "memory");  // the GEMM's maxima
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the rows kernel's bound, the GEMM's maxima
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // the threshold rounded down: a superset of the items
-    // (what the GEMM writes is read through pointers without __restrict__: a
-    // load that the compiler may take for constant could move before the wait)
-    const float thr_f = __fsub_rd(__uint_as_float(*(const volatile unsigned int *)&chmax[b]), bound);
+    // (what earlier kernels write is read through pointers without
+    // __restrict__: a load that the compiler may take for constant could move
+    // before the wait)
+    const float thr_f = __fsub_rd(__uint_as_float(chmax[b]), bound[b]);
     // scan the tile maxima; a tile at or above the threshold is narrowed to
     // its 32-template blocks at or above it (the items: j * n_blocks + block)
     const float *tm = tile_max + (size_t)b * Ntc * n_tiles;
@@ -936,7 +936,7 @@ void shift_tc_scratch_free(ShiftTcScratch &x) {
     if (x.blk_max) cudaFree(x.blk_max);
     if (x.items) cudaFree(x.items);
     if (x.X) cudaFree(x.X);
-    if (x.chan_norm) cudaFree(x.chan_norm);
+    if (x.bound) cudaFree(x.bound);
     if (x.chmax) cudaFree(x.chmax);
     if (x.chcount) cudaFree(x.chcount);
     x = ShiftTcScratch();
@@ -1002,7 +1002,7 @@ cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, Shift
     if (e == cudaSuccess) e = dev_alloc((void **)&x.items, sizeof(int) * 2 * (size_t)B * kMaxItems);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.X, sizeof(__nv_bfloat16) * (size_t)rows_alloc * sp.Kt);
     if (e == cudaSuccess) e = cudaMemset(x.X, 0, sizeof(__nv_bfloat16) * (size_t)rows_alloc * sp.Kt);
-    if (e == cudaSuccess) e = dev_alloc((void **)&x.chan_norm, sizeof(double2) * (size_t)B);
+    if (e == cudaSuccess) e = dev_alloc((void **)&x.bound, sizeof(float) * (size_t)B);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.chmax, sizeof(unsigned int) * (size_t)B);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.chcount, sizeof(int) * (size_t)B);
     if (e != cudaSuccess) {
@@ -1070,8 +1070,8 @@ bool shift_tc_uses_pairs(const ShiftTc *s, const ShiftPlan &sp, int B, bool pair
 }
 
 cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, const float *R,
-                                 int Lp, int L, int B, long long *stats, int *status, cudaStream_t st, bool pdl,
-                                 unsigned long long wait_ns, bool pairs_allowed) {
+                                 int Lp, int L, int B, int err_terms, long long *stats, int *status, cudaStream_t st,
+                                 bool pdl, unsigned long long wait_ns, bool pairs_allowed) {
     if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
     const RowTiling tl = make_tiling(sp, B);
     // rows per block: up to 16, fewer when that leaves SMs idle (at least 4);
@@ -1089,8 +1089,8 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
     const int64_t gx = (int64_t)((sp.Ntc + RJ - 1) / RJ) * n_seg;
     if (gx >= ((int64_t)1 << 31) || B > 65535) return cudaErrorInvalidValue;
     cudaError_t e = launch_kernel(k_shift_rows, dim3((unsigned)gx, B), dim3(256), rows_smem, st, pdl, tl, R, Lp,
-                                  sp.tc0, sp.m_lo, sp.Kt, RJ, KSEG, n_seg, span_pad, x.X, x.chan_norm, x.chmax,
-                                  x.chcount, stats);
+                                  sp.tc0, sp.m_lo, sp.Kt, RJ, KSEG, n_seg, span_pad, err_terms,
+                                  (const unsigned int *)sp.eps_bits, x.X, x.bound, x.chmax, x.chcount, stats);
     if (e != cudaSuccess) return e;
     const int m_tiles = tl.m_tiles;
     CUtensorMap mapA;
@@ -1120,9 +1120,8 @@ cudaError_t launch_shift_tc_gemm(const ShiftTc *s, const ShiftTcScratch &x, cons
 }
 
 // Flags the items of every channel (first step of either resolve).
-static cudaError_t launch_flag(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, int B, int err_terms,
-                               int max_items, int *fb_list, int *counters, long long *stats, cudaStream_t st,
-                               bool pdl) {
+static cudaError_t launch_flag(const ShiftTc *s, const ShiftTcScratch &x, const ShiftPlan &sp, int B, int max_items,
+                               int *fb_list, int *counters, long long *stats, cudaStream_t st, bool pdl) {
     const RowTiling tl = make_tiling(sp, B);
     int stages = 0, threads = 0;
     size_t smem = 0;
@@ -1133,10 +1132,9 @@ static cudaError_t launch_flag(const ShiftTc *s, const ShiftTcScratch &x, const 
     int slices = (entries + 255) / 256;
     const int max_slices = (4 * s->sm_count + B - 1) / B;
     if (slices > max_slices) slices = max_slices;
-    return launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32, sp.Kt,
-                         err_terms, max_items, (const float *)x.tile_max, (const float *)x.blk_max,
-                         (const double2 *)x.chan_norm, (const unsigned int *)x.chmax,
-                         (const unsigned int *)sp.eps_bits, (const int *)sp.blk_order, x.chcount, fb_list, counters,
+    return launch_kernel(k_shift_flag, dim3(slices, B), dim3(256), 0, st, pdl, sp.Ntc, n_tiles, bn / 32, max_items,
+                         (const float *)x.tile_max, (const float *)x.blk_max, (const float *)x.bound,
+                         (const unsigned int *)x.chmax, (const int *)sp.blk_order, x.chcount, fb_list, counters,
                          x.items, stats);
 }
 
@@ -1145,7 +1143,7 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
                                     long long *stats, int *status, cudaStream_t st, bool pdl,
                                     unsigned long long wait_ns) {
     if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
-    cudaError_t e = launch_flag(s, x, sp, B, L + 4, kMaxItems, fb_list, counters, stats, st, pdl);
+    cudaError_t e = launch_flag(s, x, sp, B, kMaxItems, fb_list, counters, stats, st, pdl);
     if (e != cudaSuccess) return e;
     const auto &rc = s->rescan[B <= kRescanFewChannels ? 0 : 1];
     e = launch_kernel(k_shift_rescan, dim3(s->sm_count * rc.blocks_per_sm), dim3(rc.warps * 32), rc.smem, st, true,
@@ -1166,9 +1164,7 @@ cudaError_t launch_shift_tc_resolve_rows(const ShiftTc *s, const ShiftTcScratch 
                                          int *status, int gemv_grid, cudaStream_t st, bool pdl,
                                          unsigned long long wait_ns) {
     if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
-    // |f - s| of the GEMV: its sum's rounding, and the row's own (the
-    // template's sample times the FP32 scale, both rounded) beside it
-    cudaError_t e = launch_flag(s, x, sp, B, L + 8, kMaxRowItems, fb_list, counters, stats, st, pdl);
+    cudaError_t e = launch_flag(s, x, sp, B, kMaxRowItems, fb_list, counters, stats, st, pdl);
     if (e == cudaSuccess)
         e = launch_rows_rescan(D32, K, Lp, R, x.items, counters, keys, sp.T, sp.T_pad / 32, s->sm_count, st);
     if (e != cudaSuccess) return e;
