@@ -361,8 +361,8 @@ __global__ void __launch_bounds__(256) k_select(int64_t ntiles, int bpt, const f
 // into keys[b] with the packed atomicMax (largest |score|, then lowest
 // index).  One block of 8 warps per pair.
 __global__ void __launch_bounds__(256) k_rescan(const float *__restrict__ D32, int64_t K, int Lp, int tile_atoms,
-                                                const float *__restrict__ R, const int *pairs, const int *counters,
-                                                unsigned long long *__restrict__ keys, int T, int n_blocks) {
+                                                const float *R, const int *pairs, const int *counters,
+                                                unsigned long long *keys, int T, int n_blocks) {
     // (a programmatic dependent of the kernel that flagged the items, where
     // the template GEMM screens: their number and the items are read without
     // __restrict__, which would let those loads move ahead of the wait; what

@@ -24,11 +24,8 @@ namespace act {
 // the projection of one channel on up to kProjectOneBytes of rows.
 template <int NV, bool WRITE>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__ D, int64_t K, int Lp,
-                                                       const float *__restrict__ R, int B,
-                                                       const int *__restrict__ chlist,
-                                                       const int *__restrict__ count_dev,
-                                                       unsigned long long *__restrict__ keys,
-                                                       float *__restrict__ scores, int *status,
+                                                       const float *R, int B, const int *chlist, const int *count_dev,
+                                                       unsigned long long *keys, float *scores, int *status,
                                                        unsigned long long wait_ns) {
     extern __shared__ __align__(128) float smem_r[];  // Lp floats
     __shared__ __align__(8) uint64_t bar;

@@ -73,7 +73,7 @@ __device__ __forceinline__ float warp_sum_32(float (&v)[32], int lane) {
 template <int N8, int N4, bool WRITE_SCORES>
 __global__ void __launch_bounds__(kMultiThreads, 1)
     k_gemv_multi(const float *__restrict__ D, int64_t K, int Lp, const float *R, int ng,
-                 unsigned long long *__restrict__ keys, float *__restrict__ scores, int tiles, int stages, int *status,
+                 unsigned long long *keys, float *scores, int tiles, int stages, int *status,
                  unsigned long long wait_ns) {
     constexpr int NCH = 8 * N8 + 4 * N4, G = N8 + N4;
     extern __shared__ __align__(128) float sm[];  // stages, then [NCH][Lp] residuals

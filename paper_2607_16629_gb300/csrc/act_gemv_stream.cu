@@ -43,9 +43,9 @@ StreamShape stream_shape(int Lp) {
 
 template <int NV>
 __global__ void __launch_bounds__(kStreamThreads, 1)
-    k_gemv_stream(const float *__restrict__ D, int64_t K, int Lp, const float *__restrict__ R, int B,
-                  const int *__restrict__ chlist, const int *__restrict__ count_dev,
-                  unsigned long long *__restrict__ keys, int rows_per_chunk, int stages, int *status,
+    k_gemv_stream(const float *__restrict__ D, int64_t K, int Lp, const float *R, int B,
+                  const int *chlist, const int *count_dev,
+                  unsigned long long *keys, int rows_per_chunk, int stages, int *status,
                   unsigned long long wait_ns) {
     extern __shared__ __align__(128) float sm[];  // stages x rows_per_chunk x Lp
     __shared__ __align__(8) uint64_t full[kMaxStreamStages], empty[kMaxStreamStages];

@@ -17,8 +17,10 @@ namespace act {
 // Launch on st; with pdl, as a programmatic dependent of the previous kernel
 // in the stream (it may start while that kernel runs, and must execute
 // griddepcontrol.wait in every CTA before it touches what that kernel
-// writes and before it exits).  Between a kernel and an event node (or at a
-// stream's first kernel) pdl has to be false.
+// writes and before it exits; of its pointers only those to what is constant
+// since the dictionary's build are __restrict__: accesses through such a
+// pointer may be moved ahead of the wait).  Between a kernel and an event node
+// (or at a stream's first kernel) pdl has to be false.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                  bool pdl, Args... args) {

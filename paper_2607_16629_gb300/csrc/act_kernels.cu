@@ -168,11 +168,10 @@ cudaError_t launch_init(const float *sig, int B, int L, int Lp, float *R, __nv_b
 // from its flat index, the key cleared for the next order.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kUpdateThreads + 32) k_update(const float *__restrict__ D32, int Lp, int L,
-                                                           float *__restrict__ R, __nv_bfloat16 *__restrict__ R16,
-                                                           int Lb, unsigned long long *__restrict__ keys,
-                                                           GridAxes ax, int k, int P,
-                                                           act_atom *__restrict__ atoms, float *__restrict__ coefs,
-                                                           double *__restrict__ energy, int *fb_count) {
+                                                           float *R, __nv_bfloat16 *R16, int Lb,
+                                                           unsigned long long *keys, GridAxes ax, int k, int P,
+                                                           act_atom *atoms, float *coefs, double *energy,
+                                                           int *fb_count) {
     __shared__ float shf[32];
     __shared__ ff shp[32];
     // launched as a programmatic dependent of the search: every block waits

@@ -51,7 +51,7 @@ __device__ __forceinline__ uint64_t lem_counter(int channel, int order, int axis
 constexpr int kLhsThreads = 512;
 
 __global__ void __launch_bounds__(kLhsThreads) k_lem_lhs(int n, int log2b, LemBox box, uint64_t seed, int order,
-                                                        int cap, double *__restrict__ cand, int *__restrict__ ncand) {
+                                                        int cap, double *cand, int *ncand) {
     // The samples do not depend on the residual: this kernel runs beside the
     // update of the order before it.  Nothing else reads or writes cand and
     // ncand by then (the update's own predecessors have completed before it
@@ -188,7 +188,7 @@ __device__ __forceinline__ uint64_t cycles64(double v) {
 __global__ void __launch_bounds__(kLemThreads) k_lem_screen(int cap, int level, LemBox box, LemLevel lev, int top_k,
                                                            const double *kept, const int *nkept, double *cand,
                                                            int *ncand, const float *R, int Lp, int L, double inv_fs,
-                                                           float2 *__restrict__ screen) {
+                                                           float2 *screen) {
     // (no __restrict__ on what earlier kernels write: loads through it may
     // move ahead of the wait)
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -485,9 +485,9 @@ __device__ int pick_top(PickShared &sm, int k, int entries, const unsigned long 
 __global__ void __launch_bounds__(kPickThreads) k_lem_pick(int cap, int k, int level_candidates,
                                                           const double *cand, const int *ncand, int per, int *nkept,
                                                           const float2 *screen, const float *R, int Lp, int L,
-                                                          double inv_fs, double *__restrict__ score,
-                                                          double *__restrict__ kept,
-                                                          double *__restrict__ kept_score) {
+                                                          double inv_fs, double *score,
+                                                          double *kept,
+                                                          double *kept_score) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr unsigned long long kAbs = 0x7fffffffffffffffull, kInf = 0x7ff0000000000000ull;

@@ -624,13 +624,13 @@ __global__ void __launch_bounds__(kBfgsThreads) k_refine(GridAxes ax, RefineBox 
 // the dictionary generator (float-float phase, chirp_sample_ff), formed once
 // into registers; |u|^2 is a float-float sum, c = <g, r> an FP32 block sum,
 // |r|^2 an FP64 sum.
-__global__ void __launch_bounds__(kRefineThreads) k_update_refined(int Lp, float *__restrict__ R,
-                                                                  __nv_bfloat16 *__restrict__ R16, int Lb,
-                                                                  unsigned long long *__restrict__ keys, GridAxes ax,
+__global__ void __launch_bounds__(kRefineThreads) k_update_refined(int Lp, float *R,
+                                                                  __nv_bfloat16 *R16, int Lb,
+                                                                  unsigned long long *keys, GridAxes ax,
                                                                   const double *theta, int k, int P,
-                                                                  act_atom *__restrict__ atoms,
-                                                                  float *__restrict__ coefs,
-                                                                  double *__restrict__ energy, int *fb_count) {
+                                                                  act_atom *atoms,
+                                                                  float *coefs,
+                                                                  double *energy, int *fb_count) {
     // In the hierarchical search (no keys) a programmatic dependent of the
     // refinement, and the next order's samples are drawn beside it; a template
     // search is not launched early (32 radar-like channels 3,625 -> 3,638 us

@@ -536,10 +536,8 @@ __global__ void __launch_bounds__(kShiftMaxThreads) k_shift_search(ShiftArgs A) 
 __global__ void __launch_bounds__(kShiftUpdateThreads) k_shift_update(const float *__restrict__ tpl,
                                                                      const float *__restrict__ scale,
                                                      int S, int Sa, int rows, int NtcP, int T, GridAxes ax, int Lp,
-                                                     float *__restrict__ R, unsigned long long *__restrict__ keys,
-                                                     int k, int P, act_atom *__restrict__ atoms,
-                                                     float *__restrict__ coefs, double *__restrict__ energy,
-                                                     int *__restrict__ counters) {
+                                                     float *R, unsigned long long *keys, int k, int P, act_atom *atoms,
+                                                     float *coefs, double *energy, int *counters) {
     // with a programmatic launch: the keys of the search before are read
     // only after it completes; the next search may launch now
     asm volatile("griddepcontrol.wait;" ::: "memory");

@@ -248,12 +248,12 @@ __device__ __forceinline__ void item_steps(short2 rows, short2 tpls, int &lo, in
 // template as multiplied, zero outside its tile's span; dr =
 // bf16(r) - r, the Kt term bounds FP32 accumulation in the tensor core, the
 // factor the scale product).  bound = 2 delta + 2 eps_r, rounded up.
-__global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *__restrict__ R, int Lp, int tc0,
+__global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *R, int Lp, int tc0,
                                                     int m_lo, int Kt, int RJ, int KSEG, int n_seg, int span_pad,
                                                     int err_terms, const unsigned int *__restrict__ eps_bits,
-                                                    __nv_bfloat16 *__restrict__ X, float *__restrict__ bound,
-                                                    unsigned int *__restrict__ chmax, int *__restrict__ chcount,
-                                                    long long *__restrict__ stats) {
+                                                    __nv_bfloat16 *X, float *bound,
+                                                    unsigned int *chmax, int *chcount,
+                                                    long long *stats) {
     extern __shared__ __align__(16) uint8_t rows_raw[];
     __shared__ float sh[32];
     // a programmatic dependent of the previous kernel (the residual update):
@@ -364,8 +364,8 @@ template <int BN, bool PAIR>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     k_shift_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowTiling tl,
                  int n_tiles, int nkc, int stages, int T_pad, const short2 *__restrict__ span,
-                 const float *__restrict__ scaleT, float *__restrict__ tile_max, float *__restrict__ blk_max,
-                 unsigned int *__restrict__ chmax,
+                 const float *__restrict__ scaleT, float *tile_max, float *blk_max,
+                 unsigned int *chmax,
                  int *status, unsigned long long wait_ns) {
     // shared memory: stages, then the item's scales [Jt][BN + 4] (the +4
     // floats of padding spread the Jt rows a warp reads over the banks)
@@ -690,9 +690,9 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int max_items,
                                                     const float *tile_max, const float *blk_max, const float *bound,
                                                     const unsigned int *chmax, const int *__restrict__ blk_order,
-                                                    int *__restrict__ chcount, int *__restrict__ fb_list,
-                                                    int *__restrict__ counters, int *__restrict__ items,
-                                                    long long *__restrict__ stats) {
+                                                    int *chcount, int *fb_list,
+                                                    int *counters, int *items,
+                                                    long long *stats) {
     const int b = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the rows kernel's bound, the GEMM's maxima
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bp
 __global__ void __launch_bounds__(kRescanWarps * 32) k_shift_rescan(
     const float *__restrict__ tpl, const float *__restrict__ scale, int S, int Sa, int P, int rows, int NtcP,
     int Ntc, int T, int n_blocks, int Lp, int L, const float *R, const int2 *items, int64_t max_tasks, int nb,
-    const int *counters, unsigned long long *__restrict__ keys, int *status,
+    const int *counters, unsigned long long *keys, int *status,
     unsigned long long wait_ns) {
     extern __shared__ __align__(128) float sm[];  // per warp: the residual [Lp], then nb x [P][32] rows
     __shared__ __align__(8) uint64_t bar[kRescanWarps][kRescanBufs];

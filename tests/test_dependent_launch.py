@@ -76,3 +76,10 @@ def test_nothing_earlier_kernels_write_is_used_before_the_wait(name, pointers, b
     if name == "k_shift_search":  # its pointers come in a struct; what selects the form is its own argument
         used = set(re.findall(r"\bA\.(R|keys|scores|chlist|count_dev|status)\b", before))
         assert used <= {"count_dev"} and "*A.count_dev" not in before
+
+
+@pytest.mark.parametrize("name,pointers,body", KERNELS, ids=[k[0] for k in KERNELS])
+def test_only_constants_are_restrict(name, pointers, body):
+    """An access through a __restrict__ pointer may be moved ahead of the
+    wait (the compiler has done so with a queue's length)."""
+    assert [p for p, decl in pointers.items() if "__restrict__" in decl and p not in CONSTANT] == []
