@@ -743,6 +743,8 @@ static cudaError_t make_templates(const act_grid *g, ShiftPlan &sp, unsigned lon
         if (e == cudaSuccess) e = dev_alloc((void **)&sp.blk_order, sizeof(int) * order.size());
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(sp.blk_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, st);
+        // (the table is pageable memory of this call's own: the copy has to be over before it goes)
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.scaleT, 0, bst, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.eps_bits, 0, sizeof(unsigned int), st);
     }
