@@ -845,6 +845,15 @@ constexpr int kStaticReserve = 8192;
 static_assert(sizeof(Smem) + 256 <= kStaticReserve, "static shared memory above its reserve");
 constexpr int kSmemBudget = 232448 - kStaticReserve - 1024;
 
+// Dynamic shared memory of a rescore block.  It has none of the GEMM's tables
+// beside it, so its limit does not follow theirs: one warp with two buffers
+// takes exactly these bytes at time centres one sample apart and windows of
+// 849 to 864 samples, and two samples apart and 1,665 to 1,696, the longest
+// windows that the tensor-core search serves at those steps.
+constexpr int kRescanSmem = 225280;
+static_assert(kRescanSmem + (int)sizeof(uint64_t) * kRescanWarps * kRescanBufs + 1024 <= 232448,
+              "a rescore block's shared memory");
+
 }  // namespace
 
 struct ShiftTc {
@@ -907,12 +916,12 @@ cudaError_t shift_tc_prepare(ShiftTc **out, const ShiftPlan &sp, int sm_count) {
         while (i == 0 && nb < sp.Sa && nb < kRescanBufs && res + (nb + 1) * buf <= (size_t)kRescanFewBytes) ++nb;
         const size_t per_warp = res + nb * buf;
         int rw = kRescanWarps;
-        while (rw > 1 && rw * per_warp > (size_t)kSmemBudget) --rw;
+        while (rw > 1 && rw * per_warp > (size_t)kRescanSmem) --rw;
         s->rescan[i].bufs = nb;
         s->rescan[i].warps = rw;
         s->rescan[i].smem = rw * per_warp;
         most = s->rescan[i].smem > most ? s->rescan[i].smem : most;
-        if (e == cudaSuccess && s->rescan[i].smem > (size_t)kSmemBudget) e = cudaErrorNotSupported;
+        if (e == cudaSuccess && s->rescan[i].smem > (size_t)kRescanSmem) e = cudaErrorNotSupported;
     }
     if (e == cudaSuccess) e = allow_max_smem((const void *)k_shift_rescan, most);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
