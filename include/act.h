@@ -365,12 +365,11 @@ ACT_API act_status act_chirplet_score(int32_t n_samples, double fs, const double
  * fastest, and returns its time per order in *best_ms (may be NULL).
  * Candidates: with one channel, resident CTAs per SM of the load-streaming
  * FP32 GEMV (1..4, as occupancy allows) and the bulk-copy streaming GEMV
- * (several channels have one FP32 form, which is only timed: a call with one
- * channel then takes the load-streaming GEMV); when the grid holds a BF16
- * dictionary, tile width (128 or 256 atoms) x pipeline depth (2 .. what fits
- * in shared memory) of the tensor-core GEMM over its rows, each timed with
- * its tile selection and rescan (where templates screen, that search is only
- * timed); with an ACT_DICT_RECOMPUTE build, every valid (lags per thread,
+ * (several channels have one FP32 form, which is only timed: the one-channel
+ * form in use stays as it is); when the grid holds a BF16 dictionary, tile
+ * width (128 or 256 atoms) x pipeline depth (2 .. what fits in shared memory)
+ * of the tensor-core GEMM over its rows, each timed with its tile selection
+ * and rescan (where templates screen, that search is only timed); with an ACT_DICT_RECOMPUTE build, every valid (lags per thread,
  * warps, stages, CTAs per SM) combination of the template search instead
  * (act_set_shift_tuning).
  * Results never depend on the configuration, only the speed does.

@@ -1125,35 +1125,41 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         return e;
     };
     cudaError_t err = cudaSuccess;
-    // FP32 GEMV: resident CTAs per SM of the load-streaming GEMV, and the
-    // bulk-copy streaming GEMV
+    // FP32 GEMV: with one channel, resident CTAs per SM of the load-streaming
+    // GEMV, and the bulk-copy streaming GEMV.  Several channels have one form,
+    // which is timed; the one-channel form in use is not theirs to change.
     double best32 = 1e30;
-    int best_grid = g->gemv_grid;
-    bool best_stream = false;
-    g->gemv_stream = false;
-    // (several channels have one form; its time, the one-channel forms as they are by load streaming)
-    if (channels > 1) err = time_search(false, &best32);
-    const int max_per_sm = channels > 1 ? 0 : gemv_max_ctas_per_sm(g->Lp);
-    for (int per_sm = 1; per_sm <= max_per_sm && err == cudaSuccess; ++per_sm) {
-        g->gemv_grid = g->sm_count * per_sm;
-        double ms = 0.0;
-        err = time_search(false, &ms);
-        if (err == cudaSuccess && ms < best32) {
-            best32 = ms;
-            best_grid = g->gemv_grid;
+    if (channels > 1) {
+        err = time_search(false, &best32);
+    } else {
+        const int keep_grid = g->gemv_grid;
+        const bool keep_stream = g->gemv_stream;
+        int best_grid = keep_grid;
+        bool best_stream = false;
+        g->gemv_stream = false;
+        const int max_per_sm = gemv_max_ctas_per_sm(g->Lp);
+        for (int per_sm = 1; per_sm <= max_per_sm && err == cudaSuccess; ++per_sm) {
+            g->gemv_grid = g->sm_count * per_sm;
+            double ms = 0.0;
+            err = time_search(false, &ms);
+            if (err == cudaSuccess && ms < best32) {
+                best32 = ms;
+                best_grid = g->gemv_grid;
+            }
         }
-    }
-    g->gemv_grid = best_grid;
-    if (err == cudaSuccess && channels == 1) {
-        g->gemv_stream = true;
-        double ms = 0.0;
-        err = time_search(false, &ms);
-        if (err == cudaSuccess && ms < best32) {
-            best32 = ms;
-            best_stream = true;
+        g->gemv_grid = best_grid;
+        if (err == cudaSuccess) {
+            g->gemv_stream = true;
+            double ms = 0.0;
+            err = time_search(false, &ms);
+            if (err == cudaSuccess && ms < best32) {
+                best32 = ms;
+                best_stream = true;
+            }
         }
+        g->gemv_grid = err == cudaSuccess ? best_grid : keep_grid;
+        g->gemv_stream = err == cudaSuccess ? best_stream : keep_stream;
     }
-    g->gemv_stream = best_stream;
     // tensor-core search: tile width x pipeline depth of the dense GEMM, or,
     // where the templates screen, that search as it is
     double best16 = 1e30;
