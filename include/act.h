@@ -382,7 +382,11 @@ ACT_API act_status act_autotune(act_grid *grid, const float *signals, int32_t ch
  * (-1: the bulk-copy streaming GEMV, one CTA per SM; the initial choice where
  * the FP32 rows take 64 MiB or more), tensor-core tile width in atoms
  * and pipeline stages of the GEMM over BF16 rows (0 and 0 without a BF16
- * dictionary). */
+ * dictionary).  A BF16 build autotuned with several channels, its one-channel
+ * form neither set by act_set_tuning nor chosen by an autotune with one
+ * channel, names the load-streaming GEMV's grid instead of -1: the one that
+ * the full searches queued by the tensor-core search take.  One channel's
+ * FP32 search is still the bulk-copy streaming GEMV then. */
 ACT_API act_status act_get_tuning(const act_grid *grid, int32_t *gemv_ctas, int32_t *bf16_tile_atoms,
                                   int32_t *bf16_stages);
 

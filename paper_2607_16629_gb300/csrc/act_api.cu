@@ -162,6 +162,8 @@ struct act_grid {
     int screen_channels = 0;      // most channels of a call that the templates screen
     int gemv_grid = 0;
     bool gemv_stream = false;  // FP32 search by the bulk-copy streaming GEMV (one CTA per SM)
+    bool gemv_chosen = false;  // that form was set by hand or by a one-channel autotune
+    bool queue_tuned = false;  // BF16 build autotuned with several channels (act_get_tuning)
     int refine_steps = 0;  // BFGS iterations per order (0: grid-only search)
     unsigned long long wait_ns = kWaitLimitNs;  // limit of each bounded device-side wait
     bool cta_pairs = true;  // the tensor-core template GEMM may pair SMs (cta_group::2)
@@ -1131,6 +1133,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
     double best32 = 1e30;
     if (channels > 1) {
         err = time_search(false, &best32);
+        if (err == cudaSuccess) g->queue_tuned = bf16;
     } else {
         const int keep_grid = g->gemv_grid;
         const bool keep_stream = g->gemv_stream;
@@ -1159,6 +1162,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         }
         g->gemv_grid = err == cudaSuccess ? best_grid : keep_grid;
         g->gemv_stream = err == cudaSuccess ? best_stream : keep_stream;
+        if (err == cudaSuccess) g->gemv_chosen = true;
     }
     // tensor-core search: tile width x pipeline depth of the dense GEMM, or,
     // where the templates screen, that search as it is
@@ -1204,7 +1208,8 @@ act_status act_get_tuning(const act_grid *g, int32_t *gemv_ctas_out, int32_t *bf
     if (!g) return ACT_ERR_INVALID_ARG;
     int bn = 0, stg = 0;
     if (g->bf16) bf16_search_get_config(g->bf16, &bn, &stg, nullptr);
-    if (gemv_ctas_out) *gemv_ctas_out = g->gemv_stream ? -1 : g->gemv_grid;
+    const bool names_queue = g->bf16 && g->queue_tuned && !g->gemv_chosen;
+    if (gemv_ctas_out) *gemv_ctas_out = g->gemv_stream && !names_queue ? -1 : g->gemv_grid;
     if (bf16_tile_atoms) *bf16_tile_atoms = bn;
     if (bf16_stages) *bf16_stages = stg;
     return ACT_OK;
@@ -1222,6 +1227,7 @@ act_status act_set_tuning(act_grid *g, int32_t gemv_ctas_in, int32_t bf16_tile_a
     } else if (gemv_ctas_in < -1) {
         return ACT_ERR_INVALID_ARG;
     }
+    g->gemv_chosen = true;
     if (bf16_tile_atoms > 0) {
         if (!g->bf16) return ACT_ERR_NOT_BUILT;
         cudaError_t e = bf16_search_configure(g->bf16, bf16_tile_atoms, bf16_stages);
