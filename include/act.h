@@ -281,7 +281,10 @@ ACT_API act_status act_get_fused(const act_grid *grid, int32_t channels, int32_t
  * this library from now on (any grid, any thread; nth >= 1) fails once, as
  * if the device were out of memory.  The call that makes it returns
  * ACT_ERR_OOM, frees what it had made for itself and keeps the grid usable
- * (a failed dictionary build keeps no dictionary).  0 disarms it.  Errors:
+ * (a failed dictionary build keeps no dictionary); a BF16 build or search
+ * that has no memory for template screening goes on with the dense GEMM
+ * (for as many channels and more, fewer screen as before).  0 disarms it.
+ * Errors:
  * ACT_ERR_INVALID_ARG for nth < 0. */
 ACT_API act_status act_inject_alloc_failure(int32_t nth);
 

@@ -3,6 +3,7 @@
 // matching pursuit (Eq. (4), Fig. 1) captured once per shape as a CUDA
 // graph and replayed on the caller's stream.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
 #include <stdio.h>
@@ -135,7 +136,8 @@ struct WorkBuffers {
     int lem_B = 0;
     Bf16Scratch b16;                  // dense tensor-core search maxima and rescan lists (on first use)
     ShiftTcScratch stc;               // tensor-core template search rows, maxima, items (on first use)
-    bool dense16 = false;             // no memory for a BF16 build's template screening: the dense GEMM screens
+    int dense16_from = INT_MAX;       // channels from which there was no memory to screen a BF16 build's
+                                      // atoms through their templates: there the dense GEMM screens
 };
 
 struct act_grid {
@@ -250,7 +252,7 @@ void free_dictionary(act_grid *g) {
     // the tensor-core search scratch is sized by the dictionary's shape
     bf16_scratch_free(g->w.b16);
     shift_tc_scratch_free(g->w.stc);
-    g->w.dense16 = false;
+    g->w.dense16_from = INT_MAX;
 }
 
 #define ACT_AL(ptr, bytes)                                                          \
@@ -323,7 +325,7 @@ act_status scratch_status(cudaError_t e, const char *what) {
 // Whether a BF16 search of B channels on w screens through the templates
 // (else by the dense GEMM over the BF16 rows).
 bool screens(const act_grid *g, const WorkBuffers &w, int B) {
-    return g->screen_tc && !w.dense16 && B <= g->screen_channels;
+    return g->screen_tc && B < w.dense16_from && B <= g->screen_channels;
 }
 
 // Whether w holds everything `mode` needs for B channels and P orders.
@@ -357,10 +359,12 @@ act_status grow_work(const act_grid *g, WorkBuffers &w, int B, int P, act_search
             return s;
         }
     }
-    // (without the memory for its scratch, these buffers' searches take the
-    // dense GEMM, whose scratch is smaller, from here on)
-    if (mode == ACT_SEARCH_BF16 && screens(g, w, B) && w.stc.B_cap < B)
-        w.dense16 = shift_tc_reserve(g->screen_tc, g->screen, B, w.stc) != cudaSuccess;
+    // (without the memory for its scratch, which grows with the channels, this
+    // many and more take the dense GEMM on these buffers until the next build;
+    // fewer make their own scratch again)
+    if (mode == ACT_SEARCH_BF16 && screens(g, w, B) && w.stc.B_cap < B &&
+        shift_tc_reserve(g->screen_tc, g->screen, B, w.stc) != cudaSuccess)
+        w.dense16_from = B;
     if (mode == ACT_SEARCH_BF16 && !screens(g, w, B) && w.b16.B_cap < B) {
         if ((s = scratch_status(bf16_scratch_reserve(g->bf16, B, w.b16), "bf16_scratch_reserve")) != ACT_OK)
             return s;
