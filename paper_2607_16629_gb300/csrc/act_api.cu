@@ -984,8 +984,8 @@ act_status act_project(act_grid *g, const float *signals, int32_t channels, floa
         ACT_CK(launch_shift_search(g->shift, g->w.R, g->Lp, g->L, channels, nullptr, scores, g->status, false, st,
                                    nullptr, nullptr, g->wait_ns));
     } else {
-        ACT_CK(launch_project(g->d32, g->K, g->Lp, g->w.R, channels, scores, g->status, g->sm_count, st,
-                              g->wait_ns));
+        ACT_CK(launch_project(g->d32, g->K, g->Lp, g->w.R, channels, scores, g->status, g->sm_count, g->gemv_grid,
+                              st, g->wait_ns));
     }
     return ACT_OK;
 }

@@ -20,8 +20,8 @@ namespace act {
 // warp-shuffle reduction gives every lane the row's score; the warp keeps its
 // best |score| (lowest row on ties, rows are visited in increasing order),
 // the block combines its warps and issues one 64-bit atomicMax of the packed
-// key per channel.  With WRITE every score is stored instead (scores[row]):
-// the projection of one channel on up to kProjectOneBytes of rows.
+// key per channel.  With WRITE every score is stored instead (the projection
+// of one channel, project_multi_bytes).
 template <int NV, bool WRITE>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__ D, int64_t K, int Lp,
                                                        const float *R, int B, const int *chlist, const int *count_dev,
@@ -109,8 +109,13 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
             }
             if (WRITE) {
                 if (lane == 0) {
-                    scores[row] = sa;
-                    if (has2) scores[row2] = sb;
+                    // Looked up at each row: with the channel held from outside
+                    // the loop, or left out, ptxas takes 4 to 14 registers less
+                    // and a call is slower (Lp 256, 94 MB: 20.7 us, 23.0 and
+                    // 26.7 the other ways; Lp 384, 170 MB: 32.9 and 34.8).
+                    const int cw = chlist ? chlist[g] : g;
+                    scores[(int64_t)cw * K + row] = sa;
+                    if (has2) scores[(int64_t)cw * K + row2] = sb;
                 }
             } else {
                 float x = fabsf(sa);
@@ -127,24 +132,25 @@ __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__
                 }
             }
         }
-        if (WRITE) return;  // one channel
-        if (lane == 0) {
-            red_s[wid] = best;
-            red_i[wid] = bidx;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            float bs = -1.0f;
-            uint32_t bi = 0u;
-            for (int w = 0; w < kWarps; ++w) {
-                const float s = red_s[w];
-                const uint32_t i = red_i[w];
-                if (s > bs || (s == bs && i < bi)) {
-                    bs = s;
-                    bi = i;
-                }
+        if (!WRITE) {
+            if (lane == 0) {
+                red_s[wid] = best;
+                red_i[wid] = bidx;
             }
-            if (bs >= 0.0f) atomicMax(keys + ch, pack_key(bs, bi));
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                float bs = -1.0f;
+                uint32_t bi = 0u;
+                for (int w = 0; w < kWarps; ++w) {
+                    const float s = red_s[w];
+                    const uint32_t i = red_i[w];
+                    if (s > bs || (s == bs && i < bi)) {
+                        bs = s;
+                        bi = i;
+                    }
+                }
+                if (bs >= 0.0f) atomicMax(keys + ch, pack_key(bs, bi));
+            }
         }
         __syncthreads();  // the shared residual and reduction slots are reused by the next channel
     }
@@ -207,9 +213,8 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
 }
 
 cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, float *scores, int *status,
-                               int sm_count, cudaStream_t st, unsigned long long wait_ns) {
-    return launch_gemv(D, K, Lp, R, 1, nullptr, nullptr, nullptr, scores, status, gemv_ctas(sm_count, Lp), st, wait_ns,
-                       false);
+                               int grid_ctas, cudaStream_t st, unsigned long long wait_ns) {
+    return launch_gemv(D, K, Lp, R, 1, nullptr, nullptr, nullptr, scores, status, grid_ctas, st, wait_ns, false);
 }
 
 }  // namespace act

@@ -136,17 +136,25 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
 cudaError_t launch_gemv_multi_argmax(const float *D, int64_t K, int Lp, const float *R, int B,
                                      unsigned long long *keys, int *status, int sm_count, cudaStream_t st,
                                      unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
-// Every score of one channel by the load-streaming GEMV.
+// Every score of one channel by the load-streaming GEMV, on grid_ctas CTAs.
 cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, float *scores, int *status,
-                               int sm_count, cudaStream_t st, unsigned long long wait_ns);
+                               int grid_ctas, cudaStream_t st, unsigned long long wait_ns);
 // Every score, scores[b * K + row], any number of channels.  One channel takes
-// the load-streaming GEMV up to this many bytes of rows: us per call of it and
-// of the several-channel form at 17 MB 12.2 and 14.2, 72 MB (N = 300) 16.5 and
-// 20.6, 98 MB (N = 512) 27.7 and 24.7, 170 MB (N = 300) 33.0 and 39.4, 584 MB
-// 112 and 100, 4.3 GB 739 and 627.
-constexpr int64_t kProjectOneBytes = 256ll << 20;
+// the load-streaming GEMV on gemv_grid CTAs, except where the several-channel
+// form is faster: from these bytes of rows on, which depend on the rows' width
+// (us per call of the load-streaming and of the several-channel form):
+//   Lp   128:  140 MB 37.7 and 38.8, 170 MB 44.5 and 43.3, 4.3 GB 849 and 734
+//   Lp   256:  100 MB 23.1 and 27.2, 800 MB 121 and 131, 9.0 GB 1,274 and 1,317
+//   Lp   384:  100 MB 22.6 and 26.7, 800 MB 124 and 131, 9.0 GB 1,313 and 1,325
+//   Lp   512:  200 MB 37.7 and 44.0, 800 MB 128 and 130, 1.6 GB 244 and 243, 4.3 GB 635 and 627
+//   Lp 1,024:  140 MB 33.1 and 35.0, 170 MB 40.2 and 39.6, 4.3 GB 695 and 600
+//   Lp 2,048:  200 MB 39.2 and 48.6, 800 MB 123 and 134, 9.0 GB 1,232 and 1,288
+constexpr int64_t project_multi_bytes(int Lp) {
+    return Lp == 128 || Lp == 1024 ? 160ll << 20 : (Lp == 512 ? 1536ll << 20 : INT64_MAX);
+}
 cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, int B, float *scores,
-                           int *status, int sm_count, cudaStream_t st, unsigned long long wait_ns = kWaitLimitNs);
+                           int *status, int sm_count, int gemv_grid, cudaStream_t st,
+                           unsigned long long wait_ns = kWaitLimitNs);
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
                           unsigned long long *keys, const GridAxes &ax, int k, int P, act_atom *atoms,
                           float *coefs, double *energy, int *fb_count, cudaStream_t st, bool pdl = false);
