@@ -79,9 +79,11 @@ struct ShiftArgs {
 
 // Template value u_t(m) at the integer lag m = n - tc: the dictionary
 // generator's own sample routine at offset m, so on a grid of whole-sample
-// time centres the template holds the unnormalised atom samples bit for bit.
+// time centres the template holds the unnormalised atom samples bit for bit
+// (past 2^24 samples the offset takes both halves of its pair, as there).
 __device__ __forceinline__ float template_sample(int m, const ChirpFF &k) {
-    return chirp_sample_offset({(float)m, 0.0f}, k);
+    const float hi = (float)m;
+    return chirp_sample_offset({hi, (float)(m - (int)hi)}, k);
 }
 
 // One thread per (template block, phase, lane = template): the template's
