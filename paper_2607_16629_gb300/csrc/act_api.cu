@@ -453,8 +453,8 @@ cudaError_t launch_fp32_search(const act_grid *g, const WorkBuffers &w, int B, c
         return launch_gemv_multi_argmax(g->d32, g->K, g->Lp, w.R, B, w.keys, g->status, g->sm_count, st, g->wait_ns,
                                         pdl);
     if (g->gemv_stream)
-        return launch_gemv_stream_argmax(g->d32, g->K, g->Lp, w.R, B, nullptr, nullptr, w.keys, g->status, g->sm_count,
-                                         st, g->wait_ns, pdl);
+        return launch_gemv_stream_argmax(g->d32, g->K, g->Lp, w.R, w.keys, g->status, g->sm_count, st, g->wait_ns,
+                                         pdl);
     return launch_gemv_argmax(g->d32, g->K, g->Lp, w.R, B, nullptr, nullptr, w.keys, g->status, g->gemv_grid, st,
                               g->wait_ns, pdl);
 }

@@ -180,16 +180,17 @@ cudaError_t launch_ragged_scatter(int B, int P, int L, int Lp, const int *chan, 
                                   const act_atom *atoms, const float *coefs, const double *energy, const float *R,
                                   act_atom *out_atoms, float *out_coefs, double *out_energy, float *out_resid,
                                   cudaStream_t st);
-// The same search with the dictionary streamed by TMA bulk copies through
-// shared memory, one CTA per SM (act_gemv_stream.cu); same scores, same keys.
+// The search of one channel with the dictionary streamed by TMA bulk copies
+// through shared memory, one CTA per SM (act_gemv_stream.cu); same scores,
+// same key.
 // The form one channel takes unless tuned, from dictionaries of 64 MiB on:
 // us per order of the load-streaming GEMV and of this form at 24 MB 8.5 and
 // 9.6, 95 MB 19.9 and 18.6 (N = 256; 21.4 and 18.6 at N = 512), 380 MB 62.4
 // and 60.2, 1.5 GB 234 and 213, 3.0 GB 481 and 418, 6.1 GB 914 and 823.
 constexpr int64_t kStreamMinDictBytes = 64ll << 20;
-cudaError_t launch_gemv_stream_argmax(const float *D, int64_t K, int Lp, const float *R, int B, const int *chlist,
-                                      const int *count_dev, unsigned long long *keys, int *status, int sm_count,
-                                      cudaStream_t st, unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
+cudaError_t launch_gemv_stream_argmax(const float *D, int64_t K, int Lp, const float *R, unsigned long long *key,
+                                      int *status, int sm_count, cudaStream_t st,
+                                      unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
 int gemv_ctas(int sm_count, int Lp);          // occupancy-limited, at most 4 CTAs per SM
 int gemv_max_ctas_per_sm(int Lp);
 

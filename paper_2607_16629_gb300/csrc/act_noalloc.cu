@@ -90,8 +90,7 @@ extern "C" act_status act_search_noalloc(const float *dictionary, int64_t n_atom
     // up to 16 of them per pass
     const cudaError_t e =
         channels == 1
-            ? act::launch_gemv_stream_argmax(dictionary, n_atoms, row_stride, residuals, 1, nullptr, nullptr,
-                                             scratch, status, sms, st)
+            ? act::launch_gemv_stream_argmax(dictionary, n_atoms, row_stride, residuals, scratch, status, sms, st)
             : act::launch_gemv_multi_argmax(dictionary, n_atoms, row_stride, residuals, channels, scratch, status,
                                             sms, st);
     if (e != cudaSuccess) return ACT_ERR_CUDA;
