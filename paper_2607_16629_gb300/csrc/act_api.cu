@@ -284,6 +284,7 @@ act_status alloc_base(const act_grid *g, WorkBuffers &w, int B, int P) {
     ACT_CK(cudaMemset(w.fb_count, 0, 2 * sizeof(int)));
     ACT_AL(w.theta, sizeof(double) * 4 * (size_t)B);
     ACT_AL(w.fsync, sizeof(unsigned long long) * (1 + 3 * (size_t)B));
+    ACT_CK(settle());
     w.cap_B = B;
     w.cap_P = P;
     return ACT_OK;
@@ -688,6 +689,7 @@ act_status act_grid_create(const act_grid_desc *desc, int32_t device, act_grid *
     if (e == cudaSuccess) e = cudaMemset(g->stats, 0, 3 * sizeof(long long));
     if (e == cudaSuccess) e = dev_alloc((void **)&g->degenerate, sizeof(unsigned long long));
     if (e == cudaSuccess) e = dev_alloc((void **)&g->eps_bits, sizeof(unsigned int));
+    if (e == cudaSuccess) e = settle();
     if (e != cudaSuccess) {
         note_error("act_grid_create", e);
         act_destroy(g);
@@ -883,7 +885,7 @@ act_status act_dictionary_build(act_grid *g, act_dict_mode mode, void *cuda_stre
         const int64_t ntiles = (g->K + 255) / 256;
         const size_t b16 = sizeof(__nv_bfloat16) * (size_t)ntiles * 256 * g->Lb;
         e = dev_alloc((void **)&g->d16, b16);
-        if (e == cudaSuccess) e = cudaMemset(g->d16, 0, b16);
+        if (e == cudaSuccess) e = cudaMemsetAsync(g->d16, 0, b16, st);  // in front of the rows, on their stream
         if (e != cudaSuccess) {
             cudaGetLastError();
             g->d16 = nullptr;
@@ -1010,6 +1012,7 @@ act_status act_grid_status(act_grid *g, void *cuda_stream) {
     int flags = 0;
     ACT_CK(cudaMemcpy(&flags, g->status, sizeof(int), cudaMemcpyDeviceToHost));
     ACT_CK(cudaMemset(g->status, 0, sizeof(int)));
+    ACT_CK(settle());
     if (flags & kFlagTimeout) return ACT_ERR_DEVICE_TIMEOUT;
     if (flags & kFlagNonFinite) return ACT_ERR_NONFINITE;
     return ACT_OK;
@@ -1430,6 +1433,7 @@ static act_status ragged_build(act_ragged_plan *p, act_grid *const *grids, int32
         ACT_CK(cudaStreamCreateWithFlags(&gr.st, cudaStreamNonBlocking));
         ACT_CK(cudaEventCreateWithFlags(&gr.join, cudaEventDisableTiming));
     }
+    ACT_CK(settle());
     // one graph: fork, then per length group gather -> MP loop -> scatter on
     // its own branch, then join
     ACT_CK(cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal));

@@ -115,6 +115,10 @@ constexpr int kGemvThreads = 256;
 // so that act_inject_alloc_failure can make one of them fail as if the
 // device were out of memory.
 cudaError_t dev_alloc(void **p, size_t bytes);
+// Waits for what was cleared or filled by the legacy stream (cudaMemset and
+// cudaMemcpy may return before the device is done): a caller's non-blocking
+// stream, which is not ordered behind that one, may use it from here on.
+inline cudaError_t settle() { return cudaStreamSynchronize(cudaStreamLegacy); }
 constexpr int kUpdateThreads = 256;
 constexpr int kMaxSamples = 2048;
 constexpr int kRowAlign = 128;   // FP32 row stride granule (floats)
