@@ -21,7 +21,7 @@ namespace act {
 // best |score| (lowest row on ties, rows are visited in increasing order),
 // the block combines its warps and issues one 64-bit atomicMax of the packed
 // key per channel.  With WRITE every score is stored instead (the projection
-// of one channel, project_multi_bytes).
+// of one channel, project_multi_bytes, or of few, one_by_one).
 template <int NV, bool WRITE>
 __global__ void __launch_bounds__(kGemvThreads) k_gemv(const float *__restrict__ D, int64_t K, int Lp,
                                                        const float *R, int B, const int *chlist, const int *count_dev,
@@ -212,9 +212,9 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
     return launch_gemv(D, K, Lp, R, B, chlist, count_dev, keys, nullptr, status, grid_ctas, st, wait_ns, pdl);
 }
 
-cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, float *scores, int *status,
+cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, int B, float *scores, int *status,
                                int grid_ctas, cudaStream_t st, unsigned long long wait_ns) {
-    return launch_gemv(D, K, Lp, R, 1, nullptr, nullptr, nullptr, scores, status, grid_ctas, st, wait_ns, false);
+    return launch_gemv(D, K, Lp, R, B, nullptr, nullptr, nullptr, scores, status, grid_ctas, st, wait_ns, false);
 }
 
 }  // namespace act

@@ -320,8 +320,8 @@ cudaError_t launch_gemv_multi_argmax(const float *D, int64_t K, int Lp, const fl
 
 cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, int B, float *scores, int *status,
                            int sm_count, int gemv_grid, cudaStream_t st, unsigned long long wait_ns) {
-    if (B == 1 && K * (int64_t)Lp * (int64_t)sizeof(float) < project_multi_bytes(Lp))
-        return launch_gemv_scores(D, K, Lp, R, scores, status, gemv_grid, st, wait_ns);
+    if (B == 1 ? K * (int64_t)Lp * (int64_t)sizeof(float) < project_multi_bytes(Lp) : one_by_one(K, Lp, B))
+        return launch_gemv_scores(D, K, Lp, R, B, scores, status, gemv_grid, st, wait_ns);
     return multi_passes<true>(D, K, Lp, R, B, nullptr, scores, status, sm_count, st, wait_ns, false);
 }
 

@@ -140,8 +140,8 @@ cudaError_t launch_gemv_argmax(const float *D, int64_t K, int Lp, const float *R
 cudaError_t launch_gemv_multi_argmax(const float *D, int64_t K, int Lp, const float *R, int B,
                                      unsigned long long *keys, int *status, int sm_count, cudaStream_t st,
                                      unsigned long long wait_ns = kWaitLimitNs, bool pdl = false);
-// Every score of one channel by the load-streaming GEMV, on grid_ctas CTAs.
-cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, float *scores, int *status,
+// Every score by the load-streaming GEMV, on grid_ctas CTAs, channel by channel.
+cudaError_t launch_gemv_scores(const float *D, int64_t K, int Lp, const float *R, int B, float *scores, int *status,
                                int grid_ctas, cudaStream_t st, unsigned long long wait_ns);
 // Every score, scores[b * K + row], any number of channels.  One channel takes
 // the load-streaming GEMV on gemv_grid CTAs, except where the several-channel
@@ -159,6 +159,18 @@ constexpr int64_t project_multi_bytes(int Lp) {
 cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, int B, float *scores,
                            int *status, int sm_count, int gemv_grid, cudaStream_t st,
                            unsigned long long wait_ns = kWaitLimitNs);
+// Whether several channels go one after another through the load-streaming
+// GEMV where the call is that one search or projection.  At 2,048 floats a row
+// the several-channel form takes passes of 4 channels, and with nothing in
+// front of the kernel for its first copies to overlap, a pass over few rows
+// costs what four channels of the GEMV do (us per projection of 1 to 16 MB,
+// one by one and by passes: 2 channels 16.4 and 18.5, 4 20.5 and 18.5, 5 21.0
+// and 26.4, 6 22.6 and 26.7, 8 25.7 and 26.7; at 32 MB 5 channels 28.7 and
+// 31.8, 8 36.9 and 32.8, at 64 MB 41.1 and 39.0).  In a decomposition, launched
+// as dependents, the passes are the faster from 2 channels on.
+constexpr bool one_by_one(int64_t K, int Lp, int B) {
+    return Lp == 2048 && K * Lp * (int64_t)sizeof(float) <= (32ll << 20) && (B % 4 == 1 || B % 4 == 2);
+}
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
                           unsigned long long *keys, const GridAxes &ax, int k, int P, act_atom *atoms,
                           float *coefs, double *energy, int *fb_count, cudaStream_t st, bool pdl = false);

@@ -87,10 +87,13 @@ extern "C" act_status act_search_noalloc(const float *dictionary, int64_t n_atom
         return ACT_ERR_CUDA;
     int *status = reinterpret_cast<int *>(scratch + kNoAllocMaxChannels);
     // one channel: the bulk-copy streaming GEMV; several: the form that scores
-    // up to 16 of them per pass
+    // up to 16 of them per pass, or one by one (one_by_one)
     const cudaError_t e =
         channels == 1
             ? act::launch_gemv_stream_argmax(dictionary, n_atoms, row_stride, residuals, scratch, status, sms, st)
+        : act::one_by_one(n_atoms, row_stride, channels)
+            ? act::launch_gemv_argmax(dictionary, n_atoms, row_stride, residuals, channels, nullptr, nullptr, scratch,
+                                      status, act::gemv_ctas(sms, row_stride), st)
             : act::launch_gemv_multi_argmax(dictionary, n_atoms, row_stride, residuals, channels, scratch, status,
                                             sms, st);
     if (e != cudaSuccess) return ACT_ERR_CUDA;

@@ -1,7 +1,9 @@
 """The projection of one channel has a form of its own, or the several-channel
 form, by the rows' width and size: on every width, on both sides of its limit
 where a small dictionary reaches it, and on a grid of CTAs set by hand, the
-scores are those of a two-channel call bit for bit."""
+scores are those of a two-channel call bit for bit.  Few long rows are passed
+over channel by channel where a last pass would hold one or two of them: the
+scores and selections are those of single calls."""
 import pytest
 import torch
 
@@ -32,5 +34,42 @@ def test_one_channel_equals_two(n, fc):
                 torch.cuda.synchronize()
                 assert act.act_grid_status(h) == act.ACT_OK
                 assert torch.equal(one[0], two[c])
+    finally:
+        act.act_destroy(h)
+
+
+@pytest.mark.parametrize("channels", [2, 3, 5, 6, 9])
+@pytest.mark.parametrize("fc", [3, 27])  # 20 and 178 MiB of rows of 2,048 floats
+def test_few_long_rows(fc, channels):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    grid = synth.Grid(1900, 1000.0, Axis(0.3, 55.0, 34), Axis.linspace(0.5, 32.0, fc), Axis.linspace(-3.0, -0.5, 5),
+                      Axis.linspace(-20.0, 20.0, 5))
+    K, stride = grid.n_atoms, 2048
+    x = torch.randn((channels, grid.n_samples), dtype=torch.float32, device="cuda")
+    h = act.act_grid_create(grid, 0)
+    try:
+        act.act_dictionary_build(h, act.ACT_DICT_FP32)
+        got = torch.full((channels, K), 7.0, device="cuda")
+        act.act_project(h, x, channels, got)
+        one = torch.empty((1, K), device="cuda")
+        for c in range(channels):
+            act.act_project(h, x[c:c + 1], 1, one)
+            torch.cuda.synchronize()
+            assert torch.equal(got[c], one[0])
+        rows = torch.zeros((K, stride), device="cuda")
+        flat = torch.empty((K, grid.n_samples), device="cuda")
+        act.act_dictionary_rows(h, 0, K, flat)
+        rows[:, :grid.n_samples] = flat
+        r = torch.zeros((channels, stride), device="cuda")
+        r[:, :grid.n_samples] = x
+        index = torch.empty(channels, dtype=torch.int64, device="cuda")
+        score = torch.empty(channels, device="cuda")
+        act.act_search_noalloc(rows, K, stride, r, channels, index, score)
+        torch.cuda.synchronize()
+        want = got.abs()
+        assert torch.equal(score, want.max(1).values)
+        for c in range(channels):  # the lowest of equal scores
+            assert int(index[c]) == int((want[c] == score[c]).nonzero()[0])
     finally:
         act.act_destroy(h)
