@@ -73,3 +73,23 @@ def test_few_long_rows(fc, channels):
             assert int(index[c]) == int((want[c] == score[c]).nonzero()[0])
     finally:
         act.act_destroy(h)
+
+
+@pytest.mark.parametrize("stride", [128, 512])
+@pytest.mark.parametrize("rows", [1, 7, 8, 1216, 1217, 2432, 2433, 9728, 9729])
+def test_chunks_of_few_tiles(stride, rows):
+    """Row counts on both sides of one, two and the most tiles of 8 rows a
+    chunk with a chunk for every SM (152 of them), and a last tile of less
+    than 8 rows: three channels at once equal one at a time."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    d = torch.randn((rows, stride), generator=gen, device="cuda")
+    r = torch.randn((3, stride), generator=gen, device="cuda")
+    index, score = torch.empty(3, dtype=torch.int64, device="cuda"), torch.empty(3, device="cuda")
+    act.act_search_noalloc(d, rows, stride, r, 3, index, score)
+    for c in range(3):
+        i, s = torch.empty(1, dtype=torch.int64, device="cuda"), torch.empty(1, device="cuda")
+        act.act_search_noalloc(d, rows, stride, r[c:c + 1], 1, i, s)
+        torch.cuda.synchronize()
+        assert int(i[0]) == int(index[c]) and torch.equal(s[0], score[c])
