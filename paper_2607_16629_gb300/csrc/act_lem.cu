@@ -164,9 +164,9 @@ __device__ __forceinline__ void lem_neighbour(const double *__restrict__ th, int
 // Bound by instruction issue (three slots of four busy; the special-function
 // pipe is a quarter used) beside the FP64 set-up of a block's candidates: 44
 // us for 64 channels x 2,048 candidates x 512 samples, where the float-float
-// projection of all took 230 us (118 instructions a sample).  The phase's
-// products are formed once per candidate, a lane adds its own few (6.19 ->
-// 6.13 ms per decomposition of 20 orders).  Slower or no faster: the cosine as
+// projection of all takes 230 us (118 instructions a sample).  The phase's
+// products are formed once per candidate, a lane adds its own few (every lane
+// forming them: 1 % per decomposition).  Slower or no faster: the cosine as
 // a polynomial on the FMA pipe (6 %), two samples to a packed instruction (48
 // registers: fewer warps), 32 candidates a block, 32 registers a thread.
 constexpr float kScreenX = 5.8f;
@@ -485,8 +485,7 @@ __device__ int pick_top(PickShared &sm, int k, int entries, const unsigned long 
 __global__ void __launch_bounds__(kPickThreads) k_lem_pick(int cap, int k, int level_candidates,
                                                           const double *cand, const int *ncand, int per, int *nkept,
                                                           const float2 *screen, const float *R, int Lp, int L,
-                                                          double inv_fs, double *score,
-                                                          double *kept,
+                                                          double inv_fs, double *score, double *kept,
                                                           double *kept_score) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -606,7 +605,7 @@ cudaError_t launch_lem_select(const LemConfig &cfg, int B, int order, const floa
     }
     // Each kernel a programmatic dependent of the one before it (the sampling
     // beside the update of the order before): 64 EEG-like channels, 20 orders,
-    // 6.26 -> 6.19 ms.
+    // 6.11 ms, plain launches 1 % more.
     cudaError_t e = launch_kernel(k_lem_lhs, dim3(B, 4), dim3(kLhsThreads), smem, st, pdl, cfg.n_coarse, log2b,
                                   cfg.box, cfg.seed, order, lb.cap, lb.cand, lb.ncand);
     const double inv_fs = 1.0 / fs;

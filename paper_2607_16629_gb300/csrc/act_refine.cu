@@ -306,8 +306,8 @@ __device__ __forceinline__ void eval_warp_scatter(const EvalAcc &a, int lane, fl
 // component (lane & 3) of its gradient (zeros elsewhere).  kSpan: samples a
 // thread evaluates at once, 2 where L <= 512, else 4 (with 4 there, half of
 // the evaluations and more were of samples past the window: 64 EEG-like
-// channels, hierarchical search, 6.48 -> 6.27 ms).  kShort (L <= 256): the
-// second is passed over too (a 256-sample epoch 1.11 -> 1.01 ms).  With kSpan
+// channels, hierarchical search, 3 % slower).  kShort (L <= 256): the second
+// is passed over too (a 256-sample epoch 1.02 ms, without 1.11).  With kSpan
 // 1 the compiler fuses products and sums differently, and a trajectory
 // changes with its last bits; this form keeps them.
 template <int kSpan, bool kShort>
@@ -624,17 +624,15 @@ __global__ void __launch_bounds__(kBfgsThreads) k_refine(GridAxes ax, RefineBox 
 // the dictionary generator (float-float phase, chirp_sample_ff), formed once
 // into registers; |u|^2 is a float-float sum, c = <g, r> an FP32 block sum,
 // |r|^2 an FP64 sum.
-__global__ void __launch_bounds__(kRefineThreads) k_update_refined(int Lp, float *R,
-                                                                  __nv_bfloat16 *R16, int Lb,
+__global__ void __launch_bounds__(kRefineThreads) k_update_refined(int Lp, float *R, __nv_bfloat16 *R16, int Lb,
                                                                   unsigned long long *keys, GridAxes ax,
                                                                   const double *theta, int k, int P,
-                                                                  act_atom *atoms,
-                                                                  float *coefs,
-                                                                  double *energy, int *fb_count) {
+                                                                  act_atom *atoms, float *coefs, double *energy,
+                                                                  int *fb_count) {
     // In the hierarchical search (no keys) a programmatic dependent of the
     // refinement, and the next order's samples are drawn beside it; a template
-    // search is not launched early (32 radar-like channels 3,625 -> 3,638 us
-    // where it was).  (No __restrict__ on what the refinement writes: a load
+    // search is not launched early (32 radar-like channels no faster where it
+    // is).  (No __restrict__ on what the refinement writes: a load
     // may move ahead of the wait.)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!keys) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -6,12 +6,11 @@
 //     the BF16 templates (N = 256 templates per tile) against the shifted
 //     residual rows (M = 128 rows per tile), K = Kt lags.  A tile multiplies
 //     only the lags that its rows' windows see and its templates span
-//     (k_shift_spans).  That is bounded by the tensor pipe and the issue of
-//     its MMAs, so fewer lags is what helps: by that alone 256 uneven EMG-like
-//     channels (atoms of 9-111 samples in windows of 256-2,048) went from 57.8
-//     to 34.6 ms per 30-order decomposition, 32 radar-like channels from 4.54
-//     to 4.17 ms (with the issue loop, the epilogue and the row tiles below now
-//     21.3 and 3.64; 64 EEG-like channels 2.40 and now 1.74);
+//     (k_shift_spans): the GEMM is bounded by the tensor pipe and the issue of
+//     its MMAs, so fewer lags is what helps (multiplying every lag the windows
+//     see, 256 uneven EMG-like channels, atoms of 9-111 samples in windows of
+//     256-2,048, took 57.8 ms per 30-order decomposition, now 21.2; 32
+//     radar-like channels 4.54 and 3.65, 64 EEG-like channels 2.40 and 1.74);
 //  2. the tcgen05 GEMM scales every accumulator by its atom's 1/|u| and keeps,
 //     per row, the largest |score| of every template tile and of every
 //     32-template block;
@@ -101,8 +100,8 @@ constexpr int kRescanWarps = 4;     // independent warps per rescore block
 constexpr int kRescanBufs = 8;      // phase buffers per warp, at most
 // Bytes of a warp's buffers where it has more than two: with few channels
 // (few items) one or two warps an SM with every phase in flight, with many
-// four warps an SM.  One EEG-like channel 536 -> 511 us per decomposition, 64
-// of them 1,730 us with two buffers a warp and 1,768 with four.
+// four warps an SM.  One EEG-like channel 511 us per decomposition and 536
+// with two buffers a warp, 64 of them 1,768 with four and 1,730 with two.
 constexpr int kRescanFewBytes = 108 * 1024;
 constexpr int kRescanFewChannels = 16;
 
@@ -251,9 +250,8 @@ __device__ __forceinline__ void item_steps(short2 rows, short2 tpls, int &lo, in
 __global__ void __launch_bounds__(256) k_shift_rows(RowTiling t, const float *R, int Lp, int tc0,
                                                     int m_lo, int Kt, int RJ, int KSEG, int n_seg, int span_pad,
                                                     int err_terms, const unsigned int *__restrict__ eps_bits,
-                                                    __nv_bfloat16 *X, float *bound,
-                                                    unsigned int *chmax, int *chcount,
-                                                    long long *stats) {
+                                                    __nv_bfloat16 *X, float *bound, unsigned int *chmax,
+                                                    int *chcount, long long *stats) {
     extern __shared__ __align__(16) uint8_t rows_raw[];
     __shared__ float sh[32];
     // a programmatic dependent of the previous kernel (the residual update):
@@ -364,8 +362,7 @@ template <int BN, bool PAIR>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     k_shift_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, RowTiling tl,
                  int n_tiles, int nkc, int stages, int T_pad, const short2 *__restrict__ span,
-                 const float *__restrict__ scaleT, float *tile_max, float *blk_max,
-                 unsigned int *chmax,
+                 const float *__restrict__ scaleT, float *tile_max, float *blk_max, unsigned int *chmax,
                  int *status, unsigned long long wait_ns) {
     // shared memory: stages, then the item's scales [Jt][BN + 4] (the +4
     // floats of padding spread the Jt rows a warp reads over the banks)
@@ -475,13 +472,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         // ---------------- MMA issuer (PAIR: the leader only) ----------------
         // The whole warp runs the loop and one elected lane issues: with the
         // control flow and the operands uniform over the warp, the
-        // descriptors stay in uniform registers, where the MMA takes them.  With
-        // lane 0 alone in the loop each MMA took about 230 cycles to issue
-        // (64 EEG-like channels 2.16 -> 1.89 ms, 32 radar-like 4.22 -> 3.76 ms,
-        // the uneven EMG-like batch 31.6 -> 27.0 ms).
+        // descriptors stay in uniform registers, where the MMA takes them (lane
+        // 0 alone in the loop took about 230 cycles to issue each).  What it
+        // has to keep up with is one M x 256 x 16 MMA per 128 cycles: an item
+        // of 19.7 MMAs (64 EEG-like channels) takes 3,984 cycles, the rest
+        // lost between stages of one to four MMAs.
         tc_fence_after();
-        // the issuing thread must keep up with the tensor core (one M x 256 x 16
-        // MMA per 128 cycles): no divisions, descriptors formed once per stage
         const bool issuer = elect_one();
         uint32_t s = 0, ph = 0, local = 0;
         auto test_full = [&](uint32_t st, uint32_t parity) {
@@ -514,9 +510,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
                 tc_fence_after();
                 const uint32_t s1 = s + 1 == (uint32_t)stages ? 0u : s + 1, ph1 = s1 == 0u ? ph ^ 1u : ph;
                 // look at the next stage's barrier now: the answer is there when
-                // these MMAs are issued (a look took some 290 cycles, now 170;
-                // 64 EEG-like channels 1.88 -> 1.81 ms with this, whole chunks
-                // issued without a test per step and 32-bit divisions)
+                // these MMAs are issued (a look afterwards costs some 290
+                // cycles, this one 170)
                 const bool next = test_full(s1, ph1);
                 const uint32_t b0 = base + s * (uint32_t)kStageBytes;
                 // only the chunk's steps inside [ks_lo, ks_hi]
@@ -690,8 +685,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 __global__ void __launch_bounds__(256) k_shift_flag(int Ntc, int n_tiles, int bpt, int max_items,
                                                     const float *tile_max, const float *blk_max, const float *bound,
                                                     const unsigned int *chmax, const int *__restrict__ blk_order,
-                                                    int *chcount, int *fb_list,
-                                                    int *counters, int *items,
+                                                    int *chcount, int *fb_list, int *counters, int *items,
                                                     long long *stats) {
     const int b = blockIdx.y;
     asm volatile("griddepcontrol.wait;" ::: "memory");  // the rows kernel's bound, the GEMM's maxima
@@ -955,12 +949,13 @@ void shift_tc_scratch_free(ShiftTcScratch &x) {
 // Jt as small as B allows (fewer lag chunks per tile), at most the time
 // centres (rounded up to a power of two).  Up to 16 channels past whole
 // blocks of 32 (up to 8 past one block of 16) take tiles of 8 or 16 channels x
-// 16 or 8 time centres instead of one more block that is mostly padding, unless the time centres lie so
-// far apart that such a tile's windows see over a quarter more lags.  Row
-// build + GEMM in us per order, EEG-like grid: 17 channels 41.0 -> 36.7, 33
-// 67.5 -> 49.2, 48 68.3 -> 57.5, 66 97 -> 80; EMG-like, 2,048 samples: 90 ->
-// 78, 160 -> 116, 167 -> 141, 237 -> 197; the uneven EMG-like batch (66, 60, 73 and 57 channels) 25.1 ->
-// 21.3 ms.
+// 16 or 8 time centres instead of one more block that is mostly padding,
+// unless the time centres lie so far apart that such a tile's windows see over
+// a quarter more lags.  Row build + GEMM in us per order with a padded block
+// and with such tiles, EEG-like grid: 17 channels 41.0 and 36.7, 33 67.5 and
+// 49.2, 48 68.3 and 57.5, 66 97 and 80; EMG-like, 2,048 samples: 90 and 78,
+// 160 and 116, 167 and 141, 237 and 197; the uneven EMG-like batch (66, 60, 73
+// and 57 channels) 25.1 and 21.2 ms.
 static RowTiling make_tiling(const ShiftPlan &sp, int B) {
     RowTiling t;
     int bg = 1;
