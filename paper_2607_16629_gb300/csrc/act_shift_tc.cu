@@ -98,12 +98,16 @@ constexpr int kMaxItems = 1024;    // flagged (lag, block) items per channel bef
 constexpr int kMaxRowItems = 512;  // the same where the items are rows of a stored dictionary
 constexpr int kRescanWarps = 4;     // independent warps per rescore block
 constexpr int kRescanBufs = 8;      // phase buffers per warp, at most
-// Bytes of a warp's buffers where it has more than two: with few channels
-// (few items) one or two warps an SM with every phase in flight, with many
-// four warps an SM.  One EEG-like channel 511 us per decomposition and 536
+// Bytes of a warp's residual and buffers where it has more than two: with few
+// channels (few items) one or two warps an SM with every phase in flight, with
+// many four warps an SM.  One EEG-like channel 511 us per decomposition and 536
 // with two buffers a warp, 64 of them 1,768 with four and 1,730 with two.
+// Where not every phase has a buffer there is little to gain and warps to
+// lose: EMG-like channels of 2,048 samples, 30 orders, three buffers and two,
+// 1 channel 1.414 and 1.419 ms, 4 1.796 and 1.798, 8 2.14 and 2.12, 16 2.87
+// and 2.69.
 constexpr int kRescanFewBytes = 108 * 1024;
-constexpr int kRescanFewChannels = 16;
+constexpr int kRescanFewChannels = 16, kRescanFewPhased = 4;
 
 struct Smem {
     uint64_t bar_full[kMaxStages];
@@ -854,6 +858,7 @@ struct ShiftTc {
     CUtensorMap mapB[2];    // box heights 128 and 256
     int nkc = 0, sm_count = 0, T_pad = 0;
     int pair_clusters = 0;  // co-resident CTA pairs of the paired GEMM (0: not available)
+    int few_channels = 0;   // most channels of a call whose rescore takes rescan[0]
     struct {
         int bufs = 0, warps = 0, blocks_per_sm = 0;
         size_t smem = 0;
@@ -908,6 +913,7 @@ cudaError_t shift_tc_prepare(ShiftTc **out, const ShiftPlan &sp, int sm_count) {
     for (int i = 0; i < 2; ++i) {
         int nb = 2;
         while (i == 0 && nb < sp.Sa && nb < kRescanBufs && res + (nb + 1) * buf <= (size_t)kRescanFewBytes) ++nb;
+        if (i == 0) s->few_channels = nb < sp.Sa ? kRescanFewPhased : kRescanFewChannels;
         const size_t per_warp = res + nb * buf;
         int rw = kRescanWarps;
         while (rw > 1 && rw * per_warp > (size_t)kRescanSmem) --rw;
@@ -1150,7 +1156,7 @@ cudaError_t launch_shift_tc_resolve(const ShiftTc *s, const ShiftTcScratch &x, c
     if (!s || B < 1 || B > x.B_cap) return cudaErrorInvalidValue;
     cudaError_t e = launch_flag(s, x, sp, B, kMaxItems, fb_list, counters, stats, st, pdl);
     if (e != cudaSuccess) return e;
-    const auto &rc = s->rescan[B <= kRescanFewChannels ? 0 : 1];
+    const auto &rc = s->rescan[B <= s->few_channels ? 0 : 1];
     e = launch_kernel(k_shift_rescan, dim3(s->sm_count * rc.blocks_per_sm), dim3(rc.warps * 32), rc.smem, st, true,
                       (const float *)sp.tpl, (const float *)sp.scale, sp.S, sp.Sa, sp.P, sp.rows, sp.NtcP, sp.Ntc,
                       sp.T, sp.T_pad / 32, Lp, L, R, reinterpret_cast<const int2 *>(x.items),

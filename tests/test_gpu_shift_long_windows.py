@@ -38,3 +38,23 @@ def test_equals_fp32_template_search(step, n, channels):
             assert np.array_equal(x, y)
     finally:
         act.act_destroy(h)
+
+
+@pytest.mark.parametrize("channels", [3, 5])
+@pytest.mark.parametrize("step,n", [(4, 832), (4, 833), (8, 1696), (9, 1700)])
+def test_few_channels_phases_in_flight(step, n, channels):
+    """Rescores with every phase in flight up to the last window that leaves
+    room for it (832 samples at step 4) and to eight phases, and past them
+    with the buffers there is room for (4 channels and fewer) or with two."""
+    grid = synth.Grid(n, 500.0, Axis(3.0, float(step), 70), Axis(20.0, 30.0, 5), Axis(-4.0, 0.7, 5), Axis(-60.0, 40.0, 4))
+    sig = synth.random_signals(29, channels, n)
+    h = act.act_grid_create(grid, 0)
+    try:
+        act.act_dictionary_build(h, act.ACT_DICT_RECOMPUTE)
+        act.act_set_search(h, act.ACT_SEARCH_SHIFT)
+        want = gpu_decompose(h, sig, 4)
+        act.act_set_search(h, act.ACT_SEARCH_SHIFT_BF16)
+        for x, y in zip(gpu_decompose(h, sig, 4), want):
+            assert np.array_equal(x, y)
+    finally:
+        act.act_destroy(h)
