@@ -163,13 +163,15 @@ cudaError_t launch_project(const float *D, int64_t K, int Lp, const float *R, in
 // GEMV where the call is that one search or projection.  At 2,048 floats a row
 // the several-channel form takes passes of 4 channels, and with nothing in
 // front of the kernel for its first copies to overlap, a pass over few rows
-// costs what four channels of the GEMV do (us per projection of 1 to 16 MB,
-// one by one and by passes: 2 channels 16.4 and 18.5, 4 20.5 and 18.5, 5 21.0
-// and 26.4, 6 22.6 and 26.7, 8 25.7 and 26.7; at 32 MB 5 channels 28.7 and
-// 31.8, 8 36.9 and 32.8, at 64 MB 41.1 and 39.0).  In a decomposition, launched
-// as dependents, the passes are the faster from 2 channels on.
+// costs what four channels of the GEMV do, so one or two channels left for the
+// last pass are better off without it (us per projection one by one and by
+// passes: 1 to 4 MB, 2 channels 16.4 and 18.4, 5 20.5 and 25.8, 6 22.6 and
+// 26.2, 10 28.7 and 34.9, 34 61.5 and 83; 16 MB, 2 18.5 and 18.5, 5 24.6 and
+// 26.7, 6 26.7 and 26.7, 34 73.7 and 84; 24 MB, 5 26.7 and 26.7, 6 30.3 and
+// 26.7).  In a decomposition, launched as dependents, the passes are the
+// faster from 2 channels on.
 constexpr bool one_by_one(int64_t K, int Lp, int B) {
-    return Lp == 2048 && K * Lp * (int64_t)sizeof(float) <= (32ll << 20) && (B % 4 == 1 || B % 4 == 2);
+    return Lp == 2048 && K * Lp * (int64_t)sizeof(float) <= (15ll << 20) && (B % 4 == 1 || B % 4 == 2);
 }
 cudaError_t launch_update(const float *D32, int Lp, int L, float *R, __nv_bfloat16 *R16, int Lb, int B,
                           unsigned long long *keys, const GridAxes &ax, int k, int P, act_atom *atoms,
