@@ -271,21 +271,18 @@ template <int N8, int N4, bool WS>
 cudaError_t multi_instance(const float *D, int64_t K, int Lp, const float *R, int ng, unsigned long long *keys,
                            float *scores, int *status, int sm_count, cudaStream_t st, unsigned long long wait_ns,
                            bool pdl) {
-    // Tiles per chunk, a power of two and at most 32 KB of them: the fewest
-    // that give no CTA a second chunk where that can be (a warp's first tile
-    // is then its only one in most), else as many as leave every SM two
-    // chunks.  us per order, 4 channels, rows of 128 floats: 2 MB 6.84 by the
-    // second rule alone and 6.15, 4 MB 8.12 and 6.67 (the GEMV in passes of
-    // four channels took 7.3), of 256 floats: 8 MB 7.80 and 7.12.
+    // Tiles per chunk, at most 32 KB of them: the fewest that give no CTA a
+    // second chunk where that can be (a warp's first tile is then its only one
+    // in most), else a power of two that leaves every SM two chunks.  us per
+    // order, 4 channels, rows of 128 floats: 2 MB 6.84 by the second rule
+    // alone and 6.15, 4 MB 8.12 and 6.67 (the GEMV in passes of four channels
+    // took 7.3), of 256 floats: 8 MB 7.80 and 7.12.
     const int64_t total = (K + kTileRows - 1) / kTileRows;
-    int tiles = 1, most = 1;
+    int most = 1;
     while (2 * most * kTileRows * Lp * 4 <= kMultiChunk) most *= 2;
-    if (total <= (int64_t)most * sm_count) {
-        while (total > (int64_t)tiles * sm_count) tiles *= 2;
-    } else {
-        tiles = most;
+    int tiles = (int)(total <= (int64_t)most * sm_count ? (total + sm_count - 1) / sm_count : most);
+    if (total > (int64_t)most * sm_count)
         while (tiles > 1 && (K + tiles * kTileRows - 1) / (tiles * kTileRows) < 2 * (int64_t)sm_count) tiles /= 2;
-    }
     const int chunk = tiles * kTileRows * Lp * 4;
     int stages = kMultiRing / chunk;
     if (stages > kMultiMaxStages) stages = kMultiMaxStages;

@@ -76,11 +76,12 @@ def test_few_long_rows(fc, channels):
 
 
 @pytest.mark.parametrize("stride", [128, 512])
-@pytest.mark.parametrize("rows", [1, 7, 8, 1216, 1217, 2432, 2433, 9728, 9729])
+@pytest.mark.parametrize("rows", [1, 7, 8, 1216, 1217, 2432, 2433, 5000, 8400, 9728, 9729])
 def test_chunks_of_few_tiles(stride, rows):
     """Row counts on both sides of one, two and the most tiles of 8 rows a
-    chunk with a chunk for every SM (152 of them), and a last tile of less
-    than 8 rows: three channels at once equal one at a time."""
+    chunk with a chunk for every SM (152 of them), of five and seven, and a
+    last tile of less than 8 rows: three channels at once equal one at a
+    time."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     gen = torch.Generator(device="cuda").manual_seed(rows)
