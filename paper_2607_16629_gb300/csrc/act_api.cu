@@ -267,24 +267,26 @@ void free_dictionary(act_grid *g) {
 
 // Work buffers for B channels and P orders on a grid of window L.  The BF16
 // residual copy always has a multiple of 128 rows (the tensor-core tile
-// height), padded with zeros.  On failure the caller frees what was made.
-act_status alloc_base(const act_grid *g, WorkBuffers &w, int B, int P) {
+// height), padded with zeros.  What is cleared is cleared on st, in front of
+// the caller's kernels (cudaMemset would go to the legacy stream, which a
+// non-blocking one is not ordered behind).  On failure the caller frees what
+// was made.
+act_status alloc_base(const act_grid *g, WorkBuffers &w, int B, int P, cudaStream_t st) {
     const int rows16 = round_up(B, 128);
     ACT_AL(w.sig, sizeof(float) * (size_t)B * g->L);
     ACT_AL(w.R, sizeof(float) * (size_t)B * g->Lp);
     ACT_AL(w.R16, sizeof(__nv_bfloat16) * (size_t)rows16 * g->Lb);
-    ACT_CK(cudaMemset(w.R16, 0, sizeof(__nv_bfloat16) * (size_t)rows16 * g->Lb));
+    ACT_CK(cudaMemsetAsync(w.R16, 0, sizeof(__nv_bfloat16) * (size_t)rows16 * g->Lb, st));
     ACT_AL(w.keys, sizeof(unsigned long long) * (size_t)B);
-    ACT_CK(cudaMemset(w.keys, 0, sizeof(unsigned long long) * (size_t)B));
+    ACT_CK(cudaMemsetAsync(w.keys, 0, sizeof(unsigned long long) * (size_t)B, st));
     ACT_AL(w.atoms, sizeof(act_atom) * (size_t)B * P);
     ACT_AL(w.coefs, sizeof(float) * (size_t)B * P);
     ACT_AL(w.energy, sizeof(double) * (size_t)B * (P + 1));
     ACT_AL(w.fb_list, sizeof(int) * (size_t)B);
     ACT_AL(w.fb_count, 2 * sizeof(int));
-    ACT_CK(cudaMemset(w.fb_count, 0, 2 * sizeof(int)));
+    ACT_CK(cudaMemsetAsync(w.fb_count, 0, 2 * sizeof(int), st));
     ACT_AL(w.theta, sizeof(double) * 4 * (size_t)B);
     ACT_AL(w.fsync, sizeof(unsigned long long) * (1 + 3 * (size_t)B));
-    ACT_CK(settle());
     w.cap_B = B;
     w.cap_P = P;
     return ACT_OK;
@@ -341,13 +343,13 @@ bool work_fits(const act_grid *g, const WorkBuffers &w, int B, int P, act_search
 // Grows w to what `mode` needs for B channels and P orders (each part to at
 // least its current size).  The caller has destroyed every graph recorded
 // on w.  On failure the parts that could not be made are left empty.
-act_status grow_work(const act_grid *g, WorkBuffers &w, int B, int P, act_search_mode mode) {
+act_status grow_work(const act_grid *g, WorkBuffers &w, int B, int P, act_search_mode mode, cudaStream_t st) {
     act_status s = ACT_OK;
     if (B > w.cap_B || P > w.cap_P) {
         const int nB = B > w.cap_B ? B : w.cap_B;
         const int nP = P > w.cap_P ? P : w.cap_P;
         free_base(w);
-        if ((s = alloc_base(g, w, nB, nP)) != ACT_OK) {
+        if ((s = alloc_base(g, w, nB, nP, st)) != ACT_OK) {
             free_base(w);
             return s;
         }
@@ -364,25 +366,25 @@ act_status grow_work(const act_grid *g, WorkBuffers &w, int B, int P, act_search
     // many and more take the dense GEMM on these buffers until the next build;
     // fewer make their own scratch again)
     if (mode == ACT_SEARCH_BF16 && screens(g, w, B) && w.stc.B_cap < B &&
-        shift_tc_reserve(g->screen_tc, g->screen, B, w.stc) != cudaSuccess)
+        shift_tc_reserve(g->screen_tc, g->screen, B, w.stc, st) != cudaSuccess)
         w.dense16_from = B;
     if (mode == ACT_SEARCH_BF16 && !screens(g, w, B) && w.b16.B_cap < B) {
         if ((s = scratch_status(bf16_scratch_reserve(g->bf16, B, w.b16), "bf16_scratch_reserve")) != ACT_OK)
             return s;
     }
     if (mode == ACT_SEARCH_SHIFT_BF16 && w.stc.B_cap < B) {
-        if ((s = scratch_status(shift_tc_reserve(g->shift_tc, g->shift, B, w.stc), "shift_tc_reserve")) != ACT_OK)
-            return s;
+        s = scratch_status(shift_tc_reserve(g->shift_tc, g->shift, B, w.stc, st), "shift_tc_reserve");
+        if (s != ACT_OK) return s;
     }
     return ACT_OK;
 }
 
 // The grid's own work buffers: any growth first destroys the grid's graphs,
 // which captured their addresses.
-act_status ensure_work(act_grid *g, int B, int P, act_search_mode mode) {
+act_status ensure_work(act_grid *g, int B, int P, act_search_mode mode, cudaStream_t st) {
     if (work_fits(g, g->w, B, P, mode)) return ACT_OK;
     drop_graphs(g);
-    return grow_work(g, g->w, B, P, mode);
+    return grow_work(g, g->w, B, P, mode, st);
 }
 
 // Hierarchical-search settings from the public struct; the box is the
@@ -684,12 +686,12 @@ act_status act_grid_create(const act_grid_desc *desc, int32_t device, act_grid *
     g->coop = coop != 0;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&g->cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = dev_alloc((void **)&g->status, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(g->status, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(g->status, 0, sizeof(int), g->cap);
     if (e == cudaSuccess) e = dev_alloc((void **)&g->stats, 3 * sizeof(long long));
-    if (e == cudaSuccess) e = cudaMemset(g->stats, 0, 3 * sizeof(long long));
+    if (e == cudaSuccess) e = cudaMemsetAsync(g->stats, 0, 3 * sizeof(long long), g->cap);
     if (e == cudaSuccess) e = dev_alloc((void **)&g->degenerate, sizeof(unsigned long long));
     if (e == cudaSuccess) e = dev_alloc((void **)&g->eps_bits, sizeof(unsigned int));
-    if (e == cudaSuccess) e = settle();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->cap);  // any stream may be the first to use them
     if (e != cudaSuccess) {
         note_error("act_grid_create", e);
         act_destroy(g);
@@ -750,9 +752,10 @@ static cudaError_t make_templates(const act_grid *g, ShiftPlan &sp, unsigned lon
         if (e == cudaSuccess) e = dev_alloc((void **)&sp.span, sizeof(short2) * (size_t)(sp.T_pad / 128));
         if (e == cudaSuccess) e = dev_alloc((void **)&sp.blk_order, sizeof(int) * order.size());
         if (e == cudaSuccess)
-            e = cudaMemcpyAsync(sp.blk_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, st);
-        // (the table is pageable memory of this call's own: the copy has to be over before it goes)
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            e = cudaMemcpyAsync(sp.blk_order, order.data(), sizeof(int) * order.size(), cudaMemcpyHostToDevice, g->cap);
+        // (the table is pageable memory of this call's own: the copy, on a stream
+        // with nothing else to wait for, has to be over before it goes)
+        if (e == cudaSuccess) e = cudaStreamSynchronize(g->cap);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.scaleT, 0, bst, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(sp.eps_bits, 0, sizeof(unsigned int), st);
     }
@@ -935,7 +938,7 @@ act_status act_decompose(act_grid *g, const float *signals, int32_t channels, in
     if (mode == ACT_SEARCH_LEM && n_atoms > 4096) return ACT_ERR_UNSUPPORTED;  // draw counter holds 12 bits of order
     DeviceGuard dg(g->device);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    act_status s = ensure_work(g, channels, n_atoms, mode);
+    act_status s = ensure_work(g, channels, n_atoms, mode, st);
     if (s != ACT_OK) return s;
     bool host_seen = !is_device_ptr(signals);
     // all buffers in the grid device's memory and the single-launch form
@@ -978,7 +981,7 @@ act_status act_project(act_grid *g, const float *signals, int32_t channels, floa
     if (g->built < 0) return ACT_ERR_NOT_BUILT;
     DeviceGuard dg(g->device);
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    act_status s = ensure_work(g, channels, 1, ACT_SEARCH_FP32);
+    act_status s = ensure_work(g, channels, 1, ACT_SEARCH_FP32, st);
     if (s != ACT_OK) return s;
     ACT_CK(cudaMemcpyAsync(g->w.sig, signals, sizeof(float) * (size_t)channels * g->L, cudaMemcpyDefault, st));
     ACT_CK(launch_init(g->w.sig, channels, g->L, g->Lp, g->w.R, nullptr, g->Lb, nullptr, nullptr, 1, g->status, st));
@@ -1011,8 +1014,8 @@ act_status act_grid_status(act_grid *g, void *cuda_stream) {
     ACT_CK(cudaStreamSynchronize((cudaStream_t)cuda_stream));
     int flags = 0;
     ACT_CK(cudaMemcpy(&flags, g->status, sizeof(int), cudaMemcpyDeviceToHost));
-    ACT_CK(cudaMemset(g->status, 0, sizeof(int)));
-    ACT_CK(settle());
+    ACT_CK(cudaMemsetAsync(g->status, 0, sizeof(int), g->cap));
+    ACT_CK(cudaStreamSynchronize(g->cap));
     if (flags & kFlagTimeout) return ACT_ERR_DEVICE_TIMEOUT;
     if (flags & kFlagNonFinite) return ACT_ERR_NONFINITE;
     return ACT_OK;
@@ -1081,7 +1084,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
     DeviceGuard dg(g->device);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     if (g->built == ACT_DICT_RECOMPUTE) {
-        act_status s = ensure_work(g, channels, 1, ACT_SEARCH_SHIFT);
+        act_status s = ensure_work(g, channels, 1, ACT_SEARCH_SHIFT, st);
         if (s != ACT_OK) return s;
         ACT_CK(cudaMemcpyAsync(g->w.sig, signals, sizeof(float) * (size_t)channels * g->L, cudaMemcpyDefault, st));
         ACT_CK(launch_init(g->w.sig, channels, g->L, g->Lp, g->w.R, nullptr, g->Lb, g->w.keys, nullptr, 1, g->status,
@@ -1089,7 +1092,7 @@ act_status act_autotune(act_grid *g, const float *signals, int32_t channels, voi
         return autotune_shift(g, channels, st, best_ms);
     }
     const bool bf16 = g->bf16 != nullptr;
-    act_status s = ensure_work(g, channels, 1, bf16 ? ACT_SEARCH_BF16 : ACT_SEARCH_FP32);
+    act_status s = ensure_work(g, channels, 1, bf16 ? ACT_SEARCH_BF16 : ACT_SEARCH_FP32, st);
     if (s != ACT_OK) return s;
     ACT_CK(cudaMemcpyAsync(g->w.sig, signals, sizeof(float) * (size_t)channels * g->L, cudaMemcpyDefault, st));
     ACT_CK(launch_init(g->w.sig, channels, g->L, g->Lp, g->w.R, g->w.R16, g->Lb, g->w.keys, nullptr, 1, g->status, st));
@@ -1422,18 +1425,19 @@ static act_status ragged_build(act_ragged_plan *p, act_grid *const *grids, int32
         if (!search_available(g, gr.mode)) return ACT_ERR_NOT_BUILT;
         // the plan's own buffers, search scratch included: nothing the
         // plan's graph captures belongs to the grid's work buffers
-        act_status s = grow_work(g, gr.w, B, p->P, gr.mode);
+        act_status s = grow_work(g, gr.w, B, p->P, gr.mode, p->cap);
         if (s != ACT_OK) return s;
         std::vector<int64_t> off(B);
         for (int i = 0; i < B; ++i) off[i] = offsets[gr.chan[i]];
         ACT_AL(gr.src_off, sizeof(int64_t) * B);
-        ACT_CK(cudaMemcpy(gr.src_off, off.data(), sizeof(int64_t) * B, cudaMemcpyHostToDevice));
+        ACT_CK(cudaMemcpyAsync(gr.src_off, off.data(), sizeof(int64_t) * B, cudaMemcpyHostToDevice, p->cap));
+        ACT_CK(cudaStreamSynchronize(p->cap));
         ACT_AL(gr.d_chan, sizeof(int) * B);
-        ACT_CK(cudaMemcpy(gr.d_chan, gr.chan.data(), sizeof(int) * B, cudaMemcpyHostToDevice));
+        ACT_CK(cudaMemcpyAsync(gr.d_chan, gr.chan.data(), sizeof(int) * B, cudaMemcpyHostToDevice, p->cap));
+        ACT_CK(cudaStreamSynchronize(p->cap));
         ACT_CK(cudaStreamCreateWithFlags(&gr.st, cudaStreamNonBlocking));
         ACT_CK(cudaEventCreateWithFlags(&gr.join, cudaEventDisableTiming));
     }
-    ACT_CK(settle());
     // one graph: fork, then per length group gather -> MP loop -> scatter on
     // its own branch, then join
     ACT_CK(cudaStreamBeginCapture(p->cap, cudaStreamCaptureModeThreadLocal));

@@ -115,10 +115,6 @@ constexpr int kGemvThreads = 256;
 // so that act_inject_alloc_failure can make one of them fail as if the
 // device were out of memory.
 cudaError_t dev_alloc(void **p, size_t bytes);
-// Waits for what was cleared or filled by the legacy stream (cudaMemset and
-// cudaMemcpy may return before the device is done): a caller's non-blocking
-// stream, which is not ordered behind that one, may use it from here on.
-inline cudaError_t settle() { return cudaStreamSynchronize(cudaStreamLegacy); }
 constexpr int kUpdateThreads = 256;
 constexpr int kMaxSamples = 2048;
 constexpr int kRowAlign = 128;   // FP32 row stride granule (floats)
@@ -338,8 +334,8 @@ struct ShiftTcScratch {
 cudaError_t shift_tc_prepare(ShiftTc **out, const ShiftPlan &sp, int sm_count);
 void shift_tc_free(ShiftTc *s);
 // Grows x to hold up to B channels (frees and reallocates: the caller drops
-// every graph that captured x first).
-cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, ShiftTcScratch &x);
+// every graph that captured x first), cleared on st.
+cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, ShiftTcScratch &x, cudaStream_t st);
 void shift_tc_scratch_free(ShiftTcScratch &x);
 // One search order: shifted residual rows + tcgen05 GEMM (tile maxima of the
 // scaled scores), then item selection and FP32 rescore of the flagged items;

@@ -996,7 +996,7 @@ static RowTiling make_tiling(const ShiftPlan &sp, int B) {
 }
 
 // Buffers for B channels (kept when large enough).
-cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, ShiftTcScratch &x) {
+cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, ShiftTcScratch &x, cudaStream_t st) {
     (void)s;
     if (B <= x.B_cap) return cudaSuccess;
     shift_tc_scratch_free(x);
@@ -1011,8 +1011,7 @@ cudaError_t shift_tc_reserve(const ShiftTc *s, const ShiftPlan &sp, int B, Shift
     if (e == cudaSuccess) e = dev_alloc((void **)&x.blk_max, sizeof(float) * (size_t)rows * (sp.T_pad / 32));
     if (e == cudaSuccess) e = dev_alloc((void **)&x.items, sizeof(int) * 2 * (size_t)B * kMaxItems);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.X, sizeof(__nv_bfloat16) * (size_t)rows_alloc * sp.Kt);
-    if (e == cudaSuccess) e = cudaMemset(x.X, 0, sizeof(__nv_bfloat16) * (size_t)rows_alloc * sp.Kt);
-    if (e == cudaSuccess) e = settle();
+    if (e == cudaSuccess) e = cudaMemsetAsync(x.X, 0, sizeof(__nv_bfloat16) * (size_t)rows_alloc * sp.Kt, st);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.bound, sizeof(float) * (size_t)B);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.chmax, sizeof(unsigned int) * (size_t)B);
     if (e == cudaSuccess) e = dev_alloc((void **)&x.chcount, sizeof(int) * (size_t)B);
